@@ -112,8 +112,8 @@ typedef struct gaps_layout {
                              (colour line) and side 1 (anticolour line), 255 = none */
   int64_t dip;            /* float2 [2][capacity][n_events]: per-dipole cache of the trial
                              densities (library-internal contents) */
-  int64_t dq2, dzp, dinv; /* double [2][capacity][n_events]: FP64 part of the dipole cache
-                             (Q^2, z+, 1/ln(z+/z-); library-internal contents) */
+  int64_t dq2, dzp, dinv; /* double [2][capacity][n_events]: room for the FP64 part of the dipole
+                             cache (library-internal contents) */
   int64_t t;              /* double [n_events]: evolution scale t (GeV^2) at which the event
                              finished: t_C at the cutoff, the last winner's scale otherwise */
   int64_t lnt;            /* double [n_events]: ln t while the event is showering */

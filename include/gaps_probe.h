@@ -45,6 +45,13 @@ int gaps_log_fp64_device(const double* x, double* y, int64_t n, void* stream);
  * 0 <= i < n, device arrays, asynchronous on `stream`; GAPS_ERR_INVALID for
  * n < 0 or a null array with n > 0.  Exported for the accuracy tests. */
 int gaps_sqrt_obs_device(const double* x, double* y, int64_t n, void* stream);
+/* The FP64 functions of the splitting kinematics and the dipole cache
+ * (math_fp64.cuh), y[i] = f(x[i]) for 0 <= i < n, device arrays, asynchronous
+ * on `stream`.  op: 0 1/x, 1 1/sqrt(x), 2 sqrt(x), 3 e^x, 4 e^x - 1 (x <= 0),
+ * 5 3/x, 6 and 7 the sine and cosine of 2 pi x (0 < x < 1, a 52-bit uniform).
+ * GAPS_ERR_INVALID for another op, n < 0 or a null array with n > 0.
+ * Exported for the accuracy tests. */
+int gaps_math_fp64_device(int32_t op, const double* x, double* y, int64_t n, void* stream);
 /* The CUDA error string of the last failed call of this library. */
 const char* gaps_probe_last_cuda_error(void);
 

@@ -135,6 +135,8 @@ DevParams make_dev_params(const gaps_params& p, int64_t id_offset) {
   d.ln_s = std::log(d.s);
   d.inv_as2pi_2cf = 1.0 / ((d.as_over / (2.0 * kPi)) * (2.0 * kCF));
   d.inv_as2pi_ca = 1.0 / ((d.as_over / (2.0 * kPi)) * kCA);
+  d.as2pi_ca = (d.as_over / (2.0 * kPi)) * kCA;
+  d.as2pi_qq = (d.as_over / (2.0 * kPi)) * (0.5 * kTR);
   d.tcf = static_cast<float>(p.t_cutoff);
   d.as2pi_f = static_cast<float>(d.as_over / (2.0 * kPi));
   d.lg2_tc_f = static_cast<float>(std::log2(p.t_cutoff));
@@ -170,9 +172,9 @@ Events make_events(const gaps_batch& b) {
   E.acol = reinterpret_cast<int16_t*>(base + L.acol);
   E.link = reinterpret_cast<uint8_t*>(base + L.link);
   E.dip = reinterpret_cast<float2*>(base + L.dip);
-  E.dq2 = reinterpret_cast<double*>(base + L.dq2);
-  E.dzp = reinterpret_cast<double*>(base + L.dzp);
-  E.dinv = reinterpret_cast<double*>(base + L.dinv);
+  // 32 bytes a dipole: the bytes of dq2 and dzp, which lie side by side (each
+  // is a multiple of the alignment)
+  E.drec = reinterpret_cast<DipoleRecord*>(base + L.dq2);
   E.lnt = reinterpret_cast<double*>(base + L.lnt);
   E.t = reinterpret_cast<double*>(base + L.t);
   E.weight = reinterpret_cast<double*>(base + L.weight);

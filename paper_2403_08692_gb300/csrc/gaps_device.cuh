@@ -7,6 +7,7 @@
 
 #include "gaps.h"
 #include "log_fp64.cuh"
+#include "math_fp64.cuh"
 
 namespace gaps {
 
@@ -54,6 +55,7 @@ struct DevParams {
   // event weight n_f 2 dsigma/dcos of flavour f: me_a[f-1] (1 + cos^2) + me_b[f-1] cos
   double me_a[5], me_b[5];
   double inv_as2pi_2cf, inv_as2pi_ca;  // 1 / (alpha_s^over/(2 pi) K) of q->qg and g->gg
+  double as2pi_ca, as2pi_qq;           // alpha_s^over/(2 pi) K of g->gg and g->q qbar
   // FP32 copies used by the screens
   float tcf, as2pi_f, lg2_tc_f, as_mz_over_f, as_b0_f, ln_mz2_f;
   // Philox event id of batch event ev: ev + id_offset (mod 2^32)
@@ -68,7 +70,7 @@ struct DevParams {
 // Everything GenerateEmission needs about an accepted winner (56 bytes:
 // workspaces hold fewer than 2^31 events and at most 255 partons each).
 struct EmitTask {
-  double lnt, q2, zp, inv_ls;
+  double lnt, q2, zp, ls;
   uint32_t rz_hi, rz_lo;
   int32_t ev, step;
   uint8_t i, k, n, side, kappa, kind, pad0, pad1;
@@ -121,6 +123,13 @@ __host__ __device__ inline double fixed128_to_double(unsigned long long lo, unsi
   return (neg ? -mag : mag) * scale_inv;
 }
 
+// FP64 part of a dipole's cache entry (see shower_cycle.cuh): one sector, so
+// that a winner's data comes in one access.  A dipole's record is kept at its
+// colour end (the parton whose side-0 link it is).
+struct alignas(32) DipoleRecord {
+  double q2, zp, inv_ls, ls;  // Q^2, z+, 1/ln(z+/z-), ln(z+/z-)
+};
+
 // Pointers into the workspace (gaps_layout) for one batch.
 struct Events {
   double *px, *py, *pz, *e;
@@ -128,7 +137,7 @@ struct Events {
   int16_t *col, *acol;
   uint8_t* link;  // [2][cap][n]
   float2* dip;    // [2][cap][n] dipole cache (see shower_cycle.cuh)
-  double *dq2, *dzp, *dinv;  // [2][cap][n] FP64 part of the dipole cache
+  DipoleRecord* drec;  // [cap][n] FP64 part of the dipole cache (in the bytes of the layout's dq2 and dzp)
   double* lnt;               // [n] ln t of the active events
   double *t, *weight;
   unsigned long long* hash;
@@ -435,55 +444,51 @@ __device__ __forceinline__ double mdot(const V4& a, const V4& b) {
   return fma(-a.z, b.z, fma(-a.y, b.y, fma(-a.x, b.x, a.e * b.e)));
 }
 
-__device__ __forceinline__ double det3(double a1, double a2, double a3, double b1, double b2, double b3,
-                                       double c1, double c2, double c3) {
-  const double m1 = fma(b2, c3, -(b3 * c2)), m2 = fma(b1, c3, -(b3 * c1)), m3 = fma(b1, c2, -(b2 * c1));
-  return fma(a3, m3, fma(-a2, m2, a1 * m1));
-}
-
 // Catani-Seymour final-final map for massless splitter a and spectator b:
 // p_i = z a + (1-z) y b + k, p_j = (1-z) a + z y b - k, p_b' = (1-y) b,
 // k = sqrt(z(1-z) y Q^2) (cos phi n1 + sin phi n2), with n1, n2 unit
 // spacelike vectors orthogonal to a, b and each other: n1 projects the
 // first of the references (1,1,0,0), (1,0,1,0), (1,0,0,1) whose projection
 // has |n1^2| >= 1e-4, n2 is the Minkowski-orthogonal complement of (a, b,
-// n1) (cofactor expansion of det[X; a; b; n1]).  n1 is formed scaled by a.b
-// (no division) and both normalisations take the library's rsqrt (one ulp):
-// the oracle's vectors up to rounding.
+// n1) (cofactor expansion of det[X; a; b; n1]).  n1 and n2 are left at the
+// lengths they come in (n1 scaled by a.b, so no division) and k's two
+// coefficients take their normalisations: the oracle's vectors up to
+// rounding.
 __device__ __forceinline__ void dipole_map(const V4& a, const V4& b, double z, double y, double cphi,
                                            double sphi, V4& pi, V4& pj, V4& pb) {
   const double ab = mdot(a, b);
   const double q2 = 2.0 * ab;
-  // n1 scaled by a.b (a.b > 0): ab ref - (ref.b) a - (ref.a) b, so no
-  // division; the reference test |n1^2| >= 1e-4 becomes |(ab n1)^2| >=
-  // 1e-4 ab^2, and the normalisation below removes the scale.
-  const double lim = 1e-4 * ab * ab;
+  // n1 scaled by a.b (a.b > 0): ab ref - (ref.b) a - (ref.a) b; the reference
+  // test |n1^2| >= 1e-4 becomes |(ab n1)^2| >= 1e-4 ab^2, on the bits of
+  // these non-negative numbers.
+  const long long lim = __double_as_longlong(1e-4 * ab * ab);
   V4 n1{0, 0, 0, 0};
+  double n1sq = 0.0;
+#pragma unroll 1  // the first reference serves nearly every dipole
   for (int r = 0; r < 3; ++r) {
-    const V4 ref{1.0, r == 0 ? 1.0 : 0.0, r == 1 ? 1.0 : 0.0, r == 2 ? 1.0 : 0.0};
-    const double cb = mdot(ref, b);
-    const double ca = mdot(ref, a);
+    // ref.b and ref.a: the reference's other components are zero
+    const double cb = b.e - (r == 0 ? b.x : (r == 1 ? b.y : b.z));
+    const double ca = a.e - (r == 0 ? a.x : (r == 1 ? a.y : a.z));
     n1 = V4{fma(-ca, b.e, fma(-cb, a.e, ab)), fma(-ca, b.x, fma(-cb, a.x, r == 0 ? ab : 0.0)),
             fma(-ca, b.y, fma(-cb, a.y, r == 1 ? ab : 0.0)), fma(-ca, b.z, fma(-cb, a.z, r == 2 ? ab : 0.0))};
-    if (fabs(mdot(n1, n1)) >= lim) break;
+    n1sq = mdot(n1, n1);
+    if ((__double_as_longlong(n1sq) & 0x7fffffffffffffffll) >= lim) break;
   }
-  const double s1 = rsqrt(-mdot(n1, n1));
-  n1 = V4{n1.e * s1, n1.x * s1, n1.y * s1, n1.z * s1};
-  const double c0 = det3(a.x, a.y, a.z, b.x, b.y, b.z, n1.x, n1.y, n1.z);
-  const double c1 = -det3(a.e, a.y, a.z, b.e, b.y, b.z, n1.e, n1.y, n1.z);
-  const double c2 = det3(a.e, a.x, a.z, b.e, b.x, b.z, n1.e, n1.x, n1.z);
-  const double c3 = -det3(a.e, a.x, a.y, b.e, b.x, b.y, n1.e, n1.x, n1.y);
-  V4 n2{c0, -c1, -c2, -c3};
-  const double s2 = rsqrt(-mdot(n2, n2));
-  n2 = V4{n2.e * s2, n2.x * s2, n2.y * s2, n2.z * s2};
-  const double kt = sqrt(z * (1.0 - z) * y * q2);
-  const double kc = kt * cphi, ks = kt * sphi;
+  // the 2 x 2 minors of (b, n1), each in two of the cofactors
+  const double m_yz = fma(b.y, n1.z, -(b.z * n1.y)), m_xz = fma(b.x, n1.z, -(b.z * n1.x));
+  const double m_xy = fma(b.x, n1.y, -(b.y * n1.x)), m_ez = fma(b.e, n1.z, -(b.z * n1.e));
+  const double m_ey = fma(b.e, n1.y, -(b.y * n1.e)), m_ex = fma(b.e, n1.x, -(b.x * n1.e));
+  const V4 n2{fma(a.z, m_xy, fma(-a.y, m_xz, a.x * m_yz)), fma(a.z, m_ey, fma(-a.y, m_ez, a.e * m_yz)),
+              -fma(a.z, m_ex, fma(-a.x, m_ez, a.e * m_xz)), fma(a.y, m_ex, fma(-a.x, m_ey, a.e * m_xy))};
+  const double fa_j = 1.0 - z;
+  const double kt = sqrt_fp64(z * fa_j * y * q2);
+  const double kc = kt * cphi * rsqrt_fp64(-n1sq), ks = kt * sphi * rsqrt_fp64(-mdot(n2, n2));
   const V4 k{fma(ks, n2.e, kc * n1.e), fma(ks, n2.x, kc * n1.x), fma(ks, n2.y, kc * n1.y), fma(ks, n2.z, kc * n1.z)};
-  const double fa_i = z, fb_i = (1.0 - z) * y, fa_j = 1.0 - z, fb_j = z * y;
-  pi = V4{fma(fb_i, b.e, fa_i * a.e) + k.e, fma(fb_i, b.x, fa_i * a.x) + k.x, fma(fb_i, b.y, fa_i * a.y) + k.y,
-          fma(fb_i, b.z, fa_i * a.z) + k.z};
-  pj = V4{fma(fb_j, b.e, fa_j * a.e) - k.e, fma(fb_j, b.x, fa_j * a.x) - k.x, fma(fb_j, b.y, fa_j * a.y) - k.y,
-          fma(fb_j, b.z, fa_j * a.z) - k.z};
+  const double fb_i = fa_j * y, fb_j = z * y;
+  pi = V4{fma(fb_i, b.e, fma(z, a.e, k.e)), fma(fb_i, b.x, fma(z, a.x, k.x)), fma(fb_i, b.y, fma(z, a.y, k.y)),
+          fma(fb_i, b.z, fma(z, a.z, k.z))};
+  pj = V4{fma(fb_j, b.e, fma(fa_j, a.e, -k.e)), fma(fb_j, b.x, fma(fa_j, a.x, -k.x)),
+          fma(fb_j, b.y, fma(fa_j, a.y, -k.y)), fma(fb_j, b.z, fma(fa_j, a.z, -k.z))};
   const double r = 1.0 - y;
   pb = V4{r * b.e, r * b.x, r * b.y, r * b.z};
 }

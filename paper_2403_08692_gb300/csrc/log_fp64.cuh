@@ -71,6 +71,13 @@ struct alignas(32) LogEntry {
 static __device__ const LogEntry kLogTableDevice[] = {GAPS_LOG_TABLE};
 static const LogEntry kLogTableHost[] = {GAPS_LOG_TABLE};
 
+// Out of line: the logarithm of inputs that are not positive normal numbers.
+#ifdef __CUDACC__
+static __host__ __device__ __noinline__ double log_library(double x) { return log(x); }
+#else
+static inline double log_library(double x) { return std::log(x); }
+#endif
+
 __host__ __device__ __forceinline__ double log_fp64(double x) {
 #ifdef __CUDA_ARCH__
   const uint64_t bits = static_cast<uint64_t>(__double_as_longlong(x));
@@ -80,7 +87,7 @@ __host__ __device__ __forceinline__ double log_fp64(double x) {
 #endif
   // positive normal x (tested on the bits: the FP64 pipe's compares cost as
   // much as its FMAs on this part)
-  if (bits - 0x0010000000000000ull >= 0x7fe0000000000000ull) return log(x);
+  if (bits - 0x0010000000000000ull >= 0x7fe0000000000000ull) return log_library(x);
   constexpr uint64_t kFrac = (uint64_t{1} << 52) - 1;
   constexpr uint64_t kSqrt2Frac = 0x6a09e667f3bcdull;  // fraction bits of sqrt(2)
   const uint64_t frac = bits & kFrac;

@@ -15,6 +15,7 @@
 #include "gaps.h"
 #include "gaps_probe.h"
 #include "log_fp64.cuh"
+#include "math_fp64.cuh"
 #include "sqrt_obs.cuh"
 
 namespace gaps {
@@ -137,6 +138,24 @@ __global__ void __launch_bounds__(256) k_log_fp64(const double* x, double* y, in
   if (k < n) y[k] = log_fp64(x[k]);
 }
 
+__global__ void __launch_bounds__(256) k_math_fp64(int op, const double* x, double* y, int64_t n) {
+  const int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (k >= n) return;
+  const double v = x[k];
+  double s = 0.0, c = 0.0;
+  switch (op) {
+    case 0: y[k] = rcp_fp64(v); break;
+    case 1: y[k] = rsqrt_fp64(v); break;
+    case 2: y[k] = sqrt_fp64(v); break;
+    case 3: y[k] = exp_fp64(v); break;
+    case 4: y[k] = expm1_neg_fp64(v); break;
+    case 5: y[k] = div_fp64(3.0, v); break;
+    default:
+      circle_fp64(v, static_cast<uint32_t>(v * 4294967296.0), &s, &c);
+      y[k] = op == 6 ? s : c;
+  }
+}
+
 __global__ void __launch_bounds__(256) k_sqrt_obs(const double* x, double* y, int64_t n) {
   const int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (k < n) y[k] = sqrt_obs(x[k]);
@@ -171,6 +190,14 @@ extern "C" int gaps_sqrt_obs_device(const double* x, double* y, int64_t n, void*
   if (n < 0 || (n > 0 && (!x || !y))) return GAPS_ERR_INVALID;
   if (n == 0) return GAPS_OK;
   k_sqrt_obs<<<static_cast<unsigned>((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(x, y, n);
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? GAPS_OK : record_cuda_error(e);
+}
+
+extern "C" int gaps_math_fp64_device(int32_t op, const double* x, double* y, int64_t n, void* stream) {
+  if (op < 0 || op > 7 || n < 0 || (n > 0 && (!x || !y))) return GAPS_ERR_INVALID;
+  if (n == 0) return GAPS_OK;
+  k_math_fp64<<<static_cast<unsigned>((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(op, x, y, n);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? GAPS_OK : record_cuda_error(e);
 }

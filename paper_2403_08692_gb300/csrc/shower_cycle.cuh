@@ -24,7 +24,7 @@
 //    FP64.  z and y are recomputed in FP64 for the accepted emissions.
 //  * Dipole cache.  A dipole's trial density depends only on its invariant
 //    mass, which changes only when an emission moves one of its partons, so
-//    Q^2, z+ and 1/ln(z+/z-) (FP64) and 1/c (FP32) are stored per dipole and
+//    Q^2, z+, ln(z+/z-) and its inverse (FP64) and 1/c (FP32) are stored per dipole and
 //    recomputed once per dipole an emission touches.
 #pragma once
 #include "gaps_device.cuh"
@@ -69,38 +69,42 @@ __device__ __forceinline__ size_t dip_at(const Events& E, int side, int slot, in
 // none of the cancellation in 1 - z+ (the values agree with the oracle's two
 // logarithms to about 1e-13 relative at LEP energies).
 struct DipoleEntry {
-  double q2, zp, inv_ls;
+  DipoleRecord rec;
   float2 screen;
 };
 
 __device__ __forceinline__ DipoleEntry make_dipole(const DevParams& P, double q2) {
   DipoleEntry d;
-  d.q2 = q2;
-  if (q2 < 4.0 * P.tc) {
-    d.zp = d.inv_ls = 0.0;
+  d.rec.q2 = q2;
+  // b = sqrt(1 - 4 t_C/Q^2) = a / sqrt(Q^2 a) with a = Q^2 - 4 t_C: one
+  // reciprocal square root instead of a division and a square root; the sign
+  // of a is the oracle's test Q^2 < 4 t_C (their difference is exact where
+  // they are close)
+  const double a = q2 - 4.0 * P.tc;
+  if (__double_as_longlong(a) < 0) {
+    d.rec.zp = d.rec.inv_ls = d.rec.ls = 0.0;
     d.screen = make_float2(-1.0f, -1.0f);
     return d;
   }
-  // b = sqrt(1 - 4 t_C/Q^2) = a / sqrt(Q^2 a) with a = Q^2 - 4 t_C: one
-  // reciprocal square root instead of a division and a square root
-  const double a = q2 - 4.0 * P.tc;
-  const double b = __double_as_longlong(a) > 0 ? a * rsqrt(q2 * a) : 0.0;  // a > 0, tested on the bits
+  const double b = __double_as_longlong(a) > 0 ? a * rsqrt_fp64(q2 * a) : 0.0;
   const double b1 = 1.0 + b;
-  d.zp = 0.5 * b1;
+  d.rec.zp = 0.5 * b1;
   const double ls = log_fp64((b1 * b1) * (q2 * P.inv_4tc));
-  d.inv_ls = 1.0 / ls;
+  d.rec.ls = ls;
+  d.rec.inv_ls = rcp_fp64(ls);
   d.screen = make_float2(1.0f / (P.as2pi_f * f32_from_f64(ls)),
                          1.0f / (P.as2pi_f * 0.5f * static_cast<float>(kTR) * f32_from_f64(b)));
   return d;
 }
 
-__device__ __forceinline__ void store_dipole(const Events& E, int64_t ev, int slot, int side, const DipoleEntry& d) {
-  const size_t a = dip_at(E, side, slot, ev);
-  E.dip[a] = d.screen;
+// The entry of the dipole between slots x and k, partners on x's side `side`:
+// its screen entry on both sides, its record at the colour end.
+__device__ __forceinline__ void store_dipole(const Events& E, int64_t ev, int x, int side, int k,
+                                             const DipoleEntry& d) {
+  E.dip[dip_at(E, side, x, ev)] = d.screen;
+  E.dip[dip_at(E, 1 - side, k, ev)] = d.screen;
   if (d.screen.x < 0.0f) return;
-  E.dq2[a] = d.q2;
-  E.dzp[a] = d.zp;
-  E.dinv[a] = d.inv_ls;
+  E.drec[E.at(side == 0 ? x : k, ev)] = d.rec;
 }
 
 // 32-bit float close to the 52-bit uniform built from (hi, lo): relative
@@ -125,30 +129,33 @@ __device__ __forceinline__ uint32_t pack_refresh(int t, int x, int side, int k) 
 // 1/c of a kernel for a dipole, c = alpha_s^over/(2 pi) * integral of
 // P^over over [z-, z+].
 __device__ __forceinline__ double inv_c_fp64(const DevParams& P, int kind, double zp, double inv_ls) {
-  if (kind == kGtoQQ) return 1.0 / ((P.as_over / (2.0 * kPi)) * (0.5 * kTR) * (zp - (1.0 - zp)));
+  if (kind == kGtoQQ) return rcp_fp64(P.as2pi_qq * (zp - (1.0 - zp)));
   return inv_ls * (kind == kQtoQG ? P.inv_as2pi_2cf : P.inv_as2pi_ca);
 }
 
 // 1/c of a gluon's kernels together (the per-dipole trial): c summed over
 // the kernels in their order, as the oracle sums it.
-__device__ __forceinline__ double inv_c_sum_fp64(const DevParams& P, double zp, double inv_ls) {
-  const double c_gg = 1.0 / (inv_ls * P.inv_as2pi_ca);
-  const double c_qq = (P.as_over / (2.0 * kPi)) * (0.5 * kTR) * (zp - (1.0 - zp));
+__device__ __forceinline__ double inv_c_sum_fp64(const DevParams& P, double zp, double ls) {
+  const double c_gg = ls * P.as2pi_ca;
+  const double c_qq = P.as2pi_qq * (zp - (1.0 - zp));
   double c = c_gg;
+#pragma unroll 1
   for (int f = 0; f < P.nf; ++f) c += c_qq;
-  return 1.0 / c;
+  return rcp_fp64(c);
 }
 
 // The kernel of a winning gluon dipole in the per-dipole mode: kappa with
 // probability c_kappa / c_sum, by the running sum against v c_sum.
-__device__ __forceinline__ int choose_kernel(const DevParams& P, double zp, double inv_ls, double v) {
-  const double c_gg = 1.0 / (inv_ls * P.inv_as2pi_ca);
-  const double c_qq = (P.as_over / (2.0 * kPi)) * (0.5 * kTR) * (zp - (1.0 - zp));
+__device__ __forceinline__ int choose_kernel(const DevParams& P, double zp, double ls, double v) {
+  const double c_gg = ls * P.as2pi_ca;
+  const double c_qq = P.as2pi_qq * (zp - (1.0 - zp));
   double c_sum = c_gg;
+#pragma unroll 1
   for (int f = 0; f < P.nf; ++f) c_sum += c_qq;
   const double target = v * c_sum;
   double cum = c_gg;
   if (target < cum) return 0;
+#pragma unroll 1
   for (int q = 1; q <= P.nf; ++q) {
     cum += c_qq;
     if (target < cum) return q;
@@ -185,16 +192,17 @@ __device__ inline bool select_winner_fp64_range(const DevParams& P, const Events
           const int kappa = kp + h;
           const int kind = combined ? kKindUnchosen : (gluon ? (kappa == 0 ? kGtoGG : kGtoQQ) : kQtoQG);
           const double u = h ? to_unit(r.z, r.w) : to_unit(r.x, r.y);
-          const double inv_c = combined ? inv_c_sum_fp64(P, d.zp, d.inv_ls) : inv_c_fp64(P, kind, d.zp, d.inv_ls);
+          const double inv_c =
+              combined ? inv_c_sum_fp64(P, d.rec.zp, d.rec.ls) : inv_c_fp64(P, kind, d.rec.zp, d.rec.inv_ls);
           const double lt = fma(log_fp64(u), inv_c, lnt);
           if (lt > best) {
             best = lt;
             code = (2 * i + side) * 8 + kappa;
             found = true;
             w.lnt = lt;
-            w.q2 = d.q2;
-            w.zp = d.zp;
-            w.inv_ls = d.inv_ls;
+            w.q2 = d.rec.q2;
+            w.zp = d.rec.zp;
+            w.ls = d.rec.ls;
             w.i = i;
             w.k = k;
             w.side = side;
@@ -233,7 +241,17 @@ __device__ __forceinline__ double veto_ratio_fp64(const DevParams& P, int kind, 
 __device__ __forceinline__ double z_fp64(int kind, double zp, double lsoft, double r) {
   const double zm = 1.0 - zp;
   if (kind == kGtoQQ) return fma(zp - zm, r, zm);
-  return fma(-zp, expm1(-r * lsoft), zm);
+  return fma(-zp, expm1_neg_fp64(-r * lsoft), zm);
+}
+
+// The veto decided in FP64 (a veto number within the FP32 ratio's error of
+// it, about one cycle in 10^4): out of line, its logarithm, exponentials and
+// divisions would make up much of the cycle's code.
+static __device__ __noinline__ bool accept_fp64(const DevParams& P, int kind, double lnt, double q2, double zp, double ls,
+                                                double rz, double rv) {
+  const double z = z_fp64(kind, zp, ls, rz);
+  const double ratio = veto_ratio_fp64(P, kind, exp_fp64(lnt), q2, z);
+  return ratio >= 0.0 && rv < ratio;
 }
 
 enum : int { kCycleVetoed = 0, kCycleFinished = 1, kCycleAccepted = 2 };
@@ -253,6 +271,12 @@ __device__ __forceinline__ void count_job_done(const Events& E, int64_t ev, bool
 __device__ __forceinline__ void finish_event(const Events& E, int64_t ev, int status, double t) {
   E.status[ev] = status;
   E.t[ev] = t;
+}
+
+// The same before the cutoff (a full record, the cycle limit), at ln t = lnt:
+// rare, so out of line.
+static __device__ __noinline__ void finish_early(const Events& E, int64_t ev, int status, double lnt) {
+  finish_event(E, ev, status, exp_fp64(lnt));
 }
 
 // The FP32 screen of SelectWinnerEmission over the trials of partons
@@ -398,18 +422,14 @@ __device__ __forceinline__ void screen_group_reduce(Screen& sc) {
 // FP64 selection decides (select_winner_fp64 / fallback_warp).
 enum : int { kScreenNone = 0, kScreenWinner = 1, kScreenUndecided = 2 };
 
-// The first part of the cycle once the screen is known: the cycle and work
-// counts, and the screen's verdict; for a certain winner its exact scale
-// (from the FP64 cache) and the winner's data in `task`.
+// The screen's verdict; for a certain winner its exact scale (from the FP64
+// cache) and the winner's data in `task`.  Writes nothing to the record.
 template <int kMode>
-__device__ inline int cycle_screen(const DevParams& P, const Events& E, int64_t ev, int step, double lnt,
-                                   const Screen& sc, EmitTask& task) {
+__device__ __forceinline__ int screen_verdict(const DevParams& P, const Events& E, int64_t ev, double lnt,
+                                              const Screen& sc, EmitTask& task) {
   const float best_key = sc.best_key, best_m = sc.best_m, others_hi = sc.others_hi;
   const int best_code = sc.best_code;
   const uint32_t best_hi = sc.best_hi, best_lo = sc.best_lo;
-  E.n_steps[ev] = step + 1;
-  E.n_trials[ev] += sc.trials;
-  E.n_dipoles[ev] += sc.dipoles;
 
   // Cutoff threshold in key units: t' > t_C  <=>  key > log2(t_C / t).
   const float lt2 = f32_from_f64(lnt) * 1.44269504f;
@@ -423,20 +443,21 @@ __device__ inline int cycle_screen(const DevParams& P, const Events& E, int64_t 
     // Certain winner: its scale exactly, from the FP64 cache.
     const int dcode = best_code >> 3, kappa = best_code & 7;
     const int i = dcode >> 1, side = dcode & 1;
-    const size_t a = dip_at(E, side, i, ev);
+    const int k = static_cast<int>(sc.best_aux & 255u);
+    const DipoleRecord rec = E.drec[E.at(side == 0 ? i : k, ev)];
     const bool gluon = (sc.best_aux & 256u) != 0u;  // as the screen read them: no second load
     const bool combined = gluon && per_dipole<kMode>(P);
     const int kind = combined ? kKindUnchosen : (gluon ? (kappa == 0 ? kGtoGG : kGtoQQ) : kQtoQG);
-    const double zp = E.dzp[a], inv_ls = E.dinv[a];
-    const double inv_c = combined ? inv_c_sum_fp64(P, zp, inv_ls) : inv_c_fp64(P, kind, zp, inv_ls);
+    const double inv_c =
+        combined ? inv_c_sum_fp64(P, rec.zp, rec.ls) : inv_c_fp64(P, kind, rec.zp, rec.inv_ls);
     const double lt = fma(log_fp64(to_unit(best_hi, best_lo)), inv_c, lnt);
     if (lt > P.ln_tc) {
       task.lnt = lt;
-      task.q2 = E.dq2[a];
-      task.zp = zp;
-      task.inv_ls = inv_ls;
+      task.q2 = rec.q2;
+      task.zp = rec.zp;
+      task.ls = rec.ls;
       task.i = i;
-      task.k = static_cast<uint8_t>(sc.best_aux & 255u);
+      task.k = k;
       task.side = side;
       task.kappa = kappa;
       task.kind = kind;
@@ -444,6 +465,17 @@ __device__ inline int cycle_screen(const DevParams& P, const Events& E, int64_t 
     }
   }
   return kScreenUndecided;
+}
+
+// The first part of the cycle once the screen is known: the cycle and work
+// counts, and the screen's verdict.
+template <int kMode>
+__device__ inline int cycle_screen(const DevParams& P, const Events& E, int64_t ev, int step, double lnt,
+                                   const Screen& sc, EmitTask& task) {
+  E.n_steps[ev] = step + 1;
+  E.n_trials[ev] += sc.trials;
+  E.n_dipoles[ev] += sc.dipoles;
+  return screen_verdict<kMode>(P, E, ev, lnt, sc, task);
 }
 
 // The exact FP64 selection for the undecided events of a warp, each computed
@@ -493,7 +525,8 @@ __device__ __noinline__ void fallback_warp(const DevParams& P0, const Events& E,
     if (own) {
       const int ol = __ffs(own) - 1;
       const double t_lnt = __shfl_sync(0xffffffffu, w.lnt, ol), t_q2 = __shfl_sync(0xffffffffu, w.q2, ol);
-      const double t_zp = __shfl_sync(0xffffffffu, w.zp, ol), t_inv = __shfl_sync(0xffffffffu, w.inv_ls, ol);
+      const double t_zp = __shfl_sync(0xffffffffu, w.zp, ol);
+      const double t_ls = __shfl_sync(0xffffffffu, w.ls, ol);
       const uint32_t packed = __shfl_sync(0xffffffffu,
                                           static_cast<uint32_t>(w.i) | (static_cast<uint32_t>(w.k) << 8) |
                                               (static_cast<uint32_t>(w.side) << 16) |
@@ -504,7 +537,7 @@ __device__ __noinline__ void fallback_warp(const DevParams& P0, const Events& E,
         task.lnt = t_lnt;
         task.q2 = t_q2;
         task.zp = t_zp;
-        task.inv_ls = t_inv;
+        task.ls = t_ls;
         task.i = static_cast<uint8_t>(packed & 255u);
         task.k = static_cast<uint8_t>((packed >> 8) & 255u);
         task.side = static_cast<uint8_t>((packed >> 16) & 15u);
@@ -516,25 +549,18 @@ __device__ __noinline__ void fallback_warp(const DevParams& P0, const Events& E,
   }
 }
 
-// The rest of the cycle once the winner is known (have: a trial above t_C,
-// with its data in task): CheckCutoff, AcceptOrVeto and the decision hash.
-// Returns kCycleFinished when the event left the active state (status
-// written), kCycleAccepted with `task` filled when an emission must be
-// generated, kCycleVetoed otherwise.
+// AcceptOrVeto of a known winner (its data in task): the kernel of a
+// per-dipole trial drawn (kind and kappa then written to task), z and the
+// acceptance ratio, and the decision added to the event's hash.  Returns
+// whether the emission is accepted.  The words of z's
+// uniform go to task.  Writes nothing to the record.
 template <int kMode>
-__device__ inline int cycle_conclude(const DevParams& P, const Events& E, int64_t ev, const EventKey& key, int step,
-                                     int n, bool have, EmitTask& task) {
-  // ---- CheckCutoff.
-  if (!have) {
-    finish_event(E, ev, GAPS_DONE, P.tc);
-    return kCycleFinished;
-  }
-  E.lnt[ev] = task.lnt;
-  E.n_winners[ev] += 1;
+__device__ __forceinline__ bool accept_or_veto(const DevParams& P, const Events& E, const EventKey& key, int step,
+                                               EmitTask& task, unsigned long long& hash) {
   if (task.kind == kKindUnchosen) {
     // per-dipole trial of a gluon: its kernel from the winner's second draw
     const U4 rk = philox_draw<kMode>(P, key, static_cast<uint32_t>(step), 1u, kDrawWinner);
-    const int kappa = choose_kernel(P, task.zp, task.inv_ls, to_unit(rk.z, rk.w));
+    const int kappa = choose_kernel(P, task.zp, task.ls, to_unit(rk.z, rk.w));
     task.kappa = static_cast<uint8_t>(kappa);
     task.kind = static_cast<uint8_t>(kappa == 0 ? kGtoGG : kGtoQQ);
   }
@@ -545,7 +571,7 @@ __device__ inline int cycle_conclude(const DevParams& P, const Events& E, int64_
   {
     const float zpf = f32_from_f64(task.zp);
     const float zmf = f32_from_f64(1.0 - task.zp);
-    const float lf = 1.0f / f32_from_f64(task.inv_ls);
+    const float lf = f32_from_f64(task.ls);
     const float rzf = unit_float(rw.x, rw.y);
     float z, e;  // z and 1 - z
     if (task.kind == kGtoQQ) {
@@ -571,9 +597,8 @@ __device__ inline int cycle_conclude(const DevParams& P, const Events& E, int64_
     const float margin = kVetoRel * (fabsf(ratio) + rvf) + kVetoAbs;
     if (fabsf(y - 1.0f) <= 1e-4f || fabsf(rvf - ratio) <= margin) {
       atomicAdd(&E.counters[3], 1ull);  // veto decided in FP64
-      const double zz = z_fp64(task.kind, task.zp, 1.0 / task.inv_ls, to_unit(rw.x, rw.y));
-      const double ratio64 = veto_ratio_fp64(P, task.kind, exp(task.lnt), task.q2, zz);
-      accept = ratio64 >= 0.0 && to_unit(rw.z, rw.w) < ratio64;
+      accept = accept_fp64(P, task.kind, task.lnt, task.q2, task.zp, task.ls, to_unit(rw.x, rw.y),
+                           to_unit(rw.z, rw.w));
     } else {
       accept = y < 1.0f && rvf < ratio;
     }
@@ -583,15 +608,36 @@ __device__ inline int cycle_conclude(const DevParams& P, const Events& E, int64_
                                   (static_cast<unsigned long long>(task.side) << 40) |
                                   (static_cast<unsigned long long>(task.kappa) << 48) |
                                   (static_cast<unsigned long long>(accept ? 1 : 0) << 56);
-  E.hash[ev] = fnv1a64(E.hash[ev], word);
+  hash = fnv1a64(hash, word);
+  task.rz_hi = rw.x;
+  task.rz_lo = rw.y;
+  return accept;
+}
+
+// The rest of the cycle once the winner is known (have: a trial above t_C,
+// with its data in task): CheckCutoff, AcceptOrVeto and the decision hash.
+// Returns kCycleFinished when the event left the active state (status
+// written), kCycleAccepted with `task` filled when an emission must be
+// generated, kCycleVetoed otherwise.
+template <int kMode>
+__device__ inline int cycle_conclude(const DevParams& P, const Events& E, int64_t ev, const EventKey& key, int step,
+                                     int n, bool have, EmitTask& task) {
+  // ---- CheckCutoff.
+  if (!have) {
+    finish_event(E, ev, GAPS_DONE, P.tc);
+    return kCycleFinished;
+  }
+  E.lnt[ev] = task.lnt;
+  E.n_winners[ev] += 1;
+  unsigned long long hash = E.hash[ev];
+  const bool accept = accept_or_veto<kMode>(P, E, key, step, task, hash);
+  E.hash[ev] = hash;
   if (!accept) return kCycleVetoed;
   if (n >= E.cap) {
-    finish_event(E, ev, GAPS_OVERFLOW, exp(task.lnt));
+    finish_early(E, ev, GAPS_OVERFLOW, task.lnt);
     return kCycleFinished;
   }
   task.ev = static_cast<int32_t>(ev);
-  task.rz_hi = rw.x;
-  task.rz_lo = rw.y;
   task.n = n;
   task.step = step;
   return kCycleAccepted;
@@ -621,7 +667,7 @@ __device__ inline int cycle_select_veto(const DevParams& P0, const Events& E, in
   const int step = E.n_steps[ev];
   const double lnt = E.lnt[ev];
   if (step >= P.max_steps) {
-    finish_event(E, ev, GAPS_STEP_LIMIT, exp(lnt));
+    finish_early(E, ev, GAPS_STEP_LIMIT, lnt);
     return kCycleFinished;
   }
   Screen sc;
@@ -641,95 +687,74 @@ __device__ inline void cycle_emit(const DevParams& P0, const Events& E, const Em
   const int job = kJobKey<kMode> ? static_cast<int>(E.job_of[ev]) : 0;
   const DevParams& P = job_params<kJobPhysics<kMode>>(P0, E, job);
   const EventKey key = event_key<kMode>(P, E, ev, job);
-  const double t = exp(w.lnt);
-  const double z = z_fp64(w.kind, w.zp, 1.0 / w.inv_ls, to_unit(w.rz_hi, w.rz_lo));
-  const double y = t / (w.q2 * z * (1.0 - z));
+  const double t = exp_fp64(w.lnt);
+  const double z = z_fp64(w.kind, w.zp, w.ls, to_unit(w.rz_hi, w.rz_lo));
+  const double y = div_fp64(t, w.q2 * z * (1.0 - z));
   const U4 rphi = philox_draw<kMode>(P, key, static_cast<uint32_t>(w.step), 1u, kDrawWinner);
   double sphi, cphi;
-  sincospi(2.0 * to_unit(rphi.x, rphi.y), &sphi, &cphi);
-  const V4 a = load_p(E, w.i, ev);
-  const V4 b = load_p(E, w.k, ev);
+  circle_fp64(to_unit(rphi.x, rphi.y), rphi.x, &sphi, &cphi);
+  const int i = w.i, j = w.n, k = w.k, side = w.side;
+  const V4 a = load_p(E, i, ev);
+  const V4 b = load_p(E, k, ev);
+  // the partners of the splitter and of the spectator outside their dipole
+  // (the colour chain is open, so i, j, k and these are distinct)
+  const int oi = E.link[E.link_at(1 - side, i, ev)], ok = E.link[E.link_at(side, k, ev)];
   V4 pi, pj, pb;
   dipole_map(a, b, z, y, cphi, sphi, pi, pj, pb);
-  const int j = w.n;
-  store_p(E, w.i, ev, pi);
+  store_p(E, i, ev, pi);
   store_p(E, j, ev, pj);
-  store_p(E, w.k, ev, pb);
-  const size_t ai = E.at(w.i, ev), aj = E.at(j, ev);
-  if (w.kind == kGtoQQ) {
-    // g(c, a) -> q(c, 0) + qbar(0, a); the parton holding colour a now
-    // connects to the antiquark.
-    const int q = E.link[E.link_at(1, w.i, ev)];
-    E.flav[ai] = static_cast<int8_t>(w.kappa);
-    E.flav[aj] = static_cast<int8_t>(-w.kappa);
-    E.col[aj] = 0;
-    E.acol[aj] = E.acol[ai];
-    E.acol[ai] = 0;
-    E.link[E.link_at(1, w.i, ev)] = kNoLink;
-    E.link[E.link_at(0, j, ev)] = kNoLink;
-    E.link[E.link_at(1, j, ev)] = static_cast<uint8_t>(q);
-    E.link[E.link_at(0, q, ev)] = static_cast<uint8_t>(j);
-  } else {
-    // A gluon enters the shared colour line between splitter and spectator;
-    // the splitter takes the new line m.
-    const int m = E.next_colour[ev];
+  store_p(E, k, ev, pb);
+  // Colours.  A gluon enters the shared colour line between splitter and
+  // spectator: on side `s` it takes the splitter's line and on the other a
+  // new line m, the splitter takes m on side s.  g(c, a) -> q(c, 0) +
+  // qbar(0, a) is the same on the anticolour side with no line m: the
+  // antiquark connects to the holder of colour a, and not to the quark.
+  const bool split = w.kind == kGtoQQ;
+  const int s = split ? 1 : side;
+  const int to = split && side == 0 ? oi : k;  // j's partner on side s
+  int m = 0;
+  if (!split) {
+    m = E.next_colour[ev];
     E.next_colour[ev] = m + 1;
-    E.flav[aj] = static_cast<int8_t>(kGluon);
-    if (w.side == 0) {
-      E.col[aj] = E.col[ai];
-      E.acol[aj] = static_cast<int16_t>(m);
-      E.col[ai] = static_cast<int16_t>(m);
-      E.link[E.link_at(0, w.i, ev)] = static_cast<uint8_t>(j);
-      E.link[E.link_at(0, j, ev)] = static_cast<uint8_t>(w.k);
-      E.link[E.link_at(1, j, ev)] = static_cast<uint8_t>(w.i);
-      E.link[E.link_at(1, w.k, ev)] = static_cast<uint8_t>(j);
-    } else {
-      E.col[aj] = static_cast<int16_t>(m);
-      E.acol[aj] = E.acol[ai];
-      E.acol[ai] = static_cast<int16_t>(m);
-      E.link[E.link_at(1, w.i, ev)] = static_cast<uint8_t>(j);
-      E.link[E.link_at(1, j, ev)] = static_cast<uint8_t>(w.k);
-      E.link[E.link_at(0, j, ev)] = static_cast<uint8_t>(w.i);
-      E.link[E.link_at(0, w.k, ev)] = static_cast<uint8_t>(j);
-    }
   }
-  // Every dipole with a moved parton, once: dipole (x, side) and its
-  // partner's opposite side share Q^2; a pair whose partner is a moved parton
-  // listed earlier was already taken from that side.
-  const int moved[3] = {w.i, j, w.k};
-  uint32_t mine[kMaxRefresh];
-  int count = 0;
-#pragma unroll
-  for (int m = 0; m < 3; ++m) {
-    const int x = moved[m];
-#pragma unroll
-    for (int side = 0; side < 2; ++side) {
-      const int k = E.link[E.link_at(side, x, ev)];
-      if (k == kNoLink) continue;
-      bool seen = false;
-#pragma unroll
-      for (int m2 = 0; m2 < m; ++m2) seen |= (k == moved[m2]);
-      if (seen || count == kMaxRefresh) continue;
-      mine[count++] = pack_refresh(task_index, x, side, k);
-    }
-  }
-  const int at = atomicAdd(n_jobs, count);
-  for (int c = 0; c < count; ++c) jobs[at + c] = mine[c];
+  const size_t ai = E.at(i, ev), aj = E.at(j, ev);
+  int16_t* line = s ? E.acol : E.col;
+  int16_t* other = s ? E.col : E.acol;
+  line[aj] = line[ai];
+  other[aj] = static_cast<int16_t>(m);
+  line[ai] = static_cast<int16_t>(m);
+  E.link[E.link_at(s, i, ev)] = split ? kNoLink : static_cast<uint8_t>(j);
+  E.link[E.link_at(s, j, ev)] = static_cast<uint8_t>(to);
+  E.link[E.link_at(1 - s, j, ev)] = split ? kNoLink : static_cast<uint8_t>(i);
+  E.link[E.link_at(1 - s, to, ev)] = static_cast<uint8_t>(j);
+  if (split) E.flav[ai] = static_cast<int8_t>(w.kappa);
+  E.flav[aj] = static_cast<int8_t>(split ? -w.kappa : kGluon);
+  // Every dipole with a moved parton, once.  A gluon: (i, j), (j, k) and the
+  // outer ones of i and k.  A splitting: the quark's on its colour side, the
+  // antiquark's on its anticolour side -- one of them to the spectator, the
+  // other the gluon's outer one -- and the spectator's outer one.
+  const int at = atomicAdd(n_jobs, 2 + (!split && oi != kNoLink ? 1 : 0) + (ok != kNoLink ? 1 : 0));
+  int c = at;
+  jobs[c++] = split ? pack_refresh(task_index, i, 0, side == 0 ? k : oi) : pack_refresh(task_index, i, side, j);
+  jobs[c++] = pack_refresh(task_index, j, s, to);
+  if (!split && oi != kNoLink) jobs[c++] = pack_refresh(task_index, i, 1 - side, oi);
+  if (ok != kNoLink) jobs[c++] = pack_refresh(task_index, k, side, ok);
   E.n_partons[ev] = j + 1;
   E.n_emissions[ev] += 1;
 }
 
 // Recompute one dipole of the refresh list from the stored momenta of its
 // two partons (the oracle's formulas, in the oracle's operand order).
+// refresh_task: the position, in the caller's queue, of the task whose event
+// the job belongs to.
+__device__ __forceinline__ int refresh_task(uint32_t job) { return static_cast<int>(job & 1023u); }
 template <bool kMulti>
-__device__ inline void refresh_dipole(const DevParams& P0, const Events& E, const EmitTask* tasks, uint32_t job) {
-  const int t = static_cast<int>(job & 1023u), x = static_cast<int>((job >> 10) & 255u);
+__device__ inline void refresh_dipole(const DevParams& P0, const Events& E, int64_t ev, uint32_t job) {
+  const int x = static_cast<int>((job >> 10) & 255u);
   const int k = static_cast<int>((job >> 18) & 255u), side = static_cast<int>((job >> 26) & 1u);
-  const int64_t ev = tasks[t].ev;
   const DevParams& P = params_of<kMulti>(P0, E, ev);
   const DipoleEntry d = make_dipole(P, 2.0 * mdot(load_p(E, x, ev), load_p(E, k, ev)));
-  store_dipole(E, ev, x, side, d);
-  store_dipole(E, ev, k, 1 - side, d);
+  store_dipole(E, ev, x, side, k, d);
 }
 
 }  // namespace gaps

@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(T, persist_min_blocks(T))
         EmitTask task;
         int r = kCycleFinished;
         if (limited) {
-          finish_event(E, ev, GAPS_STEP_LIMIT, exp(E.lnt[ev]));
+          finish_early(E, ev, GAPS_STEP_LIMIT, E.lnt[ev]);
         } else {
           // the rare undecided cycle takes its exact selection serially here:
           // the warp-wide form (fallback_warp) measured slower in this kernel
@@ -220,7 +220,8 @@ __global__ void __launch_bounds__(T, persist_min_blocks(T))
     if (queued > 0) {
       for (int q = tid; q < queued; q += T) cycle_emit<kMode>(P0, E, s_task[q], q, s_jobs, &s_count[4]);
       __syncthreads();
-      for (int j = tid; j < s_count[4]; j += T) refresh_dipole<kJobPhysics<kMode>>(P0, E, s_task, s_jobs[j]);
+      for (int j = tid; j < s_count[4]; j += T)
+        refresh_dipole<kJobPhysics<kMode>>(P0, E, s_task[refresh_task(s_jobs[j])].ev, s_jobs[j]);
       for (int q = tid; q < queued; q += T) s_alive[s_task[q].pad0 | (s_task[q].pad1 << 8)] = kSlotLive;
       __syncthreads();
     }

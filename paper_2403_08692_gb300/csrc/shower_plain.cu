@@ -49,8 +49,7 @@ __global__ void __launch_bounds__(256) k_me(DevParams P0, Events E) {
   E.link[E.link_at(0, 1, ev)] = kNoLink;
   E.link[E.link_at(1, 1, ev)] = 0;
   const DipoleEntry d = make_dipole(P, 2.0 * mdot(q, qbar));
-  store_dipole(E, ev, 0, 0, d);
-  store_dipole(E, ev, 1, 1, d);
+  store_dipole(E, ev, 0, 0, 1, d);
   E.weight[ev] = fma(P.me_a[fl - 1], fma(cth, cth, 1.0), P.me_b[fl - 1] * cth);
   E.me_flavour[ev] = fl;
   E.t[ev] = P.s;  // starting scale t0 = s
@@ -145,7 +144,8 @@ __global__ void __launch_bounds__(kStepThreads, GAPS_STEP_MIN_BLOCKS)
   __syncthreads();
   if (tid < s_naccept) cycle_emit<kMode>(P, E, s_task[tid], tid, s_jobs, &s_njobs);
   __syncthreads();
-  for (int j = tid; j < s_njobs; j += kStepThreads) refresh_dipole<kJobPhysics<kMode>>(P, E, s_task, s_jobs[j]);
+  for (int j = tid; j < s_njobs; j += kStepThreads) 
+    refresh_dipole<kJobPhysics<kMode>>(P, E, s_task[refresh_task(s_jobs[j])].ev, s_jobs[j]);
 }
 
 // Slot of this thread's item in an output list shared by the grid: one
@@ -246,7 +246,7 @@ __device__ __forceinline__ void select_role(const DevParams& P0, const Events& E
     if (lead) {
       const DevParams& P = job_params<kMulti>(P0, E, job);
       if (limited) {
-        finish_event(E, ev, GAPS_STEP_LIMIT, exp(E.lnt[ev]));
+        finish_early(E, ev, GAPS_STEP_LIMIT, E.lnt[ev]);
       } else {
         r = cycle_conclude<kMode>(P, E, ev, key, step, n, have, task);
       }
@@ -325,7 +325,8 @@ __global__ void __launch_bounds__(kStepThreads, GAPS_STEP_MIN_BLOCKS)
     __syncthreads();
     if (has) cycle_emit<kMode>(P0, E, s_task[tid], tid, s_jobs, &s_njobs);
     __syncthreads();
-    for (int j = tid; j < s_njobs; j += kStepThreads) refresh_dipole<kJobPhysics<kMode>>(P0, E, s_task, s_jobs[j]);
+    for (int j = tid; j < s_njobs; j += kStepThreads) 
+      refresh_dipole<kJobPhysics<kMode>>(P0, E, s_task[refresh_task(s_jobs[j])].ev, s_jobs[j]);
     if (has) E.status[s_task[tid].ev] = GAPS_ACTIVE;
     const int64_t at_list = warp_append_slot(has, list_count);
     if (at_list >= 0) list_out[at_list] = s_task[tid].ev;

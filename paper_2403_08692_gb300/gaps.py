@@ -136,6 +136,7 @@ PROBE_SIGNATURES = {
     "gaps_f32_from_f64_host": (C.c_int, [_P(C.c_double), _P(C.c_float), C.c_int64]),
     "gaps_log_fp64_device": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p]),
     "gaps_sqrt_obs_device": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p]),
+    "gaps_math_fp64_device": (C.c_int, [C.c_int32, C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p]),
     "gaps_probe_last_cuda_error": (C.c_char_p, []),
 }
 
@@ -398,6 +399,20 @@ def sqrt_obs_device(x, stream=None):
     y = torch.empty_like(x)
     _check_probe(load_probe().gaps_sqrt_obs_device(C.c_void_p(x.data_ptr()), C.c_void_p(y.data_ptr()),
                                                    int(x.numel()), _stream_handle(stream)), "gaps_sqrt_obs_device")
+    return y
+
+
+MATH_OPS = {"rcp": 0, "rsqrt": 1, "sqrt": 2, "exp": 3, "expm1": 4, "three_over": 5, "sin_2pi": 6, "cos_2pi": 7}
+
+
+def math_fp64_device(op, x, stream=None):
+    """A function of the kernels' FP64 mathematics (a name of MATH_OPS) on a
+    contiguous float64 CUDA tensor."""
+    import torch
+    x = x.contiguous()
+    y = torch.empty_like(x)
+    _check_probe(load_probe().gaps_math_fp64_device(MATH_OPS[op], C.c_void_p(x.data_ptr()), C.c_void_p(y.data_ptr()),
+                                                    int(x.numel()), _stream_handle(stream)), "gaps_math_fp64_device")
     return y
 
 
