@@ -212,13 +212,15 @@ enum {
   GAPS_SHOWER_PLAIN = 0,     /* one launch per shower step over the active events, host all-done check
                                 (App. C); a step runs the select/veto phase and the splittings the
                                 previous step accepted */
-  GAPS_SHOWER_PERSISTENT = 1 /* one launch; per-block event pools, compaction and refill (no host loop) */
+  GAPS_SHOWER_PERSISTENT = 1 /* one launch; per-warp event pools, refilled as events finish (no host loop) */
 };
 
 /* Launch shape of the persistent form.  block_threads: 64, 128, 256 or 512
- * events per block pool; compact_period: veto cycles between compactions
- * and refills of a pool (>= 1); blocks_per_sm: resident blocks per SM (0 =
- * as many as fit); layout: the record layout the autotuner found fastest
+ * threads per block (64 events per warp; batches with fewer events than the
+ * device has resident warps run one warp per block); compact_period (>= 1):
+ * a block generates its waiting emissions at the latest once 4
+ * compact_period per warp wait (at most 32); blocks_per_sm: resident blocks
+ * per SM (0 = as many as fit); layout: the record layout the autotuner found fastest
  * with this shape (gaps_autotune_persistent's output, to be used as the
  * batch's layout; launches take the layout from the batch and ignore this
  * field, which must be a valid layout). */
@@ -288,7 +290,7 @@ int gaps_pool_cycles(const gaps_batch* pool, int64_t first_cycle, int32_t n_cycl
                      const gaps_params* shared, void* stream);
 
 /* The same advance by the persistent form (time-sliced): one launch runs
- * every live event for up to `cycles` (1..255) more veto cycles in per-block
+ * every live event for up to `cycles` (1..255) more veto cycles in per-warp
  * pools (cfg as for gaps_shower_persistent, NULL for the default), and the
  * events still active afterwards make up the next active list.  `round`
  * numbers the slices (the `cycle` of gaps_pool_admit and
@@ -414,14 +416,13 @@ int gaps_shower_timed(const gaps_params* params, const gaps_batch* batch, int mo
                       double* kernel_ms_out, void* stream);
 
 /* The persistent form (Sec. 2, without the cutoff wait of Fig. 3): one
- * launch runs every event to the cutoff.  Each block keeps a pool of events,
- * two per thread for pools of up to 256 threads, runs cfg->compact_period
- * veto cycles on it (each warp on its own events, no block barrier; a
- * thread runs whichever of its events can run), generates the period's
- * accepted emissions together, packs the still-active events to the front
- * (warp ballot) and refills the free slots from a global event cursor.  An
- * event with a queued emission skips its selects until the end of the
- * period.  Events are identical to the plain form's (same draws, same cycle
+ * launch runs every event to the cutoff.  Each warp keeps a pool of 64
+ * events in shared memory and runs their veto cycles, the trials of all its
+ * events spread over its lanes; a block's warps generate the emissions its
+ * events accepted together, once enough wait (an event with an accepted
+ * emission skips its selects until then), and refill the slots of finished
+ * events from a global event cursor.  Events are identical to the plain
+ * form's (same draws, same winner, cutoff and veto
  * code).  cfg = NULL uses {128, 8, 0}.  Fully asynchronous: no host synchronisation; the
  * workspace counters record finished and step-limited events. */
 int gaps_shower_persistent(const gaps_params* params, const gaps_batch* batch,

@@ -392,14 +392,25 @@ __device__ __forceinline__ Uniforms draw2(const DevParams& P, uint32_t ev, uint3
   return Uniforms{to_unit(r.x, r.y), to_unit(r.z, r.w)};
 }
 
-// FNV-1a, 64 bit, over the eight little-endian bytes of a decision word.
-__device__ __forceinline__ unsigned long long fnv1a64(unsigned long long h, unsigned long long word) {
-#pragma unroll
-  for (int b = 0; b < 8; ++b) {
-    h ^= (word >> (8 * b)) & 0xFFull;
-    h *= 1099511628211ull;
+// FNV-1a, 64 bit, over the eight little-endian bytes of a decision word:
+// cycle (bytes 0..3), splitter slot, side, kernel, accepted.  Bytes 2 and 3
+// are zero for the first 65536 cycles: their steps only multiply, by a
+// constant together with byte 1's.
+constexpr unsigned long long kFnvPrime = 1099511628211ull;
+__device__ __forceinline__ unsigned long long fnv1a64(unsigned long long h, uint32_t cycle, uint32_t i, uint32_t side,
+                                                      uint32_t kappa, uint32_t accepted) {
+  h = (h ^ (cycle & 255u)) * kFnvPrime;
+  h ^= (cycle >> 8) & 255u;
+  if (cycle < 65536u) {
+    h *= kFnvPrime * kFnvPrime * kFnvPrime;
+  } else {
+    h = (h * kFnvPrime ^ ((cycle >> 16) & 255u)) * kFnvPrime;
+    h = (h ^ (cycle >> 24)) * kFnvPrime;
   }
-  return h;
+  h = (h ^ i) * kFnvPrime;
+  h = (h ^ side) * kFnvPrime;
+  h = (h ^ kappa) * kFnvPrime;
+  return (h ^ accepted) * kFnvPrime;
 }
 constexpr unsigned long long kFnvBasis = 14695981039346656037ull;
 

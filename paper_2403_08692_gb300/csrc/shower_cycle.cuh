@@ -73,27 +73,35 @@ struct DipoleEntry {
   float2 screen;
 };
 
+// Whether a dipole of mass squared q2 has phase space: not Q^2 < 4 t_C, the
+// sign of their difference (exact where they are close) read from its bits.
+__device__ __forceinline__ bool has_phase_space(const DevParams& P, double q2) {
+  return __double_as_longlong(q2 - 4.0 * P.tc) >= 0;
+}
+// The entry of a dipole without.
+__device__ __forceinline__ DipoleEntry no_dipole(double q2) {
+  DipoleEntry d;
+  d.rec.q2 = q2;
+  d.rec.zp = d.rec.inv_ls = d.rec.ls = 0.0;
+  d.screen = make_float2(-1.0f, -1.0f);
+  return d;
+}
+
 __device__ __forceinline__ DipoleEntry make_dipole(const DevParams& P, double q2) {
+  if (!has_phase_space(P, q2)) return no_dipole(q2);
   DipoleEntry d;
   d.rec.q2 = q2;
   // b = sqrt(1 - 4 t_C/Q^2) = a / sqrt(Q^2 a) with a = Q^2 - 4 t_C: one
-  // reciprocal square root instead of a division and a square root; the sign
-  // of a is the oracle's test Q^2 < 4 t_C (their difference is exact where
-  // they are close)
+  // reciprocal square root instead of a division and a square root
   const double a = q2 - 4.0 * P.tc;
-  if (__double_as_longlong(a) < 0) {
-    d.rec.zp = d.rec.inv_ls = d.rec.ls = 0.0;
-    d.screen = make_float2(-1.0f, -1.0f);
-    return d;
-  }
   const double b = __double_as_longlong(a) > 0 ? a * rsqrt_fp64(q2 * a) : 0.0;
   const double b1 = 1.0 + b;
   d.rec.zp = 0.5 * b1;
   const double ls = log_fp64((b1 * b1) * (q2 * P.inv_4tc));
   d.rec.ls = ls;
   d.rec.inv_ls = rcp_fp64(ls);
-  d.screen = make_float2(1.0f / (P.as2pi_f * f32_from_f64(ls)),
-                         1.0f / (P.as2pi_f * 0.5f * static_cast<float>(kTR) * f32_from_f64(b)));
+  d.screen = make_float2(__fdividef(1.0f, P.as2pi_f * f32_from_f64(ls)),
+                         __fdividef(1.0f, P.as2pi_f * 0.5f * static_cast<float>(kTR) * f32_from_f64(b)));
   return d;
 }
 
@@ -424,28 +432,28 @@ enum : int { kScreenNone = 0, kScreenWinner = 1, kScreenUndecided = 2 };
 
 // The screen's verdict; for a certain winner its exact scale (from the FP64
 // cache) and the winner's data in `task`.  Writes nothing to the record.
+// best_ub, best_lb: bounds of the best trial's key; others_hi: the largest
+// upper bound of the others'; best_code < 0: no trial.
 template <int kMode>
-__device__ __forceinline__ int screen_verdict(const DevParams& P, const Events& E, int64_t ev, double lnt,
-                                              const Screen& sc, EmitTask& task) {
-  const float best_key = sc.best_key, best_m = sc.best_m, others_hi = sc.others_hi;
-  const int best_code = sc.best_code;
-  const uint32_t best_hi = sc.best_hi, best_lo = sc.best_lo;
+__device__ __forceinline__ int screen_verdict(const DevParams& P, const Events& E, int64_t ev, double lnt, float best_ub,
+                                              float best_lb, float others_hi, int best_code, uint32_t best_aux,
+                                              uint32_t best_hi, uint32_t best_lo, EmitTask& task) {
 
   // Cutoff threshold in key units: t' > t_C  <=>  key > log2(t_C / t).
   const float lt2 = f32_from_f64(lnt) * 1.44269504f;
   const float thr = P.lg2_tc_f - lt2;
   const float thr_m = 2e-6f * (1.0f + fabsf(lt2) + fabsf(P.lg2_tc_f));
 
-  if (best_code < 0 || fmaxf(best_key + best_m, others_hi) < thr - thr_m) {
+  if (best_code < 0 || fmaxf(best_ub, others_hi) < thr - thr_m) {
     return kScreenNone;  // certainly no trial above the cutoff
   }
-  if (best_key - best_m > thr + thr_m && others_hi < best_key - best_m) {
+  if (best_lb > thr + thr_m && others_hi < best_lb) {
     // Certain winner: its scale exactly, from the FP64 cache.
     const int dcode = best_code >> 3, kappa = best_code & 7;
     const int i = dcode >> 1, side = dcode & 1;
-    const int k = static_cast<int>(sc.best_aux & 255u);
+    const int k = static_cast<int>(best_aux & 255u);
     const DipoleRecord rec = E.drec[E.at(side == 0 ? i : k, ev)];
-    const bool gluon = (sc.best_aux & 256u) != 0u;  // as the screen read them: no second load
+    const bool gluon = (best_aux & 256u) != 0u;  // as the screen read them: no second load
     const bool combined = gluon && per_dipole<kMode>(P);
     const int kind = combined ? kKindUnchosen : (gluon ? (kappa == 0 ? kGtoGG : kGtoQQ) : kQtoQG);
     const double inv_c =
@@ -475,7 +483,8 @@ __device__ inline int cycle_screen(const DevParams& P, const Events& E, int64_t 
   E.n_steps[ev] = step + 1;
   E.n_trials[ev] += sc.trials;
   E.n_dipoles[ev] += sc.dipoles;
-  return screen_verdict<kMode>(P, E, ev, lnt, sc, task);
+  return screen_verdict<kMode>(P, E, ev, lnt, sc.best_key + sc.best_m, sc.best_key - sc.best_m, sc.others_hi,
+                               sc.best_code, sc.best_aux, sc.best_hi, sc.best_lo, task);
 }
 
 // The exact FP64 selection for the undecided events of a warp, each computed
@@ -569,28 +578,30 @@ __device__ __forceinline__ bool accept_or_veto(const DevParams& P, const Events&
   const U4 rw = philox_draw<kMode>(P, key, static_cast<uint32_t>(step), 0u, kDrawWinner);
   bool accept;
   {
-    const float zpf = f32_from_f64(task.zp);
-    const float zmf = f32_from_f64(1.0 - task.zp);
-    const float lf = f32_from_f64(task.ls);
+    // z- = t_C / (Q^2 z+) (the same as 1 - z+, without its cancellation);
+    // quotients by the two-ulp __fdividef.
+    const float zpf = seed_of(task.zp);  // z+ in [1/2, 1]
+    const float q2f = f32_from_f64(task.q2);
+    const float zmf = __fdividef(P.tcf, q2f * zpf);
     const float rzf = unit_float(rw.x, rw.y);
     float z, e;  // z and 1 - z
     if (task.kind == kGtoQQ) {
       z = fmaf(zpf - zmf, rzf, zmf);
       e = fmaf(-(zpf - zmf), rzf, zpf);
     } else {
-      z = zmf - zpf * expm1f(-rzf * lf);
-      e = zpf * __expf(-rzf * lf);
+      const float x = -rzf * f32_from_f64(task.ls);
+      z = fmaf(-zpf, expm1f(x), zmf);
+      e = zpf * __expf(x);
     }
     const float lnt_f = f32_from_f64(task.lnt);
-    const float y = __expf(lnt_f) / (f32_from_f64(task.q2) * z * e);
-    const float as_ratio = P.fixed ? 1.0f : P.as_mz_over_f / (1.0f + P.as_b0_f * (lnt_f - P.ln_mz2_f));
+    const float y = __fdividef(__expf(lnt_f), q2f * z * e);
+    const float as_ratio = P.fixed ? 1.0f : __fdividef(P.as_mz_over_f, fmaf(P.as_b0_f, lnt_f - P.ln_mz2_f, 1.0f));
     float pr;  // P(z, y) / P^over(z)
-    if (task.kind == kQtoQG) {
-      pr = e / (e + z * y) - 0.5f * (1.0f + z) * e;
-    } else if (task.kind == kGtoGG) {
-      pr = e / (e + z * y) - e + 0.5f * z * e * e;
+    if (task.kind == kGtoQQ) {
+      pr = fmaf(-2.0f * z, e, 1.0f);
     } else {
-      pr = 1.0f - 2.0f * z * e;
+      const float soft = __fdividef(e, fmaf(z, y, e));
+      pr = task.kind == kQtoQG ? fmaf(-0.5f * (1.0f + z), e, soft) : fmaf(0.5f * z * e, e, soft - e);
     }
     const float ratio = (1.0f - y) * as_ratio * pr;
     const float rvf = unit_float(rw.z, rw.w);
@@ -603,12 +614,7 @@ __device__ __forceinline__ bool accept_or_veto(const DevParams& P, const Events&
       accept = y < 1.0f && rvf < ratio;
     }
   }
-  const unsigned long long word = static_cast<unsigned long long>(step) |
-                                  (static_cast<unsigned long long>(task.i) << 32) |
-                                  (static_cast<unsigned long long>(task.side) << 40) |
-                                  (static_cast<unsigned long long>(task.kappa) << 48) |
-                                  (static_cast<unsigned long long>(accept ? 1 : 0) << 56);
-  hash = fnv1a64(hash, word);
+  hash = fnv1a64(hash, static_cast<uint32_t>(step), task.i, task.side, task.kappa, accept ? 1u : 0u);
   task.rz_hi = rw.x;
   task.rz_lo = rw.y;
   return accept;
@@ -677,12 +683,13 @@ __device__ inline int cycle_select_veto(const DevParams& P0, const Events& E, in
 
 // Phase 2: GenerateEmission -- azimuth, the final-final dipole map, colours
 // and the new parton in slot n.  The dipoles whose invariant mass moved are
-// appended to the block's refresh list (jobs, *n_jobs) under task_index; the
-// caller recomputes them with refresh_dipole after a block barrier, spread
-// over all of its threads, so that this FP64-heavy step runs in full warps.
-template <int kMode>
-__device__ inline void cycle_emit(const DevParams& P0, const Events& E, const EmitTask& w, int task_index,
-                                  uint32_t* jobs, int* n_jobs) {
+// put in the block's refresh list (reserve(count) gives their first place,
+// put(place, job) writes one) under task_index; the caller recomputes them
+// after a block barrier, spread over all of its threads, so that this
+// FP64-heavy step runs in full warps.
+template <int kMode, class Reserve, class Put>
+__device__ inline void cycle_emit(const DevParams& P0, const Events& E, const EmitTask& w, Reserve reserve, Put put,
+                                  int task_index) {
   const int64_t ev = w.ev;
   const int job = kJobKey<kMode> ? static_cast<int>(E.job_of[ev]) : 0;
   const DevParams& P = job_params<kJobPhysics<kMode>>(P0, E, job);
@@ -733,28 +740,34 @@ __device__ inline void cycle_emit(const DevParams& P0, const Events& E, const Em
   // outer ones of i and k.  A splitting: the quark's on its colour side, the
   // antiquark's on its anticolour side -- one of them to the spectator, the
   // other the gluon's outer one -- and the spectator's outer one.
-  const int at = atomicAdd(n_jobs, 2 + (!split && oi != kNoLink ? 1 : 0) + (ok != kNoLink ? 1 : 0));
-  int c = at;
-  jobs[c++] = split ? pack_refresh(task_index, i, 0, side == 0 ? k : oi) : pack_refresh(task_index, i, side, j);
-  jobs[c++] = pack_refresh(task_index, j, s, to);
-  if (!split && oi != kNoLink) jobs[c++] = pack_refresh(task_index, i, 1 - side, oi);
-  if (ok != kNoLink) jobs[c++] = pack_refresh(task_index, k, side, ok);
+  int at = reserve(2 + (!split && oi != kNoLink ? 1 : 0) + (ok != kNoLink ? 1 : 0));
+  put(at++, split ? pack_refresh(task_index, i, 0, side == 0 ? k : oi) : pack_refresh(task_index, i, side, j));
+  put(at++, pack_refresh(task_index, j, s, to));
+  if (!split && oi != kNoLink) put(at++, pack_refresh(task_index, i, 1 - side, oi));
+  if (ok != kNoLink) put(at++, pack_refresh(task_index, k, side, ok));
   E.n_partons[ev] = j + 1;
   E.n_emissions[ev] += 1;
 }
 
-// Recompute one dipole of the refresh list from the stored momenta of its
-// two partons (the oracle's formulas, in the oracle's operand order).
+// One dipole of the refresh list.
 // refresh_task: the position, in the caller's queue, of the task whose event
 // the job belongs to.
 __device__ __forceinline__ int refresh_task(uint32_t job) { return static_cast<int>(job & 1023u); }
-template <bool kMulti>
-__device__ inline void refresh_dipole(const DevParams& P0, const Events& E, int64_t ev, uint32_t job) {
+// The invariant mass of a refresh job's dipole from the stored momenta of its
+// two partons (the oracle's formula, in the oracle's operand order).
+__device__ __forceinline__ double refresh_mass(const Events& E, int64_t ev, uint32_t job) {
+  const int x = static_cast<int>((job >> 10) & 255u), k = static_cast<int>((job >> 18) & 255u);
+  return 2.0 * mdot(load_p(E, x, ev), load_p(E, k, ev));
+}
+__device__ __forceinline__ void refresh_store(const Events& E, int64_t ev, uint32_t job, const DipoleEntry& d) {
   const int x = static_cast<int>((job >> 10) & 255u);
   const int k = static_cast<int>((job >> 18) & 255u), side = static_cast<int>((job >> 26) & 1u);
-  const DevParams& P = params_of<kMulti>(P0, E, ev);
-  const DipoleEntry d = make_dipole(P, 2.0 * mdot(load_p(E, x, ev), load_p(E, k, ev)));
   store_dipole(E, ev, x, side, k, d);
+}
+template <bool kMulti>
+__device__ inline void refresh_dipole(const DevParams& P0, const Events& E, int64_t ev, uint32_t job) {
+  const DevParams& P = params_of<kMulti>(P0, E, ev);
+  refresh_store(E, ev, job, make_dipole(P, refresh_mass(E, ev, job)));
 }
 
 }  // namespace gaps

@@ -142,7 +142,9 @@ __global__ void __launch_bounds__(kStepThreads, GAPS_STEP_MIN_BLOCKS)
     }
   }
   __syncthreads();
-  if (tid < s_naccept) cycle_emit<kMode>(P, E, s_task[tid], tid, s_jobs, &s_njobs);
+  if (tid < s_naccept)
+    cycle_emit<kMode>(P, E, s_task[tid], [&](int count) { return atomicAdd(&s_njobs, count); },
+                      [&](int at, uint32_t job) { s_jobs[at] = job; }, tid);
   __syncthreads();
   for (int j = tid; j < s_njobs; j += kStepThreads) 
     refresh_dipole<kJobPhysics<kMode>>(P, E, s_task[refresh_task(s_jobs[j])].ev, s_jobs[j]);
@@ -323,7 +325,9 @@ __global__ void __launch_bounds__(kStepThreads, GAPS_STEP_MIN_BLOCKS)
     const bool has = k < len;
     if (has) s_task[tid] = tasks_in[k];
     __syncthreads();
-    if (has) cycle_emit<kMode>(P0, E, s_task[tid], tid, s_jobs, &s_njobs);
+    if (has)
+      cycle_emit<kMode>(P0, E, s_task[tid], [&](int count) { return atomicAdd(&s_njobs, count); },
+                        [&](int at, uint32_t job) { s_jobs[at] = job; }, tid);
     __syncthreads();
     for (int j = tid; j < s_njobs; j += kStepThreads) 
       refresh_dipole<kJobPhysics<kMode>>(P0, E, s_task[refresh_task(s_jobs[j])].ev, s_jobs[j]);
