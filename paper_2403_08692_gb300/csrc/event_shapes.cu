@@ -6,22 +6,22 @@
 // a warp handle events of the same size: the O(n^3) loops of thrust and
 // Durham then run with no lane waiting on a larger neighbour.  Events of up
 // to 16 partons take one thread each, with per-thread arrays (in batches of
-// fewer than 50 000 events, groups of 4 lanes).  Larger events take a warp
-// each: the event's momenta sit in shared memory, the lanes split the O(n^2)
-// pairs of each search and reduce their partial results in the serial
-// loop's order (the first pair wins ties, as in the oracle), and the O(n)
-// FP64 steps run on every lane alike.  A single thread takes about 0.2 ms
-// for one 16-parton event and 64 times that for 64 partons, and a launch
-// waits for its largest event; the groups cut that wait by their width.
+// fewer than 50 000 events, groups of 4 lanes: the event's momenta sit in
+// shared memory, the lanes split the pairs of each search and reduce their
+// partial results in the serial loop's order, and the O(n) FP64 steps run on
+// every lane alike, so the results are the one-thread results).  Larger
+// events take a warp each (event_shapes_warp), with the O(n) steps spread
+// over the lanes and a nearest-neighbour table in the clustering.
 //
 // Precision.  As in the shower, the searches run in FP32 and the answers in
 // FP64:
 //  * Thrust.  Every candidate partition P = sum s_i p_i of the exact
 //    algorithm (planes through every pair, both signs of the pair) is scored
-//    |P|^2 in FP32 and identified by its bitmask; the two best distinct
+//    |P|^2 in FP32 and identified by its bitmask; the best distinct
 //    partitions are tracked.  When the best beats the runner-up by more than
-//    the FP32 error bound, its |P| and axis are recomputed in FP64; otherwise
-//    (or for more than 64 partons) the whole search runs in FP64.
+//    the FP32 error bound (or, in large events, is the longest of those within
+//    it), its |P| and axis are recomputed in FP64; otherwise the whole search
+//    runs in FP64.
 //  * Durham.  Pair distances min(E_i^2, E_j^2) |u_i - u_j|^2 (u = unit
 //    momentum, free of the 1 - cos cancellation) are compared in FP32 with a
 //    per-pair error bound; every pair that could be the minimum is evaluated
@@ -724,6 +724,622 @@ __device__ void event_shapes_group(const DevParams& P0, const Events& E, int64_t
     for (int h = 0; h < 4; ++h) E.obs[h * E.stride + ev] = yres[h];
 }
 
+// ------------------------------------------------- a warp per large event
+// The event of a warp in shared memory.  f: FP32 momenta in the thrust
+// search, then unit directions with E^2.  Durham's nearest neighbours: jet
+// r's smallest upper bound ub of the distance to another jet (near, with
+// lower bound lb) and a lower bound lb2 of all others: the smallest of theirs
+// (near2's), or no more than that once near2 is gone (near2 = kGone).
+template <int MAXJ>
+struct WarpEvent {
+  double j[4][MAXJ];  // E, px, py, pz
+  float4 f[MAXJ];
+  float ub[MAXJ], lb[MAXJ], lb2[MAXJ];
+  uint8_t near[MAXJ], near2[MAXJ];
+};
+
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// A partition of up to 32 W partons as sign bits (set: the minus side), the
+// first of each 32 highest.  Top two distinct ones by score, as Top2.
+template <int W>
+struct Partition {
+  uint32_t w[W];
+  __device__ __forceinline__ bool operator==(const Partition& o) const {
+    uint32_t d = 0u;
+#pragma unroll
+    for (int c = 0; c < W; ++c) d |= w[c] ^ o.w[c];
+    return d == 0u;
+  }
+};
+// The kTop best distinct partitions by score, in no order; `least` is the
+// smallest of their scores.
+constexpr int kTop = 4;
+template <int W>
+struct TopPartitions {
+  float s[kTop];
+  Partition<W> m[kTop];
+  float least = -1.0f;
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int t = 0; t < kTop; ++t) {
+      s[t] = -1.0f;
+#pragma unroll
+      for (int c = 0; c < W; ++c) m[t].w[c] = 0u;
+    }
+  }
+  // (a score at or below the least changes nothing)
+  __device__ __forceinline__ void add(float v, const Partition<W>& p) {
+    int at = -1, low = 0;
+#pragma unroll
+    for (int t = 0; t < kTop; ++t) {
+      if (s[t] >= 0.0f && m[t] == p) at = t;
+      if (s[t] == least) low = t;
+    }
+    const int to = at >= 0 ? at : low;
+    least = INFINITY;
+#pragma unroll
+    for (int t = 0; t < kTop; ++t) {
+      if (t == to) {
+        s[t] = at >= 0 ? fmaxf(s[t], v) : v;
+        m[t] = p;
+      }
+      least = fminf(least, s[t]);
+    }
+  }
+};
+
+// FP32 bounds of the distance of jets a and b (unit directions, E^2 in w):
+// per-pair relative error 4e-6 + 1e-6 / |u_a - u_b|.
+__device__ __forceinline__ void pair_bounds(const float4& a, const float4& b, float& ub, float& lb) {
+  const float dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z;
+  const float d = dot3f(dx, dy, dz, dx, dy, dz);
+  const float y = fminf(a.w, b.w) * d;
+  const float rel = 4.0e-6f + 1.0e-6f * rsqrtf(fmaxf(d, 1e-30f));
+  ub = fmaf(y, 1.0f + rel, 1e-30f);
+  lb = y * (1.0f - rel);
+}
+
+// A row of the nearest-neighbour table.
+constexpr int kGone = 255;
+struct Row {
+  float ub, lb, lb2;
+  int near, near2;
+  __device__ __forceinline__ void clear() {
+    ub = lb = lb2 = INFINITY;
+    near = near2 = kGone;
+  }
+  __device__ __forceinline__ void add(float u, float l, int k) {
+    if (u < ub) {
+      if (lb < lb2) {
+        lb2 = lb;
+        near2 = near;
+      }
+      ub = u;
+      lb = l;
+      near = k;
+    } else if (l < lb2) {
+      lb2 = l;
+      near2 = k;
+    }
+  }
+};
+template <int MAXJ>
+__device__ __forceinline__ Row load_row(const WarpEvent<MAXJ>& a, int r) {
+  return Row{a.ub[r], a.lb[r], a.lb2[r], a.near[r], a.near2[r]};
+}
+template <int MAXJ>
+__device__ __forceinline__ void store_row(WarpEvent<MAXJ>& a, int r, const Row& row) {
+  a.ub[r] = row.ub;
+  a.lb[r] = row.lb;
+  a.lb2[r] = row.lb2;
+  a.near[r] = static_cast<uint8_t>(row.near);
+  a.near2[r] = static_cast<uint8_t>(row.near2);
+}
+
+// |p| of jet i.
+template <int MAXJ>
+__device__ __forceinline__ double jet_length(const WarpEvent<MAXJ>& a, int i) {
+  return sqrt_obs(dot3(a.j[1][i], a.j[2][i], a.j[3][i], a.j[1][i], a.j[2][i], a.j[3][i]));
+}
+// y of jets i and k with the oracle's FP64 formula.
+template <int MAXJ>
+__device__ __forceinline__ double jet_distance(const WarpEvent<MAXJ>& a, int i, int k, double inv_s) {
+  const double cosik = dot3(a.j[1][i], a.j[2][i], a.j[3][i], a.j[1][k], a.j[2][k], a.j[3][k]) /
+                       (jet_length(a, i) * jet_length(a, k));
+  return 2.0 * fmin(a.j[0][i] * a.j[0][i], a.j[0][k] * a.j[0][k]) * (1.0 - cosik) * inv_s;
+}
+
+// thrust_fp64 over the warp (see thrust_fp64_group).
+template <int MAXJ>
+__device__ __noinline__ double thrust_fp64_warp(int n, const WarpEvent<MAXJ>& a, double sum_abs, int lane, double& ax,
+                                                double& ay, double& az) {
+  double best2 = -1.0, bx = 0.0, by = 0.0, bz = 0.0;
+  int bidx = 0x7fffffff;
+  PairWalk w;
+  for (w.start(n, lane); w.valid(n); w.next<32>(n)) {
+    const int j = w.j, k = w.k();
+    const double nx = cross(a.j[2][j], a.j[3][k], a.j[3][j], a.j[2][k]);
+    const double ny = cross(a.j[3][j], a.j[1][k], a.j[1][j], a.j[3][k]);
+    const double nz = cross(a.j[1][j], a.j[2][k], a.j[2][j], a.j[1][k]);
+    if (nx == 0.0 && ny == 0.0 && nz == 0.0) continue;
+    double px = 0.0, py = 0.0, pz = 0.0;
+    for (int i = 0; i < n; ++i) {
+      if (i == j || i == k) continue;
+      const double sg = dot3(a.j[1][i], a.j[2][i], a.j[3][i], nx, ny, nz) >= 0.0 ? 1.0 : -1.0;
+      px = fma(sg, a.j[1][i], px);
+      py = fma(sg, a.j[2][i], py);
+      pz = fma(sg, a.j[3][i], pz);
+    }
+    for (int c = 0; c < 4; ++c) {
+      const double fj = (c & 2) ? -1.0 : 1.0, fk = (c & 1) ? -1.0 : 1.0;
+      const double cx = fma(fk, a.j[1][k], fma(fj, a.j[1][j], px));
+      const double cy = fma(fk, a.j[2][k], fma(fj, a.j[2][j], py));
+      const double cz = fma(fk, a.j[3][k], fma(fj, a.j[3][j], pz));
+      const double c2 = dot3(cx, cy, cz, cx, cy, cz);
+      if (c2 > best2) {  // within a lane the positions rise: the first wins ties
+        best2 = c2;
+        bidx = 4 * w.p + c;
+        bx = cx;
+        by = cy;
+        bz = cz;
+      }
+    }
+  }
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const double o2 = __shfl_xor_sync(0xffffffffu, best2, off);
+    const int oi = __shfl_xor_sync(0xffffffffu, bidx, off);
+    const double ox = __shfl_xor_sync(0xffffffffu, bx, off), oy = __shfl_xor_sync(0xffffffffu, by, off);
+    const double oz = __shfl_xor_sync(0xffffffffu, bz, off);
+    if (o2 > best2 || (o2 == best2 && oi < bidx)) {
+      best2 = o2;
+      bidx = oi;
+      bx = ox;
+      by = oy;
+      bz = oz;
+    }
+  }
+  if (best2 < 0.0) {  // collinear: T = 1 along the first momentum
+    const double l = jet_length(a, 0);
+    ax = a.j[1][0] / l;
+    ay = a.j[2][0] / l;
+    az = a.j[3][0] / l;
+    return 1.0;
+  }
+  const double l = sqrt_obs(best2), inv_l = 1.0 / l;
+  ax = bx * inv_l;
+  ay = by * inv_l;
+  az = bz * inv_l;
+  return l / sum_abs;
+}
+
+// The observables of one event of more than 16 partons, by a warp.
+//
+// Thrust: the lanes take the pairs; a pair's partition is built from the
+// signs of the other momenta's products with its normal without a branch (the
+// pair's own two, whose products are rounding, are taken out of the sum
+// afterwards).  With the four best distinct partitions known, those within
+// the FP32 error of the best are compared in FP64, unless the fourth is one
+// of them (with many partons the best two often are: one event in fifty of 17
+// .. 80 partons was left to the exact search, which takes half a
+// millisecond); the winner must also be the one its own axis defines, which
+// the longest one is.
+//
+// Durham: a merge changes the distances to one jet only, so every jet keeps
+// its nearest neighbour and a lower bound of the others' (Row); a merge renews
+// the rows that pointed at the two merged jets, by the whole warp, and offers
+// the new jet to the others.  A row whose second neighbour is gone keeps the
+// old bound, and is renewed only where that bound is too low to decide.  One jet pair decides a merge from its
+// FP32 bounds as before; y in FP64 is only formed for the four merges that
+// are recorded.
+//
+// Bound by FP32 issue in the thrust pairs (n^3 / 2 products; issue slots 65 %
+// busy).  20 000 RAMBO events of 17 .. 80 partons: 25.3 -> 3.2 ms against every
+// merge searching all its pairs twice, events beyond 64 partons searched in
+// FP64, and two blocks per SM with a fixed share of the events each (with
+// these in place: 7.3 ms with two partitions kept and every row that pointed
+// at a merged jet renewed, 4.8 ms with fixed shares).
+template <int MAXJ>
+__device__ void event_shapes_warp(const DevParams& P0, const Events& E, int64_t ev, int n, WarpEvent<MAXJ>& a, int lane) {
+  constexpr int W = MAXJ / 32;
+  const DevParams& P = params_of_event(P0, E, ev);
+  double sum_abs = 0.0;
+  for (int i = lane; i < n; i += 32) {
+    const size_t at = E.at(i, ev);
+    const double x = E.px[at], y = E.py[at], z = E.pz[at];
+    a.j[0][i] = E.e[at];
+    a.j[1][i] = x;
+    a.j[2][i] = y;
+    a.j[3][i] = z;
+    a.f[i] = make_float4(f32_from_f64(x), f32_from_f64(y), f32_from_f64(z), 0.0f);
+    sum_abs += sqrt_obs(dot3(x, y, z, x, y, z));
+  }
+  sum_abs = warp_sum(sum_abs);
+  const float sum_absf = f32_from_f64(sum_abs);
+  __syncwarp();
+
+  // ---- thrust
+  TopPartitions<W> top;
+  top.clear();
+  uint32_t full[W];  // the bits in use
+#pragma unroll
+  for (int c = 0; c < W; ++c) {
+    const int r = n - 32 * c;
+    full[c] = r >= 32 ? 0xffffffffu : (r > 0 ? (1u << r) - 1u : 0u);
+  }
+  // bit of parton i: the last of its word is lowest
+  const auto bit_of = [&](int i, int c) { return i >> 5 == c ? 1u << (min(n - 32 * c, 32) - 1 - (i & 31)) : 0u; };
+  PairWalk pw;
+#pragma unroll 1
+  for (pw.start(n, lane); pw.valid(n); pw.next<32>(n)) {
+    const int j = pw.j, k = pw.k();
+    const float4 pj = a.f[j], pk = a.f[k];
+    const float nx = crossf(pj.y, pk.z, pj.z, pk.y);
+    const float ny = crossf(pj.z, pk.x, pj.x, pk.z);
+    const float nz = crossf(pj.x, pk.y, pj.y, pk.x);
+    if (nx == 0.0f && ny == 0.0f && nz == 0.0f) continue;
+    float px = 0.0f, py = 0.0f, pz = 0.0f;
+    Partition<W> m;
+#pragma unroll
+    for (int c = 0; c < W; ++c) {
+      uint32_t bits = 0u;
+      const int end = min(n, 32 * c + 32);
+#pragma unroll 4
+      for (int i = 32 * c; i < end; ++i) {
+        const float4 q = a.f[i];
+        const uint32_t s = __float_as_uint(dot3f(q.x, q.y, q.z, nx, ny, nz));
+        const float sg = __uint_as_float((s & 0x80000000u) | 0x3f800000u);
+        px = fmaf(sg, q.x, px);
+        py = fmaf(sg, q.y, py);
+        pz = fmaf(sg, q.z, pz);
+        bits = __funnelshift_l(s, bits, 1);
+      }
+      m.w[c] = bits;
+    }
+    // without the pair itself
+    uint32_t bj = 0u, bk = 0u;
+#pragma unroll
+    for (int c = 0; c < W; ++c) {
+      const uint32_t jb = bit_of(j, c), kb = bit_of(k, c);
+      bj |= m.w[c] & jb;
+      bk |= m.w[c] & kb;
+      m.w[c] &= ~(jb | kb);
+    }
+    const float sj = bj ? 1.0f : -1.0f, sk = bk ? 1.0f : -1.0f;
+    px = fmaf(sk, pk.x, fmaf(sj, pj.x, px));
+    py = fmaf(sk, pk.y, fmaf(sj, pj.y, py));
+    pz = fmaf(sk, pk.z, fmaf(sj, pj.z, pz));
+#pragma unroll 1
+    for (int c4 = 0; c4 < 4; ++c4) {
+      const float fj = (c4 & 2) ? -1.0f : 1.0f, fk = (c4 & 1) ? -1.0f : 1.0f;
+      const float cx = fmaf(fk, pk.x, fmaf(fj, pj.x, px));
+      const float cy = fmaf(fk, pk.y, fmaf(fj, pj.y, py));
+      const float cz = fmaf(fk, pk.z, fmaf(fj, pj.z, pz));
+      const float score = dot3f(cx, cy, cz, cx, cy, cz);
+      if (score <= top.least) continue;
+      Partition<W> t;
+#pragma unroll
+      for (int c = 0; c < W; ++c)
+        t.w[c] = m.w[c] | ((c4 & 2) ? bit_of(j, c) : 0u) | ((c4 & 1) ? bit_of(k, c) : 0u);
+      if (t.w[0] & bit_of(0, 0)) {  // a partition and its complement are one candidate
+#pragma unroll
+        for (int c = 0; c < W; ++c) t.w[c] = ~t.w[c] & full[c];
+      }
+      top.add(score, t);
+    }
+  }
+#pragma unroll 1
+  for (int off = 1; off < 32; off <<= 1) {
+    float os[kTop];
+    Partition<W> om[kTop];
+#pragma unroll
+    for (int t = 0; t < kTop; ++t) {  // all before the first addition
+      os[t] = __shfl_xor_sync(0xffffffffu, top.s[t], off);
+#pragma unroll
+      for (int c = 0; c < W; ++c) om[t].w[c] = __shfl_xor_sync(0xffffffffu, top.m[t].w[c], off);
+    }
+#pragma unroll
+    for (int t = 0; t < kTop; ++t)
+      if (os[t] > top.least) top.add(os[t], om[t]);
+  }
+  float best = top.s[0];
+#pragma unroll
+  for (int t = 1; t < kTop; ++t) best = fmaxf(best, top.s[t]);
+  const float margin = 8.0f * static_cast<float>(n + 2) * 6.0e-8f * sum_absf * sum_absf;
+  double thrust = 1.0, ax = 0.0, ay = 0.0, az = 0.0;
+  bool decided = best >= 0.0f && top.least < best - margin;
+  if (decided) {
+    // the partitions within the error of the best, in FP64: the longest, if
+    // it is longer than the others by more than their rounding
+    double l2 = -1.0, next2 = -1.0;
+    Partition<W> won{};
+#pragma unroll 1
+    for (int t = 0; t < kTop; ++t) {
+      Partition<W> m = top.m[0];
+      float v = top.s[0];
+#pragma unroll
+      for (int u = 1; u < kTop; ++u)
+        if (t == u) {
+          m = top.m[u];
+          v = top.s[u];
+        }
+      // every lane holds the same partitions, but not in the same places:
+      // lane 0's
+      v = __shfl_sync(0xffffffffu, v, 0);
+#pragma unroll
+      for (int c = 0; c < W; ++c) m.w[c] = __shfl_sync(0xffffffffu, m.w[c], 0);
+      if (v < best - margin) continue;
+      double px = 0.0, py = 0.0, pz = 0.0;
+      for (int i = lane; i < n; i += 32) {
+        uint32_t minus = 0u;
+#pragma unroll
+        for (int c = 0; c < W; ++c) minus |= m.w[c] & bit_of(i, c);
+        const double sg = minus ? -1.0 : 1.0;
+        px = fma(sg, a.j[1][i], px);
+        py = fma(sg, a.j[2][i], py);
+        pz = fma(sg, a.j[3][i], pz);
+      }
+      px = warp_sum(px);
+      py = warp_sum(py);
+      pz = warp_sum(pz);
+      const double c2 = dot3(px, py, pz, px, py, pz);
+      if (c2 > l2) {
+        next2 = l2;
+        l2 = c2;
+        won = m;
+        ax = px;
+        ay = py;
+        az = pz;
+      } else {
+        next2 = fmax(next2, c2);
+      }
+    }
+    decided = next2 < l2 * (1.0 - 1e-12);
+    const double l = sqrt_obs(l2), inv_l = 1.0 / l;
+    thrust = l / sum_abs;
+    ax *= inv_l;
+    ay *= inv_l;
+    az *= inv_l;
+    // every parton on the side of the axis its sign says
+    for (int i = lane; i < n; i += 32) {
+      uint32_t minus = 0u;
+#pragma unroll
+      for (int c = 0; c < W; ++c) minus |= won.w[c] & bit_of(i, c);
+      const double d = dot3(a.j[1][i], a.j[2][i], a.j[3][i], ax, ay, az);
+      decided = decided && (minus ? d <= 0.0 : d >= 0.0);
+    }
+    decided = __all_sync(0xffffffffu, decided);
+  }
+  if (!decided) {
+    if (lane == 0) atomicAdd(&E.counters[4], 1ull);  // thrust decided by the exact FP64 search
+    thrust = thrust_fp64_warp<MAXJ>(n, a, sum_abs, lane, ax, ay, az);
+  }
+  // Hemispheres: heavy-jet mass and jet broadenings.
+  double hp[4] = {0, 0, 0, 0}, hm[4] = {0, 0, 0, 0};
+  double bp = 0.0, bm = 0.0;
+  for (int i = lane; i < n; i += 32) {
+    const double x = a.j[1][i], y = a.j[2][i], z = a.j[3][i];
+    const long long pn = __double_as_longlong(dot3(x, y, z, ax, ay, az));
+    const bool plus = pn >= 0 || pn == static_cast<long long>(0x8000000000000000ull);
+    const double cx = cross(y, az, z, ay), cy = cross(z, ax, x, az), cz = cross(x, ay, y, ax);
+    const double pt = sqrt_obs(dot3(cx, cy, cz, cx, cy, cz));
+    double* h = plus ? hp : hm;
+    h[0] += a.j[0][i];
+    h[1] += x;
+    h[2] += y;
+    h[3] += z;
+    if (plus) {
+      bp += pt;
+    } else {
+      bm += pt;
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    hp[c] = warp_sum(hp[c]);
+    hm[c] = warp_sum(hm[c]);
+  }
+  bp = warp_sum(bp);
+  bm = warp_sum(bm);
+  if (lane == 0) {
+    const double mp = mass2(hp), mm = mass2(hm);
+    E.obs[4 * E.stride + ev] = 1.0 - thrust;
+    E.obs[5 * E.stride + ev] = fmax(mp, mm) * P.inv_s;
+    const double inv_2sum = 0.5 / sum_abs;
+    bp *= inv_2sum;
+    bm *= inv_2sum;
+    E.obs[6 * E.stride + ev] = bp + bm;
+    E.obs[7 * E.stride + ev] = fmax(bp, bm);
+  }
+
+  // ---- Durham (E-scheme)
+  const auto direction = [&](int i) {
+    const float e = f32_from_f64(a.j[0][i]);
+    const float x = f32_from_f64(a.j[1][i]), y = f32_from_f64(a.j[2][i]), z = f32_from_f64(a.j[3][i]);
+    const float r = rsqrtf(dot3f(x, y, z, x, y, z));
+    return make_float4(x * r, y * r, z * r, e * e);
+  };
+  __syncwarp();  // every lane is done with the FP32 momenta
+  for (int i = lane; i < n; i += 32) a.f[i] = direction(i);
+  __syncwarp();
+  for (int r = lane; r < n; r += 32) {
+    Row row;
+    row.clear();
+    const float4 fr = a.f[r];
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) {
+      if (k == r) continue;
+      float u, l;
+      pair_bounds(fr, a.f[k], u, l);
+      row.add(u, l, k);
+    }
+    store_row(a, r, row);
+  }
+  // Row t anew from the jets 0 .. m - 1, by the whole warp.
+  const auto renew_row = [&](int t, int m) {
+    const float4 ft = a.f[t];
+    Row row;
+    row.clear();
+    for (int k = lane; k < m; k += 32) {
+      if (k == t) continue;
+      float u, l;
+      pair_bounds(ft, a.f[k], u, l);
+      row.add(u, l, k);
+    }
+#pragma unroll 1
+    for (int off = 1; off < 32; off <<= 1) {
+      const float ou = __shfl_xor_sync(0xffffffffu, row.ub, off), ol = __shfl_xor_sync(0xffffffffu, row.lb, off);
+      const float o2 = __shfl_xor_sync(0xffffffffu, row.lb2, off);
+      const int both = __shfl_xor_sync(0xffffffffu, row.near | (row.near2 << 8), off);
+      const int on = both & 255, on2 = both >> 8;
+      // the better nearest stays; the other's and both seconds compete
+      const bool theirs = ou < row.ub || (ou == row.ub && on < row.near);
+      float c1 = theirs ? row.lb : ol;
+      int k1 = theirs ? row.near : on;
+      if (theirs) {
+        row.ub = ou;
+        row.lb = ol;
+        row.near = on;
+      }
+      if (o2 < c1) {
+        c1 = o2;
+        k1 = on2;
+      }
+      if (c1 < row.lb2) {
+        row.lb2 = c1;
+        row.near2 = k1;
+      }
+    }
+    if (lane == 0) store_row(a, t, row);
+  };
+  double yres[4] = {-1.0, -1.0, -1.0, -1.0};
+#pragma unroll 1
+  for (int m = n; m > 2; --m) {  // y of the last two jets is not recorded
+    __syncwarp();
+    // the smallest upper bound and its pair
+    float ubest = INFINITY;
+    int br = 0;
+    for (int r = lane; r < m; r += 32)
+      if (a.ub[r] < ubest) {
+        ubest = a.ub[r];
+        br = r;
+      }
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const float ou = __shfl_xor_sync(0xffffffffu, ubest, off);
+      const int orow = __shfl_xor_sync(0xffffffffu, br, off);
+      if (ou < ubest || (ou == ubest && orow < br)) {
+        ubest = ou;
+        br = orow;
+      }
+    }
+    const int bn = a.near[br];
+    int bi = min(br, bn), bj = max(br, bn);
+    // other pairs whose lower bound reaches it; a stale bound is renewed first
+    bool other = bn >= m;  // (no finite distance at all)
+#pragma unroll 1
+    for (int r0 = 0; r0 < m; r0 += 32) {
+      const int r = r0 + lane;
+      const bool low2 = r < m && a.lb2[r] <= ubest;
+      unsigned stale = __ballot_sync(0xffffffffu, low2 && a.near2[r] == kGone);
+#pragma unroll 1
+      while (stale != 0u) {
+        renew_row(r0 + __ffs(stale) - 1, m);
+        stale &= stale - 1u;
+      }
+      __syncwarp();
+      if (r < m) other = other || a.lb2[r] <= ubest || (r != bi && r != bj && a.lb[r] <= ubest);
+    }
+    double ymin = 0.0;
+    if (!__any_sync(0xffffffffu, other)) {
+      if (m <= 6) ymin = jet_distance(a, bi, bj, P.inv_s);
+    } else {
+      if (lane == 0) atomicAdd(&E.counters[5], 1ull);  // merges with several FP64 candidates
+      int bp_ = 0x7fffffff;
+      ymin = INFINITY;
+      bi = 0;
+      bj = 1;
+      PairWalk w;
+      for (w.start(m, lane); w.valid(m); w.next<32>(m)) {
+        float u, l;
+        pair_bounds(a.f[w.j], a.f[w.k()], u, l);
+        if (l > ubest) continue;
+        const double yy = jet_distance(a, w.j, w.k(), P.inv_s);
+        if (bp_ == 0x7fffffff || yy < ymin) {
+          ymin = yy;
+          bp_ = w.p;
+          bi = w.j;
+          bj = w.k();
+        }
+      }
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const double oy = __shfl_xor_sync(0xffffffffu, ymin, off);
+        const int op = __shfl_xor_sync(0xffffffffu, bp_, off), oi = __shfl_xor_sync(0xffffffffu, bi, off);
+        const int oj = __shfl_xor_sync(0xffffffffu, bj, off);
+        // lanes without a candidate hold position 0x7fffffff
+        if (op != 0x7fffffff && (bp_ == 0x7fffffff || oy < ymin || (oy == ymin && op < bp_))) {
+          ymin = oy;
+          bp_ = op;
+          bi = oi;
+          bj = oj;
+        }
+      }
+      bi = __shfl_sync(0xffffffffu, bi, 0);  // one pair for all lanes, undefined distances included
+      bj = __shfl_sync(0xffffffffu, bj, 0);
+    }
+    if (m <= 6) yres[m - 3] = ymin;
+    // jet bi takes the sum, the last jet moves into bj
+    const int last = m - 1;
+    __syncwarp();  // every lane is done reading the jets of this merge
+    if (lane < 4) {
+      a.j[lane][bi] += a.j[lane][bj];
+      a.j[lane][bj] = a.j[lane][last];
+    }
+    __syncwarp();
+    const float4 moved = a.f[last], merged = direction(bi);
+    __syncwarp();
+    if (lane == 0) {
+      a.f[bj] = moved;  // (bj == last: beyond the jets that are left)
+      a.f[bi] = merged;
+    }
+    __syncwarp();
+    // the rows of the jets that are left: those that pointed at the merged
+    // ones are renewed, the new jet is offered to the others
+#pragma unroll 1
+    for (int r0 = 0; r0 < last; r0 += 32) {
+      const int r = r0 + lane;
+      bool renew = false;
+      if (r < last) {
+        Row row = load_row(a, r == bj ? last : r);
+        renew = r == bi || row.near == bi || row.near == bj;
+        if (!renew) {
+          if (row.near2 == bi || row.near2 == bj) row.near2 = kGone;
+          if (row.near == last) row.near = bj;
+          if (row.near2 == last) row.near2 = bj;
+          float u, l;
+          pair_bounds(a.f[r], merged, u, l);
+          row.add(u, l, bi);
+          store_row(a, r, row);
+        }
+      }
+      unsigned todo = __ballot_sync(0xffffffffu, renew);
+#pragma unroll 1
+      while (todo != 0u) {
+        renew_row(r0 + __ffs(todo) - 1, last);
+        todo &= todo - 1u;
+      }
+    }
+  }
+  if (lane == 0)
+    for (int h = 0; h < 4; ++h) E.obs[h * E.stride + ev] = yres[h];
+}
+
 // ------------------------------------------------------------- buckets
 // Parton count of event ev if it gets observables: finished, with 2 ..
 // capacity partons (the shower never writes another count; callers that pass
@@ -837,6 +1453,28 @@ __global__ void __launch_bounds__(T) k_event_shapes_group(DevParams P, Events E,
   }
 }
 
+// Events of buckets n_lo..n_hi (all with n <= MAXJ), a warp each, T threads
+// per block, the largest first; the warps of the resident blocks take them
+// one by one from *cursor (zero before the launch).
+template <int MAXJ, int T>
+__global__ void __launch_bounds__(T) k_event_shapes_warp(DevParams P, Events E, const int* order, const int* offsets,
+                                                         int n_lo, int n_hi, int* cursor) {
+  extern __shared__ __align__(16) unsigned char s_shapes[];
+  WarpEvent<MAXJ>& a = reinterpret_cast<WarpEvent<MAXJ>*>(s_shapes)[threadIdx.x >> 5];
+  const int lane = static_cast<int>(threadIdx.x & 31);
+  const int begin = offsets[n_lo], end = offsets[n_hi + 1 > 256 ? 256 : n_hi + 1];
+  if (begin == end) return;
+  for (;;) {
+    int k = 0;
+    if (lane == 0) k = atomicAdd(cursor, 1);
+    k = __shfl_sync(0xffffffffu, k, 0);
+    if (k >= end - begin) return;
+    const int64_t ev = order[end - 1 - k];
+    event_shapes_warp<MAXJ>(P, E, ev, E.n_partons[ev], a, lane);
+    __syncwarp();  // the arrays are free for the next event
+  }
+}
+
 // Events of up to 16 partons take one thread each in batches of at least
 // GAPS_SHAPES_GROUP_BELOW events (throughput), groups of
 // GAPS_SHAPES_SMALL_LANES lanes in smaller ones (a launch then waits for its
@@ -869,10 +1507,8 @@ cudaError_t preload_observables() {
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_bucket_scatter);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes<16>);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_group<16, kSmallLanes, 128>);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_group<32, 32, 128>);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_group<64, 32, 128>);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_group<128, 32, 128>);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_group<256, 32, 64>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_warp<128, 128>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_warp<256, 64>);
   return e;
 }
 
@@ -906,10 +1542,15 @@ cudaError_t launch_observables(const DevParams& P, const Events& E, int* buckets
   } else {
     k_event_shapes<16><<<grid(kShapeThreads, GAPS_SHAPES_BLOCKS_PER_SM), kShapeThreads, 0, s>>>(P, E, order, offsets, 0, 16);
   }
-  if (E.cap > 16) k_event_shapes_group<32, 32, 128><<<grid(4, 2), 128, 0, s>>>(P, E, order, offsets, 17, 32);
-  if (E.cap > 32) k_event_shapes_group<64, 32, 128><<<grid(4, 2), 128, 0, s>>>(P, E, order, offsets, 33, 64);
-  if (E.cap > 64) k_event_shapes_group<128, 32, 128><<<grid(4, 2), 128, 0, s>>>(P, E, order, offsets, 65, 128);
-  if (E.cap > 128) k_event_shapes_group<256, 32, 64><<<grid(2, 2), 64, 0, s>>>(P, E, order, offsets, 129, 255);
+  // One class up to 128 partons (96 registers leave five blocks per SM), one
+  // beyond.  Their cursors are the bucket cursors of 0 and 1 partons, which no
+  // event has: zero.
+  if (E.cap > 16)
+    k_event_shapes_warp<128, 128>
+        <<<grid(4, 5), 128, 4 * sizeof(WarpEvent<128>), s>>>(P, E, order, offsets, 17, 128, cursor);
+  if (E.cap > 128)
+    k_event_shapes_warp<256, 64>
+        <<<grid(2, 6), 64, 2 * sizeof(WarpEvent<256>), s>>>(P, E, order, offsets, 129, 255, cursor + 1);
   return cudaGetLastError();
 }
 
