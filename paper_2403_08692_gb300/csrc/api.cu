@@ -404,6 +404,9 @@ HostCounters& host_counters() {
 
 // The plain form rebuilds its active list in event order after a launch
 // while the list holds at least 1/GAPS_REBUILD_DIV of the batch.
+#ifndef GAPS_REBUILD_MIN
+#define GAPS_REBUILD_MIN 50000
+#endif
 #ifndef GAPS_REBUILD_DIV
 #define GAPS_REBUILD_DIV 16
 #endif
@@ -515,7 +518,7 @@ int shower_impl(const gaps_params* params, const gaps_batch* batch, int mode, in
     if (kernel_ms_out && (err = cudaEventRecord(tev[2 * c + 1], s)) != cudaSuccess) return err;
     // While the list is long, put it back in event order (appends scatter
     // it); the same events, so its length stands.
-    if (bound * GAPS_REBUILD_DIV >= E.n &&
+    if (E.n >= GAPS_REBUILD_MIN && bound * GAPS_REBUILD_DIV >= E.n &&
         (err = launch_list_active(E, list_out, &E.counters[kListScratchWord], s)) != cudaSuccess)
       return err;
     return cudaSuccess;

@@ -79,6 +79,9 @@ __global__ void __launch_bounds__(256) k_me(DevParams P0, Events E) {
 #ifndef GAPS_EMIT_WARPS_PER_SM
 #define GAPS_EMIT_WARPS_PER_SM 4
 #endif
+#ifndef GAPS_EMIT_CHUNK
+#define GAPS_EMIT_CHUNK 8
+#endif
 constexpr int kStepThreads = GAPS_STEP_THREADS;
 
 
@@ -312,17 +315,21 @@ __global__ void __launch_bounds__(kStepThreads, GAPS_STEP_MIN_BLOCKS)
     return;
   }
   const int64_t len = n_tasks_dev ? min(n_tasks, static_cast<int64_t>(*n_tasks_dev)) : n_tasks;
+  // Tasks a block takes at a time: an even share of a short list, so that the
+  // dipoles they moved fit one round of the block.
+  const int chunk = static_cast<int>(
+      min(static_cast<int64_t>(kStepThreads), max((len + emit_blocks - 1) / emit_blocks, static_cast<int64_t>(GAPS_EMIT_CHUNK))));
   for (;;) {
     __syncthreads();  // the previous round is done with s_task, s_jobs and s_base
     if (tid == 0) {
       s_njobs = 0;
-      s_base = atomicAdd(emit_cursor, static_cast<unsigned long long>(kStepThreads));
+      s_base = atomicAdd(emit_cursor, static_cast<unsigned long long>(chunk));
     }
     __syncthreads();
     const int64_t base = static_cast<int64_t>(s_base);
     if (base >= len) break;
     const int64_t k = base + tid;
-    const bool has = k < len;
+    const bool has = tid < chunk && k < len;
     if (has) s_task[tid] = tasks_in[k];
     __syncthreads();
     if (has)
@@ -460,7 +467,7 @@ cudaError_t launch_step_deferred(const DevParams& P, const Events& E, const int*
   const int lanes = lanes_for(n_list, resident);
   const int64_t select_blocks = (n_list * lanes + kStepThreads - 1) / kStepThreads;
   const int64_t emit_per_sm = std::max(1, 32 * GAPS_EMIT_WARPS_PER_SM / kStepThreads);
-  const int64_t emit_blocks = std::min((n_tasks + kStepThreads - 1) / kStepThreads, resident / 1024 * emit_per_sm);
+  const int64_t emit_blocks = std::min((n_tasks + GAPS_EMIT_CHUNK - 1) / GAPS_EMIT_CHUNK, resident / 1024 * emit_per_sm);
   if (select_blocks + emit_blocks == 0) return cudaSuccess;
   const unsigned grid = static_cast<unsigned>(select_blocks + emit_blocks);
 #define GAPS_DEFERRED_CASE(MULTI, LN)                                                                     \
