@@ -51,171 +51,122 @@ namespace {
 // Events of a warp's pool: 32 can run while 32 wait for their emission, so
 // both the cycles and the emissions fill the warp.
 constexpr int kSlots = 64;
-// Dipoles with phase space kept per event in shared memory; an event with
-// more takes its screen's inputs from the record.  Six hold nearly every LEP
-// event; 8 or 4 were 5 and 14 % slower at 10^6 events (less first-level cache,
-// more events in the record).
-constexpr int kDips = 6;
-constexpr uint8_t kInRecord = 255;
 // The register budget is set for 16 warps per SM.
 constexpr int kMaxThreads = 512;
 // Veto cycles a warp runs between two votes of its block (1 to 8 were alike).
 constexpr int kTurns = 3;
 
-// Slot states of a pool: empty, live, live with an emission waiting, live
-// with its screen's dipoles to be loaded, and four ways to leave: at the
-// cutoff, with a full record, at the cycle limit, or at the end of a slice.
-// A slot that has left is written back and refilled together with others.
-enum : uint8_t {
-  kSlotEmpty = 0,
-  kSlotLive = 1,
-  kSlotPending = 2,
-  kSlotLoad = 3,
-  kSlotDone = 4,  // and above: the event has left
-  kSlotOverflow = 5,
-  kSlotLimit = 6,
-  kSlotSliced = 7
-};
+// Dipoles with phase space kept per event in shared memory; an event with
+// more takes its screen's inputs from the record.  Six hold nearly every LEP
+// event; 8 or 4 were 5 and 14 % slower for the persistent form at 10^6 events
+// (less first-level cache, more events in the record).
+constexpr int kDips = 6;
+constexpr uint8_t kInRecord = 255;
 
-struct WarpPool {
-  double lnt[kSlots];
-  unsigned long long hash[kSlots];
-  float dip_x[kDips][kSlots], dip_y[kDips][kSlots];  // the screen's dipoles
-  uint32_t dip_m[kDips][kSlots];                     // slot on side 0 | slot on side 1 << 8 | gluons << 16, 17
+// What the screens of a warp read of its events, S slots.
+template <int S>
+struct ScreenPool {
+  float dip_x[kDips][S], dip_y[kDips][S];  // the dipoles' screen entries
+  uint32_t dip_m[kDips][S];                // slot on side 0 | slot on side 1 << 8 | gluons << 16, 17
+  int32_t ev[S];
   // the event's splitters, dipole * 2 + side: those with a gluon's kernels
-  // from the front, those with one trial from the back
-  uint8_t split[2 * kDips][kSlots];
-  uint32_t rz_hi[kSlots], rz_lo[kSlots], won[kSlots];  // the waiting emission
-  int32_t ev[kSlots], step[kSlots];
-  int32_t first_step[kSlots];    // cycle the event came in at
-  int32_t settled_step[kSlots];  // cycle up to which its work counts are in the record
-  uint16_t trials[kSlots], dipoles[kSlots];  // per cycle, until its next emission
-  uint16_t job[kSlots];
-  uint8_t n[kSlots], state[kSlots], cyc[kSlots];
-  uint8_t n_all[kSlots], n_one[kSlots];  // splitters of either kind (n_all = kInRecord: in the record)
-  uint8_t list[kSlots], owner[64];
-  union {
-    struct {  // the screens' results, per lane
-      uint32_t best[32], second[32], code[32], hi[32], lo[32];
-      float invc[32];
-    } r;
-    // a warp's share of the block's lists of an emission turn: the waiting
-    // events (warp * 64 + slot), the dipoles their emissions move, and those
-    // of them with phase space
-    struct {
-      double q2[kMaxRefresh * 32];
-      uint32_t jobs[kMaxRefresh * 32], kept[kMaxRefresh * 32];
-      uint16_t tasks[32];
-    } m;
-  };
+  // from the front, those with one trial from the back; how many of either
+  // kind (n_all = kInRecord: in the record)
+  uint8_t split[2 * kDips][S];
+  uint8_t n_all[S], n_one[S], n[S];
+  uint8_t owner[64];
 };
-
-// What the warps of a block agree on.
-struct BlockShared {
-  uint32_t vote[2][kMaxThreads / 32];  // running | waiting << 16 of every warp, in turn
-  int n_jobs, n_kept;
-  double pad;  // the pools behind it stay aligned
+// The screens' results, per lane.
+struct ScreenResults {
+  uint32_t best[32], second[32], code[32], hi[32], lo[32];
+  float invc[32];
 };
-
-static_assert(sizeof(BlockShared) + sizeof(WarpPool) * (kMaxThreads / 32) <= 227 * 1024, "16 warps' pools fit an SM");
-
-// Where a launch takes its events from and how far it runs them.  Whole
-// batch (kSlice false): events 0 .. E.n - 1 to the cutoff, cursor in counter
-// word 6.  Slice (kSlice true): the events of list_in (length *n_in_dev, at
-// most n_in), each for at most `cycles` veto cycles; those still active then
-// go to list_out (one atomic per warp).
-struct SliceArgs {
-  const int* list_in;
-  const unsigned long long* n_in_dev;
-  int64_t n_in;
-  unsigned long long* cursor;
-  int cycles;
-  int* list_out;
-  unsigned long long* out_count;
-};
-
 __device__ __forceinline__ unsigned lanes_below(int lane) { return (1u << lane) - 1u; }
 
-// The screen's dipoles of slot q's event, from its record: those with phase
-// space, each once (from its colour end), and the trials and dipoles a cycle
-// counts for them.
-template <int kMode>
-__device__ __forceinline__ void load_dipoles(const DevParams& P, const Events& E, WarpPool& w, int q) {
-  const int64_t ev = w.ev[q];
-  const int n = w.n[q];
-  const int per_gluon = per_dipole<kMode>(P) ? 1 : 1 + P.nf;
-  int nd = 0, trials = 0, all = 0, one = 0;
+// Lanes of a warp per event for up to 32 events: a power of two.
+__device__ __forceinline__ int lanes_each(int events) { return 1 << min(max(__clz(events - 1) - 27, 0), 5); }
+
+// Splitters (sides of dipoles with phase space) of an event, and those of
+// them that are gluons.
+struct SideCounts {
+  int all, gluons;
+};
+
+// Load the screen's dipoles of the events in slots q of the warp's first 32 /
+// L lanes (q < 0: none), L lanes per event: those with phase space, each once
+// (from its colour end).  Returns each such lane its event's counts.  The
+// partons' data are loaded side by side over the lanes, so a few events take
+// one or two memory latencies whatever their size.  Every lane of the warp
+// must call it.
+template <int kMode, int S>
+__device__ __forceinline__ SideCounts load_dipoles(const DevParams& P0, const Events& E, ScreenPool<S>& w, int q, int job,
+                                                   int L) {
+  const int lane = static_cast<int>(threadIdx.x & 31);
+  const int el = lane / L, sub = lane - el * L;
+  const unsigned group = (L == 32 ? 0xffffffffu : (1u << L) - 1u) << (el * L);
+  const unsigned before = group & lanes_below(lane);
+  const int eq = __shfl_sync(0xffffffffu, q, el);
+  const bool combined = per_dipole<kMode>(job_params<kJobPhysics<kMode>>(P0, E, __shfl_sync(0xffffffffu, job, el)));
+  const int64_t ev = eq >= 0 ? w.ev[eq] : 0;
+  const int n = eq >= 0 ? w.n[eq] : 0;
+  const int rounds = (__reduce_max_sync(0xffffffffu, n) + L - 1) / L;
+  int nd = 0, all = 0, one = 0;
+  SideCounts mine{0, 0};
   // the next parton's loads are in flight while this one is taken in
-  int k = E.link[E.link_at(0, 0, ev)];
-  float2 d = E.dip[dip_at(E, 0, 0, ev)];
-  bool gi = E.flav[E.at(0, ev)] == kGluon;
+  int k = kNoLink;
+  float2 d = make_float2(-1.0f, -1.0f);
+  bool gi = false;
+  if (sub < n) {
+    k = E.link[E.link_at(0, sub, ev)];
+    d = E.dip[dip_at(E, 0, sub, ev)];
+    gi = E.flav[E.at(sub, ev)] == kGluon;
+  }
 #pragma unroll 1
-  for (int i = 0; i < n; ++i) {
+  for (int t = 0; t < rounds; ++t) {
+    const int i = t * L + sub, next = i + L;
     const int ck = k;
     const float2 cd = d;
     const bool cg = gi;
-    if (i + 1 < n) {
-      k = E.link[E.link_at(0, i + 1, ev)];
-      d = E.dip[dip_at(E, 0, i + 1, ev)];
-      gi = E.flav[E.at(i + 1, ev)] == kGluon;
+    const bool has = i < n && ck != kNoLink && cd.x >= 0.0f;
+    // the partner's flavour: from its lane where it was loaded with this one
+    const unsigned gluons = __ballot_sync(0xffffffffu, i < n && cg) >> (el * L);
+    const bool here = ck >= t * L && ck < (t + 1) * L;
+    const bool gk = has && (here ? (gluons >> (ck - t * L) & 1u) != 0u : E.flav[E.at(ck, ev)] == kGluon);
+    if (next < n) {
+      k = E.link[E.link_at(0, next, ev)];
+      d = E.dip[dip_at(E, 0, next, ev)];
+      gi = E.flav[E.at(next, ev)] == kGluon;
     }
-    if (ck == kNoLink || cd.x < 0.0f) continue;
-    const bool gk = E.flav[E.at(ck, ev)] == kGluon;
-    trials += (cg ? per_gluon : 1) + (gk ? per_gluon : 1);
-    if (nd < kDips) {
-      w.dip_x[nd][q] = cd.x;
-      w.dip_y[nd][q] = cd.y;
-      w.dip_m[nd][q] = static_cast<uint32_t>(i) | (static_cast<uint32_t>(ck) << 8) | (cg ? 1u << 16 : 0u) |
-                       (gk ? 1u << 17 : 0u);
-      const int a0 = cg && per_gluon > 1 ? all++ : 2 * kDips - 1 - one++;
-      w.split[a0][q] = static_cast<uint8_t>(2 * nd);
-      const int a1 = gk && per_gluon > 1 ? all++ : 2 * kDips - 1 - one++;
-      w.split[a1][q] = static_cast<uint8_t>(2 * nd + 1);
+    const unsigned hm = __ballot_sync(0xffffffffu, has);
+    const unsigned g0 = __ballot_sync(0xffffffffu, has && cg), g1 = __ballot_sync(0xffffffffu, has && gk);
+    if (has) {
+      const int at = nd + __popc(hm & before);
+      if (at < kDips) {
+        w.dip_x[at][eq] = cd.x;
+        w.dip_y[at][eq] = cd.y;
+        w.dip_m[at][eq] = static_cast<uint32_t>(i) | (static_cast<uint32_t>(ck) << 8) | (cg ? 1u << 16 : 0u) |
+                          (gk ? 1u << 17 : 0u);
+        const int sides = 2 * __popc(hm & before), gs = __popc(g0 & before) + __popc(g1 & before);
+        int front = all + (combined ? 0 : gs), back = one + sides - (combined ? 0 : gs);
+        w.split[cg && !combined ? front++ : 2 * kDips - 1 - back++][eq] = static_cast<uint8_t>(2 * at);
+        w.split[gk && !combined ? front : 2 * kDips - 1 - back][eq] = static_cast<uint8_t>(2 * at + 1);
+      }
     }
-    ++nd;
+    const int sides = 2 * __popc(hm & group), gs = __popc(g0 & group) + __popc(g1 & group);
+    nd += sides / 2;
+    all += combined ? 0 : gs;
+    one += sides - (combined ? 0 : gs);
+    mine.all += sides;
+    mine.gluons += gs;
   }
-  w.trials[q] = static_cast<uint16_t>(trials);
-  w.dipoles[q] = static_cast<uint16_t>(2 * nd);
-  w.n_all[q] = nd <= kDips ? static_cast<uint8_t>(all) : kInRecord;
-  w.n_one[q] = nd <= kDips ? static_cast<uint8_t>(one) : static_cast<uint8_t>(0);
-}
-
-// Whether a block (or a warp, at its share) should generate its waiting
-// emissions: half of its live events wait, so that the others still fill the
-// warps, or flush_at per warp do (a third or a quarter of them was 6 and 13 %
-// slower at 10^6 events, two thirds 1 %).
-__device__ __forceinline__ bool emission_due(int running, int waiting, int flush_at) {
-  return waiting > 0 && (running == 0 || waiting >= flush_at || 2 * waiting >= running + waiting);
-}
-
-// Add the work counts of slot q's cycles since its last emission to the
-// record.
-__device__ __forceinline__ void settle_counts(const Events& E, WarpPool& w, int q) {
-  const int cycles = w.step[q] - w.settled_step[q];
-  const int ev = w.ev[q];
-  atomicAdd(&E.n_trials[ev], cycles * static_cast<int>(w.trials[q]));
-  atomicAdd(&E.n_dipoles[ev], cycles * static_cast<int>(w.dipoles[q]));
-  w.settled_step[q] = w.step[q];
-}
-
-// The event of slot q, which left with `state`, back to the record: its
-// scalars, and its status and final scale unless its slice ended.
-template <int kMode>
-__device__ __forceinline__ void write_back(const DevParams& P0, const Events& E, WarpPool& w, int q, int state) {
-  settle_counts(E, w, q);
-  const int ev = w.ev[q];
-  const double lnt = w.lnt[q];
-  E.lnt[ev] = lnt;
-  E.hash[ev] = w.hash[q];
-  E.n_steps[ev] = w.step[q];
-  // every cycle of the stay had a winner but the one that found the cutoff
-  atomicAdd(&E.n_winners[ev], w.step[q] - w.first_step[q] - (state == kSlotDone ? 1 : 0));
-  if (state == kSlotDone) {
-    finish_event(E, ev, GAPS_DONE, job_params<kJobPhysics<kMode>>(P0, E, w.job[q]).tc);
-  } else if (state != kSlotSliced) {
-    finish_early(E, ev, state == kSlotLimit ? GAPS_STEP_LIMIT : GAPS_OVERFLOW, lnt);
-    if (state == kSlotLimit) atomicAdd(&E.counters[1], 1ull);
+  if (sub == 0 && eq >= 0) {
+    w.n_all[eq] = nd <= kDips ? static_cast<uint8_t>(all) : kInRecord;
+    w.n_one[eq] = nd <= kDips ? static_cast<uint8_t>(one) : static_cast<uint8_t>(0);
   }
+  const int from = lane * L & 31;
+  mine.all = __shfl_sync(0xffffffffu, mine.all, from);
+  mine.gluons = __shfl_sync(0xffffffffu, mine.gluons, from);
+  return mine;
 }
 
 // The |key| bound of a trial, h = |key| - m >= 0 with key = log2(u)/c <= 0
@@ -237,15 +188,15 @@ __device__ __forceinline__ float trial_bound(uint32_t hi, uint32_t lo, float inv
 // is not the smallest is displaced or loses exactly once, whatever the order.
 // Equal bounds leave the cycle undecided, so which of them is kept is
 // immaterial.
-template <int kMode>
-__device__ __forceinline__ void screen_warp(const DevParams& P0, const DevParams& P, const Events& E, WarpPool& w, int q,
+template <int kMode, int S>
+__device__ __forceinline__ void screen_warp(const DevParams& P0, const DevParams& P, const Events& E, ScreenPool<S>& w, ScreenResults& r, int q,
                                             const EventKey& key, int step) {
   constexpr float kInvCF2 = static_cast<float>(1.0 / (2.0 * kCF));
   constexpr float kInvCA = static_cast<float>(1.0 / kCA);
   constexpr uint32_t kInf = 0x7f800000u;
   const int lane = static_cast<int>(threadIdx.x & 31);
   const unsigned below = lanes_below(lane);
-  w.r.best[lane] = w.r.second[lane] = kInf;
+  r.best[lane] = r.second[lane] = kInf;
   const int n_all = q >= 0 ? w.n_all[q] : 0;
   const bool in_record = n_all == kInRecord;
   const uint32_t mine =
@@ -363,11 +314,11 @@ __device__ __forceinline__ void screen_warp(const DevParams& P0, const DevParams
           h1 = fminf(h1, h[c]);
         }
       }
-      const uint32_t old = atomicMin(&w.r.best[el], __float_as_uint(h1));
-      atomicMin(&w.r.second[el], min(max(old, __float_as_uint(h1)), __float_as_uint(h2)));
+      const uint32_t old = atomicMin(&r.best[el], __float_as_uint(h1));
+      atomicMin(&r.second[el], min(max(old, __float_as_uint(h1)), __float_as_uint(h2)));
     }
     __syncwarp();
-    if (has && w.r.best[el] == __float_as_uint(h1)) {
+    if (has && r.best[el] == __float_as_uint(h1)) {
       // this splitter's best trial is its event's best so far: its kernel,
       // random words and 1/c
       uint32_t hi = r0.x, lo = r0.y, kappa = 0u;
@@ -375,17 +326,132 @@ __device__ __forceinline__ void screen_warp(const DevParams& P0, const DevParams
         invc = y;
         kappa = h1 == h[1] ? 1u : (h1 == h[2] ? 2u : (h1 == h[3] ? 3u : (h1 == h[4] ? 4u : 5u)));
         const bool odd = (kappa & 1u) != 0u;
-        const U4 r = kappa == 1u ? r0 : (kappa < 4u ? r1 : r2);
-        hi = odd ? r.z : r.x;
-        lo = odd ? r.w : r.y;
+        const U4 words = kappa == 1u ? r0 : (kappa < 4u ? r1 : r2);
+        hi = odd ? words.z : words.x;
+        lo = odd ? words.w : words.y;
       }
-      w.r.code[el] = (static_cast<uint32_t>(2 * i + side) << 3) | kappa | (static_cast<uint32_t>(k) << 16) |
+      r.code[el] = (static_cast<uint32_t>(2 * i + side) << 3) | kappa | (static_cast<uint32_t>(k) << 16) |
                      (gluon ? 1u << 24 : 0u);
-      w.r.hi[el] = hi;
-      w.r.lo[el] = lo;
-      w.r.invc[el] = invc;
+      r.hi[el] = hi;
+      r.lo[el] = lo;
+      r.invc[el] = invc;
     }
     __syncwarp();
+  }
+}
+
+// The verdict of the calling lane's screen, from screen_warp's results: its
+// best trial's bounds are |key| - m = h1 and, from it, |key| + m.
+template <int kMode>
+__device__ __forceinline__ int screen_verdict(const DevParams& P, const Events& E, int64_t ev, double lnt,
+                                              const ScreenResults& r, EmitTask& task) {
+  const int lane = static_cast<int>(threadIdx.x & 31);
+  const uint32_t best = r.best[lane], code = r.code[lane];
+  const float h1 = __uint_as_float(best), invc = r.invc[lane];
+  const float most = fmaf(2.0f * kKeyRelInvc, invc, h1) * (1.0f + 2.1f * kKeyRelKey);
+  return screen_verdict<kMode>(P, E, ev, lnt, -h1, -most, -__uint_as_float(r.second[lane]),
+                               best == 0x7f800000u ? -1 : static_cast<int>(code & 4095u), code >> 16, r.hi[lane],
+                               r.lo[lane], task);
+}
+
+// Slot states of a pool: empty, live, live with an emission waiting, live
+// with its screen's dipoles to be loaded, and four ways to leave: at the
+// cutoff, with a full record, at the cycle limit, or at the end of a slice.
+// A slot that has left is written back and refilled together with others.
+enum : uint8_t {
+  kSlotEmpty = 0,
+  kSlotLive = 1,
+  kSlotPending = 2,
+  kSlotLoad = 3,
+  kSlotDone = 4,  // and above: the event has left
+  kSlotOverflow = 5,
+  kSlotLimit = 6,
+  kSlotSliced = 7
+};
+
+struct WarpPool {
+  double lnt[kSlots];
+  unsigned long long hash[kSlots];
+  ScreenPool<kSlots> sc;
+  uint32_t rz_hi[kSlots], rz_lo[kSlots], won[kSlots];  // the waiting emission
+  int32_t step[kSlots];
+  int32_t first_step[kSlots];    // cycle the event came in at
+  int32_t settled_step[kSlots];  // cycle up to which its work counts are in the record
+  uint16_t trials[kSlots], dipoles[kSlots];  // per cycle, until its next emission
+  uint16_t job[kSlots];
+  uint8_t state[kSlots], cyc[kSlots], list[kSlots];
+  union {
+    ScreenResults r;
+    // a warp's share of the block's lists of an emission turn: the waiting
+    // events (warp * 64 + slot), the dipoles their emissions move, and those
+    // of them with phase space
+    struct {
+      double q2[kMaxRefresh * 32];
+      uint32_t jobs[kMaxRefresh * 32], kept[kMaxRefresh * 32];
+      uint16_t tasks[32];
+    } m;
+  };
+};
+
+// What the warps of a block agree on.
+struct BlockShared {
+  uint32_t vote[2][kMaxThreads / 32];  // running | waiting << 16 of every warp, in turn
+  int n_jobs, n_kept;
+  double pad;  // the pools behind it stay aligned
+};
+
+static_assert(sizeof(BlockShared) + sizeof(WarpPool) * (kMaxThreads / 32) <= 227 * 1024, "16 warps' pools fit an SM");
+
+// Where a launch takes its events from and how far it runs them.  Whole
+// batch (kSlice false): events 0 .. E.n - 1 to the cutoff, cursor in counter
+// word 6.  Slice (kSlice true): the events of list_in (length *n_in_dev, at
+// most n_in), each for at most `cycles` veto cycles; those still active then
+// go to list_out (one atomic per warp).
+struct SliceArgs {
+  const int* list_in;
+  const unsigned long long* n_in_dev;
+  int64_t n_in;
+  unsigned long long* cursor;
+  int cycles;
+  int* list_out;
+  unsigned long long* out_count;
+};
+
+// Whether a block (or a warp, at its share) should generate its waiting
+// emissions: half of its live events wait, so that the others still fill the
+// warps, or flush_at per warp do (a third or a quarter of them was 6 and 13 %
+// slower at 10^6 events, two thirds 1 %).
+__device__ __forceinline__ bool emission_due(int running, int waiting, int flush_at) {
+  return waiting > 0 && (running == 0 || waiting >= flush_at || 2 * waiting >= running + waiting);
+}
+
+// Add the work counts of slot q's cycles since its last emission to the
+// record.
+__device__ __forceinline__ void settle_counts(const Events& E, WarpPool& w, int q) {
+  const int cycles = w.step[q] - w.settled_step[q];
+  const int ev = w.sc.ev[q];
+  atomicAdd(&E.n_trials[ev], cycles * static_cast<int>(w.trials[q]));
+  atomicAdd(&E.n_dipoles[ev], cycles * static_cast<int>(w.dipoles[q]));
+  w.settled_step[q] = w.step[q];
+}
+
+// The event of slot q, which left with `state`, back to the record: its
+// scalars, and its status and final scale unless its slice ended.
+template <int kMode>
+__device__ __forceinline__ void write_back(const DevParams& P0, const Events& E, WarpPool& w, int q, int state) {
+  settle_counts(E, w, q);
+  const int ev = w.sc.ev[q];
+  const double lnt = w.lnt[q];
+  E.lnt[ev] = lnt;
+  E.hash[ev] = w.hash[q];
+  E.n_steps[ev] = w.step[q];
+  // every cycle of the stay had a winner but the one that found the cutoff
+  atomicAdd(&E.n_winners[ev], w.step[q] - w.first_step[q] - (state == kSlotDone ? 1 : 0));
+  if (state == kSlotDone) {
+    finish_event(E, ev, GAPS_DONE, job_params<kJobPhysics<kMode>>(P0, E, w.job[q]).tc);
+  } else if (state != kSlotSliced) {
+    finish_early(E, ev, state == kSlotLimit ? GAPS_STEP_LIMIT : GAPS_OVERFLOW, lnt);
+    if (state == kSlotLimit) atomicAdd(&E.counters[1], 1ull);
   }
 }
 
@@ -445,7 +511,7 @@ __global__ void __launch_bounds__(kMaxThreads)
         if (out) write_back<kMode>(P0, E, w, q, state);
         const unsigned dm = __ballot_sync(0xffffffffu, done);
         if (dm != 0u && lane == 0) atomicAdd(&E.counters[0], static_cast<unsigned long long>(__popc(dm)));
-        count_job_done(E, out ? w.ev[q] : 0, done);
+        count_job_done(E, out ? w.sc.ev[q] : 0, done);
         if constexpr (kSlice) {
           const bool sliced = state == kSlotSliced;
           const unsigned sm = __ballot_sync(0xffffffffu, sliced);
@@ -453,7 +519,7 @@ __global__ void __launch_bounds__(kMaxThreads)
             unsigned long long at = 0;
             if (lane == 0) at = atomicAdd(sl.out_count, static_cast<unsigned long long>(__popc(sm)));
             at = __shfl_sync(0xffffffffu, at, 0);
-            if (sliced) sl.list_out[at + __popc(sm & below)] = w.ev[q];
+            if (sliced) sl.list_out[at + __popc(sm & below)] = w.sc.ev[q];
           }
         }
         const bool open = out || state == kSlotEmpty;
@@ -463,9 +529,9 @@ __global__ void __launch_bounds__(kMaxThreads)
         if (open && r < take) {
           const int64_t at = static_cast<int64_t>(base) + r;
           const int ev = kSlice && sl.list_in ? sl.list_in[at] : static_cast<int>(at);
-          w.ev[q] = ev;
+          w.sc.ev[q] = ev;
           w.job[q] = kJobKey<kMode> ? E.job_of[ev] : static_cast<uint16_t>(0);
-          w.n[q] = static_cast<uint8_t>(E.n_partons[ev]);
+          w.sc.n[q] = static_cast<uint8_t>(E.n_partons[ev]);
           w.step[q] = w.first_step[q] = w.settled_step[q] = E.n_steps[ev];
           w.lnt[q] = E.lnt[ev];
           w.hash[q] = E.hash[ev];
@@ -511,7 +577,7 @@ __global__ void __launch_bounds__(kMaxThreads)
         const int task = w.m.tasks[lane], q = task & (kSlots - 1);
         WarpPool& o = pools[task >> 6];
         const uint32_t won = o.won[q];
-        const int64_t ev = o.ev[q];
+        const int64_t ev = o.sc.ev[q];
         EmitTask t;
         t.ev = static_cast<int32_t>(ev);
         t.i = static_cast<uint8_t>(won & 255u);
@@ -519,7 +585,7 @@ __global__ void __launch_bounds__(kMaxThreads)
         t.side = static_cast<uint8_t>((won >> 16) & 15u);
         t.kappa = static_cast<uint8_t>((won >> 20) & 15u);
         t.kind = static_cast<uint8_t>(won >> 24);
-        t.n = o.n[q];
+        t.n = o.sc.n[q];
         t.step = o.step[q] - 1;
         t.lnt = o.lnt[q];
         t.rz_hi = o.rz_hi[q];
@@ -531,7 +597,7 @@ __global__ void __launch_bounds__(kMaxThreads)
         settle_counts(E, o, q);
         cycle_emit<kMode>(P0, E, t, [&](int count) { return atomicAdd(&blk.n_jobs, count); },
                           [&](int at, uint32_t job) { pools[at >> 7].m.jobs[at & 127] = job; }, tid);
-        o.n[q] = static_cast<uint8_t>(t.n + 1);
+        o.sc.n[q] = static_cast<uint8_t>(t.n + 1);
         bool over = false;
         if constexpr (kSlice) over = o.cyc[q] >= sl.cycles;
         o.state[q] = over ? kSlotSliced : kSlotLoad;
@@ -548,7 +614,7 @@ __global__ void __launch_bounds__(kMaxThreads)
           job = pools[j >> 7].m.jobs[j & 127];
           const int task = pools[refresh_task(job) >> 5].m.tasks[refresh_task(job) & 31];
           const WarpPool& o = pools[task >> 6];
-          const int64_t ev = o.ev[task & (kSlots - 1)];
+          const int64_t ev = o.sc.ev[task & (kSlots - 1)];
           q2 = refresh_mass(E, ev, job);
           keep = has_phase_space(job_params<kJobPhysics<kMode>>(P0, E, o.job[task & (kSlots - 1)]), q2);
           if (!keep) refresh_store(E, ev, job, no_dipole(q2));
@@ -569,7 +635,7 @@ __global__ void __launch_bounds__(kMaxThreads)
         const uint32_t job = pools[j >> 7].m.kept[j & 127];
         const int task = pools[refresh_task(job) >> 5].m.tasks[refresh_task(job) & 31];
         const WarpPool& o = pools[task >> 6];
-        refresh_store(E, o.ev[task & (kSlots - 1)], job,
+        refresh_store(E, o.sc.ev[task & (kSlots - 1)], job,
                       make_dipole(job_params<kJobPhysics<kMode>>(P0, E, o.job[task & (kSlots - 1)]),
                                   pools[j >> 7].m.q2[j & 127]));
       }
@@ -586,10 +652,16 @@ __global__ void __launch_bounds__(kMaxThreads)
       __syncwarp();
       const int count = __popc(l0) + __popc(l1);
 #pragma unroll 1
-      for (int k = lane; k < count; k += 32) {
-        const int q = w.list[k];
-        load_dipoles<kMode>(job_params<kJobPhysics<kMode>>(P0, E, w.job[q]), E, w, q);
-        w.state[q] = kSlotLive;
+      for (int k0 = 0; k0 < count; k0 += 32) {
+        const int q = k0 + lane < count ? w.list[k0 + lane] : -1;
+        const SideCounts sides =
+            load_dipoles<kMode>(P0, E, w.sc, q, q >= 0 ? w.job[q] : 0, lanes_each(min(count - k0, 32)));
+        if (q >= 0) {
+          const DevParams& P = job_params<kJobPhysics<kMode>>(P0, E, w.job[q]);
+          w.trials[q] = static_cast<uint16_t>(sides.all + sides.gluons * (per_dipole<kMode>(P) ? 0 : P.nf));
+          w.dipoles[q] = static_cast<uint16_t>(sides.all);
+          w.state[q] = kSlotLive;
+        }
       }
       __syncwarp();
     }
@@ -609,32 +681,26 @@ __global__ void __launch_bounds__(kMaxThreads)
       if (s1 == kSlotLive) w.list[__popc(run1 & below) + (swap ? 0 : __popc(run0))] = static_cast<uint8_t>(lane + 32);
       __syncwarp();
       const int q = lane < running ? w.list[lane] : -1;
-      const int64_t ev = q >= 0 ? w.ev[q] : -1;
+      const int64_t ev = q >= 0 ? w.sc.ev[q] : -1;
       const int job = q >= 0 ? w.job[q] : 0;
       const DevParams& P = job_params<kJobPhysics<kMode>>(P0, E, job);
       const int step = q >= 0 ? w.step[q] : 0;
       const bool limited = q >= 0 && step >= P.max_steps;
       EventKey key{0u, 0u, 0u};
       if (q >= 0) key = event_key<kMode>(P, E, ev, job);
-      screen_warp<kMode>(P0, P, E, w, limited ? -1 : q, key, step);
+      screen_warp<kMode>(P0, P, E, w.sc, w.r, limited ? -1 : q, key, step);
       const bool lead = q >= 0 && !limited;
       int verdict = kScreenNone;
       double lnt = 0.0;
       EmitTask task;
       if (lead) {
-        // the best trial's bounds: |key| - m = h1 and, from it, |key| + m
-        const uint32_t best = w.r.best[lane], code = w.r.code[lane];
-        const float h1 = __uint_as_float(best), invc = w.r.invc[lane];
-        const float most = fmaf(2.0f * kKeyRelInvc, invc, h1) * (1.0f + 2.1f * kKeyRelKey);
         lnt = w.lnt[q];
-        verdict = screen_verdict<kMode>(P, E, ev, lnt, -h1, -most, -__uint_as_float(w.r.second[lane]),
-                                        best == 0x7f800000u ? -1 : static_cast<int>(code & 4095u), code >> 16, w.r.hi[lane],
-                                        w.r.lo[lane], task);
+        verdict = screen_verdict<kMode>(P, E, ev, lnt, w.r, task);
         if (verdict == kScreenUndecided) atomicAdd(&E.counters[2], 1ull);  // full FP64 cycle
       }
       bool have = verdict == kScreenWinner;
       if (__any_sync(0xffffffffu, verdict == kScreenUndecided))
-        fallback_warp<kMode>(P0, E, verdict == kScreenUndecided, ev, job, key, step, q >= 0 ? w.n[q] : 0, lnt, have,
+        fallback_warp<kMode>(P0, E, verdict == kScreenUndecided, ev, job, key, step, q >= 0 ? w.sc.n[q] : 0, lnt, have,
                              task);
       if (limited) w.state[q] = kSlotLimit;
       if (lead) {
@@ -652,7 +718,7 @@ __global__ void __launch_bounds__(kMaxThreads)
             w.won[q] = static_cast<uint32_t>(task.i) | (static_cast<uint32_t>(task.k) << 8) |
                        (static_cast<uint32_t>(task.side) << 16) | (static_cast<uint32_t>(task.kappa) << 20) |
                        (static_cast<uint32_t>(task.kind) << 24);
-            state = w.n[q] >= E.cap ? kSlotOverflow : kSlotPending;
+            state = w.sc.n[q] >= E.cap ? kSlotOverflow : kSlotPending;
           }
           if constexpr (kSlice) {
             const int cyc = w.cyc[q] + 1;
