@@ -403,7 +403,11 @@ HostCounters& host_counters() {
 }
 
 // The plain form rebuilds its active list in event order after a launch
-// while the list holds at least 1/GAPS_REBUILD_DIV of the batch.
+// while the list holds at least 1/GAPS_REBUILD_DIV of the batch, in batches of
+// GAPS_REBUILD_MIN events or more: below, the second-level cache serves the
+// scattered loads and the rebuild only costs its launch (10^3 events 1.53 ->
+// 1.20 ms and 1.2x10^4 4.60 -> 4.11 ms without it
+// above; 10^5 events 2.89 with it, 2.99 ms without).
 #ifndef GAPS_REBUILD_MIN
 #define GAPS_REBUILD_MIN 50000
 #endif
