@@ -6,7 +6,7 @@
 // a warp handle events of the same size: the O(n^3) loops of thrust and
 // Durham then run with no lane waiting on a larger neighbour.  Events of up
 // to 16 partons take one thread each, with per-thread arrays (in batches of
-// fewer than 50 000 events, groups of 4 lanes: the event's momenta sit in
+// fewer than 180 000 events, groups of 4 to 16 lanes: the event's momenta sit in
 // shared memory, the lanes split the pairs of each search and reduce their
 // partial results in the serial loop's order, and the O(n) FP64 steps run on
 // every lane alike, so the results are the one-thread results).  Larger
@@ -30,6 +30,8 @@
 //  * Final scalings take reciprocals (1/s, 1/|P|, 1/(2 sum |p|)): the
 //    oracle's divisions up to an ulp.  The cosine inside Durham's 1 - cos
 //    keeps the oracle's division, since 1 - cos magnifies its rounding.
+#include <type_traits>
+
 #include "gaps_launch.hpp"
 #include "sqrt_obs.cuh"
 
@@ -303,7 +305,7 @@ __device__ void event_shapes(const DevParams& P0, const Events& E, int64_t ev, i
     double ymin = 0.0;
     int bi = ui, bj = uj;
     if (n_cand == 1) {
-      ymin = y_exact(ui, uj);
+      if (m <= 6) ymin = y_exact(ui, uj);  // the merges that are recorded
     } else {
       atomicAdd(&E.counters[5], 1ull);  // merges with several FP64 candidates
       bi = -1;
@@ -391,11 +393,14 @@ struct PairWalk {
   }
 };
 
-// The event's arrays in shared memory, one set per group.
+// The event's arrays in shared memory, one set per group.  j: E, px, py, pz;
+// ja: |p|; pt, plus: |p x n_T| and the hemisphere of every parton; sums: the
+// hemispheres' sums of E, px, py, pz and pt.
 template <int MAXJ>
 struct GroupArrays {
-  double je[MAXJ], jx[MAXJ], jy[MAXJ], jz[MAXJ], ja[MAXJ];
+  double j[4][MAXJ], ja[MAXJ], pt[MAXJ], sums[2][5];
   float fx[MAXJ], fy[MAXJ], fz[MAXJ], fe2[MAXJ];
+  uint8_t plus[MAXJ];
 };
 
 // thrust_fp64 over the group: each lane takes its pairs, the group keeps the
@@ -409,23 +414,23 @@ __device__ double thrust_fp64_group(int n, const GroupArrays<MAXJ>& a, double su
   PairWalk w;
   for (w.start(n, sub); w.valid(n); w.next<L>(n)) {
     const int j = w.j, k = w.k();
-    const double nx = cross(a.jy[j], a.jz[k], a.jz[j], a.jy[k]);
-    const double ny = cross(a.jz[j], a.jx[k], a.jx[j], a.jz[k]);
-    const double nz = cross(a.jx[j], a.jy[k], a.jy[j], a.jx[k]);
+    const double nx = cross(a.j[2][j], a.j[3][k], a.j[3][j], a.j[2][k]);
+    const double ny = cross(a.j[3][j], a.j[1][k], a.j[1][j], a.j[3][k]);
+    const double nz = cross(a.j[1][j], a.j[2][k], a.j[2][j], a.j[1][k]);
     if (nx == 0.0 && ny == 0.0 && nz == 0.0) continue;
     double px = 0.0, py = 0.0, pz = 0.0;
     for (int i = 0; i < n; ++i) {
       if (i == j || i == k) continue;
-      const double sg = dot3(a.jx[i], a.jy[i], a.jz[i], nx, ny, nz) >= 0.0 ? 1.0 : -1.0;
-      px = fma(sg, a.jx[i], px);
-      py = fma(sg, a.jy[i], py);
-      pz = fma(sg, a.jz[i], pz);
+      const double sg = dot3(a.j[1][i], a.j[2][i], a.j[3][i], nx, ny, nz) >= 0.0 ? 1.0 : -1.0;
+      px = fma(sg, a.j[1][i], px);
+      py = fma(sg, a.j[2][i], py);
+      pz = fma(sg, a.j[3][i], pz);
     }
     for (int c = 0; c < 4; ++c) {
       const double fj = (c & 2) ? -1.0 : 1.0, fk = (c & 1) ? -1.0 : 1.0;
-      const double cx = fma(fk, a.jx[k], fma(fj, a.jx[j], px));
-      const double cy = fma(fk, a.jy[k], fma(fj, a.jy[j], py));
-      const double cz = fma(fk, a.jz[k], fma(fj, a.jz[j], pz));
+      const double cx = fma(fk, a.j[1][k], fma(fj, a.j[1][j], px));
+      const double cy = fma(fk, a.j[2][k], fma(fj, a.j[2][j], py));
+      const double cz = fma(fk, a.j[3][k], fma(fj, a.j[3][j], pz));
       const double c2 = dot3(cx, cy, cz, cx, cy, cz);
       if (c2 > best2) {  // within a lane the positions rise: the first wins ties
         best2 = c2;
@@ -451,10 +456,10 @@ __device__ double thrust_fp64_group(int n, const GroupArrays<MAXJ>& a, double su
     }
   }
   if (best2 < 0.0) {  // collinear: T = 1 along the first momentum
-    const double l = sqrt_obs(dot3(a.jx[0], a.jy[0], a.jz[0], a.jx[0], a.jy[0], a.jz[0]));
-    ax = a.jx[0] / l;
-    ay = a.jy[0] / l;
-    az = a.jz[0] / l;
+    const double l = sqrt_obs(dot3(a.j[1][0], a.j[2][0], a.j[3][0], a.j[1][0], a.j[2][0], a.j[3][0]));
+    ax = a.j[1][0] / l;
+    ay = a.j[2][0] / l;
+    az = a.j[3][0] / l;
     return 1.0;
   }
   const double l = sqrt_obs(best2), inv_l = 1.0 / l;
@@ -464,12 +469,14 @@ __device__ double thrust_fp64_group(int n, const GroupArrays<MAXJ>& a, double su
   return l / sum_abs;
 }
 
-// event_shapes for one event by a group of L lanes (every lane of the group
-// calls it for the same event).  The searches give exactly the serial
+// event_shapes for one event by a group of L >= 4 lanes (every lane of the
+// group calls it for the same event).  The searches give exactly the serial
 // results: each lane screens its pairs in the serial order, the group merges
-// the lanes' bests with the serial tie rule, and the O(n) FP64 steps (the
-// thrust sum, hemispheres, broadenings, the merged jets) run on every lane in
-// the serial order.  Lane 0 of the group writes the observables.
+// the lanes' bests with the serial tie rule, and the sums (thrust,
+// hemispheres, broadenings, the merged jets) run one component per lane in
+// the serial order: a warp can issue an FP64 instruction every 64 cycles
+// only, so a lone event's time is their number.  Lane 0 of the group writes
+// the observables.
 template <int MAXJ, int L>
 __device__ void event_shapes_group(const DevParams& P0, const Events& E, int64_t ev, int n, GroupArrays<MAXJ>& a,
                                    int sub, unsigned gm) {
@@ -477,10 +484,10 @@ __device__ void event_shapes_group(const DevParams& P0, const Events& E, int64_t
   for (int i = sub; i < n; i += L) {
     const size_t at = E.at(i, ev);
     const double x = E.px[at], y = E.py[at], z = E.pz[at];
-    a.je[i] = E.e[at];
-    a.jx[i] = x;
-    a.jy[i] = y;
-    a.jz[i] = z;
+    a.j[0][i] = E.e[at];
+    a.j[1][i] = x;
+    a.j[2][i] = y;
+    a.j[3][i] = z;
     a.fx[i] = f32_from_f64(x);
     a.fy[i] = f32_from_f64(y);
     a.fz[i] = f32_from_f64(z);
@@ -496,9 +503,9 @@ __device__ void event_shapes_group(const DevParams& P0, const Events& E, int64_t
   bool decided = false;
   if (n == 2) {
     const double inv_l = 1.0 / a.ja[0];
-    ax = a.jx[0] * inv_l;
-    ay = a.jy[0] * inv_l;
-    az = a.jz[0] * inv_l;
+    ax = a.j[1][0] * inv_l;
+    ay = a.j[2][0] * inv_l;
+    az = a.j[3][0] * inv_l;
     decided = true;
   } else if (n <= kMaskMax) {
     Top2 top;
@@ -549,13 +556,13 @@ __device__ void event_shapes_group(const DevParams& P0, const Events& E, int64_t
     }
     const float margin = 8.0f * static_cast<float>(n + 2) * 6.0e-8f * sum_absf * sum_absf;
     if (top.s1 >= 0.0f && top.s2 < top.s1 - margin) {
-      double px = 0.0, py = 0.0, pz = 0.0;
-      for (int i = 0; i < n; ++i) {
-        const double sg = ((top.m1 >> i) & 1ull) ? 1.0 : -1.0;
-        px = fma(sg, a.jx[i], px);
-        py = fma(sg, a.jy[i], py);
-        pz = fma(sg, a.jz[i], pz);
-      }
+      // a component per lane, each summed in the serial order
+      double sum = 0.0;
+      const int c = 1 + min(sub, 2);
+      for (int i = 0; i < n; ++i) sum = fma(((top.m1 >> i) & 1ull) ? 1.0 : -1.0, a.j[c][i], sum);
+      const int g0 = static_cast<int>(threadIdx.x & 31u) - sub;
+      const double px = __shfl_sync(gm, sum, g0), py = __shfl_sync(gm, sum, g0 + 1);
+      const double pz = __shfl_sync(gm, sum, g0 + 2);
       const double l = sqrt_obs(dot3(px, py, pz, px, py, pz)), inv_l = 1.0 / l;
       thrust = l / sum_abs;
       ax = px * inv_l;
@@ -568,33 +575,36 @@ __device__ void event_shapes_group(const DevParams& P0, const Events& E, int64_t
     if (sub == 0) atomicAdd(&E.counters[4], 1ull);  // thrust decided by the exact FP64 search
     thrust = thrust_fp64_group<MAXJ, L>(n, a, sum_abs, sub, gm, ax, ay, az);
   }
-  double hp[4] = {0, 0, 0, 0}, hm[4] = {0, 0, 0, 0};
-  double bp = 0.0, bm = 0.0;
-  for (int i = 0; i < n; ++i) {
-    const double x = a.jx[i], y = a.jy[i], z = a.jz[i];
+  // Hemispheres: every parton's side and |p x n_T| on a lane of its own, the
+  // sums one per lane in the serial order.
+  for (int i = sub; i < n; i += L) {
+    const double x = a.j[1][i], y = a.j[2][i], z = a.j[3][i];
     const long long pn = __double_as_longlong(dot3(x, y, z, ax, ay, az));
-    const bool plus = pn >= 0 || pn == static_cast<long long>(0x8000000000000000ull);
-    double* h = plus ? hp : hm;
-    h[0] += a.je[i];
-    h[1] += x;
-    h[2] += y;
-    h[3] += z;
+    a.plus[i] = pn >= 0 || pn == static_cast<long long>(0x8000000000000000ull);
     const double cx = cross(y, az, z, ay), cy = cross(z, ax, x, az), cz = cross(x, ay, y, ax);
-    const double pt = sqrt_obs(dot3(cx, cy, cz, cx, cy, cz));
-    if (plus) {
-      bp += pt;
-    } else {
-      bm += pt;
-    }
+    a.pt[i] = sqrt_obs(dot3(cx, cy, cz, cx, cy, cz));
   }
+  __syncwarp(gm);
+  for (int c = sub; c < 5; c += L) {
+    const double* v = c < 4 ? a.j[c] : a.pt;
+    double plus = 0.0, minus = 0.0;
+    for (int i = 0; i < n; ++i) {
+      const bool p = a.plus[i] != 0;
+      const double sum = (p ? plus : minus) + v[i];
+      plus = p ? sum : plus;
+      minus = p ? minus : sum;
+    }
+    a.sums[0][c] = plus;
+    a.sums[1][c] = minus;
+  }
+  __syncwarp(gm);
   if (sub == 0) {
-    const double mp = mass2(hp);
-    const double mm = mass2(hm);
+    const double mp = mass2(a.sums[0]);
+    const double mm = mass2(a.sums[1]);
     E.obs[4 * E.stride + ev] = 1.0 - thrust;
     E.obs[5 * E.stride + ev] = fmax(mp, mm) * P.inv_s;
     const double inv_2sum = 0.5 / sum_abs;
-    bp *= inv_2sum;
-    bm *= inv_2sum;
+    const double bp = a.sums[0][4] * inv_2sum, bm = a.sums[1][4] * inv_2sum;
     E.obs[6 * E.stride + ev] = bp + bm;
     E.obs[7 * E.stride + ev] = fmax(bp, bm);
   }
@@ -602,7 +612,7 @@ __device__ void event_shapes_group(const DevParams& P0, const Events& E, int64_t
   // ---- Durham (E-scheme)
   __syncwarp(gm);  // every lane has read the FP32 momenta
   for (int i = sub; i < n; i += L) {
-    const float e = f32_from_f64(a.je[i]);
+    const float e = f32_from_f64(a.j[0][i]);
     a.fe2[i] = e * e;
     const float r = rsqrtf(dot3f(a.fx[i], a.fy[i], a.fz[i], a.fx[i], a.fy[i], a.fz[i]));
     a.fx[i] *= r;
@@ -612,8 +622,8 @@ __device__ void event_shapes_group(const DevParams& P0, const Events& E, int64_t
   __syncwarp(gm);
   double yres[4] = {-1.0, -1.0, -1.0, -1.0};
   auto y_exact = [&](int i, int j) {
-    const double cosij = dot3(a.jx[i], a.jy[i], a.jz[i], a.jx[j], a.jy[j], a.jz[j]) / (a.ja[i] * a.ja[j]);
-    return 2.0 * fmin(a.je[i] * a.je[i], a.je[j] * a.je[j]) * (1.0 - cosij) * P.inv_s;
+    const double cosij = dot3(a.j[1][i], a.j[2][i], a.j[3][i], a.j[1][j], a.j[2][j], a.j[3][j]) / (a.ja[i] * a.ja[j]);
+    return 2.0 * fmin(a.j[0][i] * a.j[0][i], a.j[0][j] * a.j[0][j]) * (1.0 - cosij) * P.inv_s;
   };
   auto bounds = [&](int i, int j, float& y, float& rel) {
     const float dx = a.fx[i] - a.fx[j], dy = a.fy[i] - a.fy[j], dz = a.fz[i] - a.fz[j];
@@ -661,7 +671,7 @@ __device__ void event_shapes_group(const DevParams& P0, const Events& E, int64_t
     double ymin = 0.0;
     int bi = ui, bj = uj;
     if (n_cand == 1) {
-      ymin = y_exact(ui, uj);
+      if (m <= 6) ymin = y_exact(ui, uj);  // the merges that are recorded
     } else {
       if (sub == 0) atomicAdd(&E.counters[5], 1ull);  // merges with several FP64 candidates
       int bp_ = 0x7fffffff;
@@ -695,24 +705,22 @@ __device__ void event_shapes_group(const DevParams& P0, const Events& E, int64_t
     const int idx = m - 3;
     if (idx >= 0 && idx < 4) yres[idx] = ymin;
     __syncwarp(gm);  // every lane is done reading the jets of this merge
+    if (sub < 4) {  // a component per lane (L >= 4)
+      a.j[sub][bi] += a.j[sub][bj];
+      a.j[sub][bj] = a.j[sub][m - 1];
+    }
+    __syncwarp(gm);
     if (sub == 0) {
-      a.je[bi] += a.je[bj];
-      a.jx[bi] += a.jx[bj];
-      a.jy[bi] += a.jy[bj];
-      a.jz[bi] += a.jz[bj];
-      a.je[bj] = a.je[m - 1];
-      a.jx[bj] = a.jx[m - 1];
-      a.jy[bj] = a.jy[m - 1];
-      a.jz[bj] = a.jz[m - 1];
+      const double jx = a.j[1][bi], jy = a.j[2][bi], jz = a.j[3][bi];
       a.ja[bj] = a.ja[m - 1];
-      a.ja[bi] = sqrt_obs(dot3(a.jx[bi], a.jy[bi], a.jz[bi], a.jx[bi], a.jy[bi], a.jz[bi]));
+      a.ja[bi] = sqrt_obs(dot3(jx, jy, jz, jx, jy, jz));
       a.fe2[bj] = a.fe2[m - 1];
       a.fx[bj] = a.fx[m - 1];
       a.fy[bj] = a.fy[m - 1];
       a.fz[bj] = a.fz[m - 1];
-      const float e = f32_from_f64(a.je[bi]);
+      const float e = f32_from_f64(a.j[0][bi]);
       a.fe2[bi] = e * e;
-      const float x = f32_from_f64(a.jx[bi]), y = f32_from_f64(a.jy[bi]), z = f32_from_f64(a.jz[bi]);
+      const float x = f32_from_f64(jx), y = f32_from_f64(jy), z = f32_from_f64(jz);
       const float r = rsqrtf(dot3f(x, y, z, x, y, z));
       a.fx[bi] = x * r;
       a.fy[bi] = y * r;
@@ -1352,6 +1360,7 @@ __device__ __forceinline__ int shape_partons(const Events& E, int64_t ev) {
 
 // counts[n] = finished events with n partons (2 <= n <= capacity <= 255).
 __global__ void __launch_bounds__(256) k_bucket_count(Events E, int* counts, Ranges R) {
+  follow_launch();
   __shared__ int sh[256];
   sh[threadIdx.x] = 0;
   __syncthreads();
@@ -1366,9 +1375,13 @@ __global__ void __launch_bounds__(256) k_bucket_count(Events E, int* counts, Ran
 
 // offsets[n] = first position of bucket n; cursor[n] = offsets[n];
 // offsets[256] = number of finished events.
-__global__ void __launch_bounds__(256) k_bucket_scan(const int* counts, int* offsets, int* cursor) {
+// Clears the observables' counter words too (the kernels behind it count).
+__global__ void __launch_bounds__(256) k_bucket_scan(const int* counts, int* offsets, int* cursor,
+                                                     unsigned long long* counters) {
+  follow_launch();
   __shared__ int sh[256];
   const int t = threadIdx.x;
+  if (t == 4 || t == 5 || t == 8) counters[t] = 0ull;
   sh[t] = counts[t];
   __syncthreads();
   for (int d = 1; d < 256; d <<= 1) {
@@ -1391,6 +1404,7 @@ __global__ void __launch_bounds__(256) k_bucket_scan(const int* counts, int* off
 // few hot buckets (a handful of multiplicities hold most events) see a
 // thousand times fewer global atomics than with one per event.
 __global__ void __launch_bounds__(256) k_bucket_scatter(Events E, int* cursor, int* order, Ranges R) {
+  follow_launch();
   __shared__ int s_cnt[256];
   __shared__ int s_base[256];
   const int tid = threadIdx.x, lane = tid & 31;
@@ -1421,6 +1435,53 @@ __global__ void __launch_bounds__(256) k_bucket_scatter(Events E, int* cursor, i
   }
 }
 
+// Count, scan and scatter of a small batch by one block: the same buckets in
+// one launch instead of a clearing and three.
+constexpr int64_t kSmallBuckets = 4096;
+__global__ void __launch_bounds__(1024) k_buckets_small(Events E, int* offsets, int* cursor, int* order, Ranges R) {
+  follow_launch();
+  __shared__ int sh[256], place[256];
+  const int tid = threadIdx.x;
+  constexpr int kEach = static_cast<int>(kSmallBuckets) / 1024;
+  int n[kEach];
+  int64_t ev[kEach];
+  if (tid < 256) sh[tid] = 0;
+  if (tid == 4 || tid == 5 || tid == 8) E.counters[tid] = 0ull;
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < kEach; ++c) {
+    const int64_t t = c * 1024 + tid;
+    n[c] = -1;
+    if (t >= E.n) continue;
+    ev[c] = R.event(t);
+    n[c] = shape_partons(E, ev[c]);
+    if (n[c] >= 0) {
+      atomicAdd(&sh[n[c]], 1);
+    } else {
+      if (E.status[ev[c]] == GAPS_DONE) atomicAdd(&E.counters[8], 1ull);
+      for (int h = 0; h < GAPS_N_OBS; ++h) E.obs[h * E.stride + ev[c]] = -1.0;
+    }
+  }
+  __syncthreads();
+  for (int d = 1; d < 256; d <<= 1) {
+    const int v = tid < 256 && tid >= d ? sh[tid - d] : 0;
+    __syncthreads();
+    if (tid < 256) sh[tid] += v;
+    __syncthreads();
+  }
+  if (tid < 256) {
+    const int excl = tid ? sh[tid - 1] : 0;
+    offsets[tid] = excl;
+    place[tid] = excl;
+    if (tid == 255) offsets[256] = sh[255];
+    if (tid < 2) cursor[tid] = 0;  // the large events' cursors (no event has 0 or 1 partons)
+  }
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < kEach; ++c)
+    if (n[c] >= 0) order[atomicAdd(&place[n[c]], 1)] = static_cast<int>(ev[c]);
+}
+
 // Events of buckets n_lo..n_hi (all with n <= MAXJ), the largest first: the
 // order list holds the buckets by rising multiplicity, and the threads take
 // it from its end, so the blocks with the costliest events start first and
@@ -1429,6 +1490,7 @@ __global__ void __launch_bounds__(256) k_bucket_scatter(Events E, int* cursor, i
 template <int MAXJ>
 __global__ void __launch_bounds__(kShapeThreads) k_event_shapes(DevParams P, Events E, const int* order,
                                                                 const int* offsets, int n_lo, int n_hi) {
+  follow_launch();
   const int begin = offsets[n_lo], end = offsets[n_hi + 1 > 256 ? 256 : n_hi + 1];
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < end - begin; j += gridDim.x * blockDim.x) {
     const int64_t ev = order[end - 1 - j];
@@ -1441,6 +1503,7 @@ __global__ void __launch_bounds__(kShapeThreads) k_event_shapes(DevParams P, Eve
 template <int MAXJ, int L, int T>
 __global__ void __launch_bounds__(T) k_event_shapes_group(DevParams P, Events E, const int* order,
                                                           const int* offsets, int n_lo, int n_hi) {
+  follow_launch();
   constexpr int G = T / L;
   __shared__ GroupArrays<MAXJ> s_ev[G];
   const int g = threadIdx.x / L, sub = threadIdx.x % L;
@@ -1459,6 +1522,7 @@ __global__ void __launch_bounds__(T) k_event_shapes_group(DevParams P, Events E,
 template <int MAXJ, int T>
 __global__ void __launch_bounds__(T) k_event_shapes_warp(DevParams P, Events E, const int* order, const int* offsets,
                                                          int n_lo, int n_hi, int* cursor) {
+  follow_launch();
   extern __shared__ __align__(16) unsigned char s_shapes[];
   WarpEvent<MAXJ>& a = reinterpret_cast<WarpEvent<MAXJ>*>(s_shapes)[threadIdx.x >> 5];
   const int lane = static_cast<int>(threadIdx.x & 31);
@@ -1476,37 +1540,30 @@ __global__ void __launch_bounds__(T) k_event_shapes_warp(DevParams P, Events E, 
 }
 
 // Events of up to 16 partons take one thread each in batches of at least
-// GAPS_SHAPES_GROUP_BELOW events (throughput), groups of
-// GAPS_SHAPES_SMALL_LANES lanes in smaller ones (a launch then waits for its
-// slowest event, not for the SMs).  At 10^6 LEP events one thread per event
-// up to 16 partons measured 1.04 ms for the observables, against 1.47 ms with
-// 9..16-parton events in groups of 8 and 1.36 ms with the per-thread events
-// in two launches (up to 8 partons, 9..16).  The per-thread grid holds one
-// thread per event up to GAPS_SHAPES_BLOCKS_PER_SM blocks per SM (largest
-// events first, above): 0.919 ms at 10^6 events and 0.623 ms at 5x10^5,
-// against 0.967 and 0.702 ms for 16 blocks per SM striding over the events
-// in rising size, and 1.168 and 0.726 ms for a grid of the resident blocks
-// only.
-#ifndef GAPS_SHAPES_BLOCKS_PER_SM
-#define GAPS_SHAPES_BLOCKS_PER_SM 64
-#endif
-#ifndef GAPS_SHAPES_GROUP_BELOW
-#define GAPS_SHAPES_GROUP_BELOW 50000
-#endif
-#ifndef GAPS_SHAPES_SMALL_LANES
-#define GAPS_SHAPES_SMALL_LANES 4
-#endif
-constexpr int kSmallLanes = GAPS_SHAPES_SMALL_LANES;
+// kThreadsFrom events (throughput), groups of lanes in smaller ones (a launch
+// then waits for its slowest event, not for the SMs), the more the smaller the
+// batch: the stage at 10^3 events takes 122, 92 and 72 us with 4, 8 and 16
+// lanes, at 2x10^4 138, 122 and 178, at 4.9x10^4 172, 201 and 380; at 10^5 254
+// with 4 lanes and 349 with one thread per event, at 3x10^5 613 and 490 us.
+// The per-thread grid holds one thread per event up to kShapeBlocksPerSm
+// blocks per SM (largest events first, above): 0.86 ms at 10^6 events; a
+// second launch of lane groups for 7, 9, 11 or 13 .. 16 partons there took the
+// stage to 1.10, 1.00, 0.99 and 0.93.
+constexpr int kShapeBlocksPerSm = 64;
+constexpr int64_t kThreadsFrom = 180000;
 
 }  // namespace
 
 cudaError_t preload_observables() {
   cudaFuncAttributes a;
   cudaError_t e = cudaFuncGetAttributes(&a, k_bucket_count);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_buckets_small);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_bucket_scan);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_bucket_scatter);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes<16>);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_group<16, kSmallLanes, 128>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_group<16, 4, 128>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_group<16, 8, 128>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_group<16, 16, 128>);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_warp<128, 128>);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_warp<256, 64>);
   return e;
@@ -1520,16 +1577,19 @@ cudaError_t launch_observables(const DevParams& P, const Events& E, int* buckets
   int* counts = buckets;
   int* offsets = buckets + 256;
   int* cursor = buckets + 256 + 257;
-  cudaError_t e = cudaMemsetAsync(counts, 0, 256 * sizeof(int), s);
+  const bool chain = E.n < kChainBelow;
+  cudaError_t e = cudaSuccess;
+  if (E.n <= kSmallBuckets) {
+    e = launch_chained(chain, k_buckets_small, 1, 1024, 0, s, E, offsets, cursor, order, R);
+  } else {
+    const int64_t want = (E.n + 255) / 256;
+    const int64_t grid_count = want < 4 * sms ? want : 4 * sms;
+    e = cudaMemsetAsync(counts, 0, 256 * sizeof(int), s);
+    if (e == cudaSuccess) e = launch_chained(chain, k_bucket_count, grid_count, 256, 0, s, E, counts, R);
+    if (e == cudaSuccess) e = launch_chained(chain, k_bucket_scan, 1, 256, 0, s, counts, offsets, cursor, E.counters);
+    if (e == cudaSuccess) e = launch_chained(chain, k_bucket_scatter, grid_count, 256, 0, s, E, cursor, order, R);
+  }
   if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(E.counters + 4, 0, 2 * sizeof(unsigned long long), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(E.counters + 8, 0, sizeof(unsigned long long), s);
-  if (e != cudaSuccess) return e;
-  const int64_t want = (E.n + 255) / 256;
-  const unsigned grid_count = static_cast<unsigned>(want < 4 * sms ? want : 4 * sms);
-  k_bucket_count<<<grid_count, 256, 0, s>>>(E, counts, R);
-  k_bucket_scan<<<1, 256, 0, s>>>(counts, offsets, cursor);
-  k_bucket_scatter<<<grid_count, 256, 0, s>>>(E, cursor, order, R);
   // One launch per multiplicity class; grids cover the largest possible
   // class (blocks of one event per thread or per group) and stride over the
   // actual one.
@@ -1537,21 +1597,30 @@ cudaError_t launch_observables(const DevParams& P, const Events& E, int* buckets
     const int64_t want = (E.n + per_block - 1) / per_block;
     return static_cast<unsigned>(want < static_cast<int64_t>(per_sm) * sms ? want : static_cast<int64_t>(per_sm) * sms);
   };
-  if (E.n < GAPS_SHAPES_GROUP_BELOW) {
-    k_event_shapes_group<16, kSmallLanes, 128><<<grid(128 / kSmallLanes, 8), 128, 0, s>>>(P, E, order, offsets, 0, 16);
+  const auto groups = [&](auto lanes) {
+    constexpr int L = decltype(lanes)::value;
+    return launch_chained(chain, k_event_shapes_group<16, L, 128>, grid(128 / L, 8), 128, 0, s, P, E, order, offsets, 0, 16);
+  };
+  if (E.n < 10000) {
+    e = groups(std::integral_constant<int, 16>{});
+  } else if (E.n < 30000) {
+    e = groups(std::integral_constant<int, 8>{});
+  } else if (E.n < kThreadsFrom) {
+    e = groups(std::integral_constant<int, 4>{});
   } else {
-    k_event_shapes<16><<<grid(kShapeThreads, GAPS_SHAPES_BLOCKS_PER_SM), kShapeThreads, 0, s>>>(P, E, order, offsets, 0, 16);
+    e = launch_chained(chain, k_event_shapes<16>, grid(kShapeThreads, kShapeBlocksPerSm), kShapeThreads, 0, s, P, E, order,
+                       offsets, 0, 16);
   }
   // One class up to 128 partons (96 registers leave five blocks per SM), one
   // beyond.  Their cursors are the bucket cursors of 0 and 1 partons, which no
   // event has: zero.
-  if (E.cap > 16)
-    k_event_shapes_warp<128, 128>
-        <<<grid(4, 5), 128, 4 * sizeof(WarpEvent<128>), s>>>(P, E, order, offsets, 17, 128, cursor);
-  if (E.cap > 128)
-    k_event_shapes_warp<256, 64>
-        <<<grid(2, 6), 64, 2 * sizeof(WarpEvent<256>), s>>>(P, E, order, offsets, 129, 255, cursor + 1);
-  return cudaGetLastError();
+  if (e == cudaSuccess && E.cap > 16)
+    e = launch_chained(chain, k_event_shapes_warp<128, 128>, grid(4, 5), 128, 4 * sizeof(WarpEvent<128>), s, P, E, order,
+                       offsets, 17, 128, cursor);
+  if (e == cudaSuccess && E.cap > 128)
+    e = launch_chained(chain, k_event_shapes_warp<256, 64>, grid(2, 6), 64, 2 * sizeof(WarpEvent<256>), s, P, E, order,
+                       offsets, 129, 255, cursor + 1);
+  return e;
 }
 
 }  // namespace gaps

@@ -205,6 +205,16 @@ inline void set_layout(Events& E, int layout, int64_t n_events, int capacity) {
   }
 }
 
+// At the top of a kernel that may be launched as a programmatic dependent
+// (launch_chained): let the stream's next launch be set up beside this one,
+// and wait for the one before to be complete.  Every thread of every block
+// passes it, so the launches stay ordered.  Without that attribute it does
+// nothing.
+__device__ __forceinline__ void follow_launch() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // The events a finalisation kernel visits: positions t = 0 .. E.n - 1 of a
 // view, or of a list of disjoint event ranges (several finished jobs of a
 // serving pool at once): range j holds positions prefix[j] ..

@@ -13,6 +13,29 @@ DevParams make_dev_params(const gaps_params& p, int64_t id_offset);
 int record_cuda_error(cudaError_t e);
 Events make_events(const gaps_batch& b);
 
+// Launch a kernel that starts with follow_launch().  chain: its blocks may be
+// placed while the stream's previous kernel runs (programmatic dependent
+// launch), so that a sequence of short launches does not pay each one's
+// latency; where launches fill the device their blocks would spread unevenly
+// over the SMs.
+template <class... Params, class... Args>
+cudaError_t launch_chained(bool chain, void (*kernel)(Params...), int64_t blocks, int threads, size_t smem,
+                           cudaStream_t s, const Args&... args) {
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3(static_cast<unsigned>(blocks));
+  lc.blockDim = dim3(static_cast<unsigned>(threads));
+  lc.dynamicSmemBytes = smem;
+  lc.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = &at;
+  lc.numAttrs = chain ? 1 : 0;
+  return cudaLaunchKernelEx(&lc, kernel, static_cast<Params>(args)...);
+}
+// Batches whose finalisation launches are chained.
+constexpr int64_t kChainBelow = 50000;
+
 cudaError_t launch_me(const DevParams& P, const Events& E, cudaStream_t s);
 // One plain-form cycle over list_in[0 .. n_in) (list_in = NULL: events
 // 0 .. n_in); survivors are appended to list_out (may be NULL) through

@@ -153,13 +153,6 @@ __global__ void __launch_bounds__(kStepThreads, GAPS_STEP_MIN_BLOCKS)
     refresh_dipole<kJobPhysics<kMode>>(P, E, s_task[refresh_task(s_jobs[j])].ev, s_jobs[j]);
 }
 
-// A launch of the plain form's chain (launch_chained): let the next one be
-// set up beside this one, and wait for the one before to be complete.
-__device__ __forceinline__ void follow_launch() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-
 // Slot of this thread's item in an output list shared by the grid: one
 // atomic per warp.  Every lane of the warp must call it; returns -1 where
 // flag is false.
@@ -406,29 +399,6 @@ __global__ void __launch_bounds__(256) k_list_active(Events E, int64_t n, int* l
 
 }  // namespace
 
-namespace {
-
-// Launch a kernel that starts with follow_launch(): its blocks may be placed
-// while the stream's previous kernel runs (programmatic dependent launch), so
-// the steps, each of which has to wait for the one before, follow one another
-// without the launch's own latency.  Shower 10^3 events 1.23 -> 1.06 ms,
-// 1.2x10^4 (200 GeV) 4.19 -> 3.95, 10^5 2.92 -> 2.83, 10^6 8.53 -> 8.37.
-template <class... Params, class... Args>
-cudaError_t launch_chained(void (*kernel)(Params...), int64_t blocks, int threads, cudaStream_t s, const Args&... args) {
-  cudaLaunchConfig_t lc{};
-  lc.gridDim = dim3(static_cast<unsigned>(blocks));
-  lc.blockDim = dim3(static_cast<unsigned>(threads));
-  lc.stream = s;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  lc.attrs = &at;
-  lc.numAttrs = 1;
-  return cudaLaunchKernelEx(&lc, kernel, static_cast<Params>(args)...);
-}
-
-}  // namespace
-
 cudaError_t launch_me(const DevParams& P, const Events& E, cudaStream_t s) {
   if (E.n == 0) return cudaSuccess;
   const int threads = 256;
@@ -501,9 +471,12 @@ cudaError_t launch_step_deferred(const DevParams& P, const Events& E, const int*
   const int64_t emit_blocks = std::min((n_tasks + kEmitChunk - 1) / kEmitChunk, resident / 1024 * emit_per_sm);
   if (select_blocks + emit_blocks == 0) return cudaSuccess;
   const int64_t grid = select_blocks + emit_blocks;
+  // Chained: the steps follow one another without the launch's own latency.
+  // Shower 10^3 events 1.23 -> 1.06 ms, 1.2x10^4 (200 GeV) 4.19 -> 3.95, 10^5
+  // 2.92 -> 2.83, 10^6 8.53 -> 8.37.
 #define GAPS_DEFERRED_CASE(MULTI, LN)                                                                            \
   case LN:                                                                                                       \
-    return launch_chained(k_step_deferred<MULTI, LN>, grid, kStepThreads, s, P, E, select_blocks, list_in, n_list, \
+    return launch_chained(true, k_step_deferred<MULTI, LN>, grid, kStepThreads, 0, s, P, E, select_blocks, list_in, n_list, \
                           n_list_dev, tasks_in, n_tasks, n_tasks_dev, list_out, list_count, tasks_out, task_count, \
                           reset_list, reset_tasks, emit_cursor, reset_cursor, pub);
 #define GAPS_DEFERRED_SWITCH(MULTI)  \
