@@ -147,6 +147,7 @@ __device__ __forceinline__ void validate_event(const DevParams& P0, const Events
 constexpr int kValidateThreads = GAPS_VALIDATE_THREADS;
 
 __global__ void __launch_bounds__(kValidateThreads) k_validate(DevParams P0, Events E, Ranges R) {
+  follow_launch();
   __shared__ int s_bin[256];  // counts per parton count, then the first slot of each
   __shared__ int s_pos[kValidateThreads];
   const int tid = threadIdx.x;
@@ -184,6 +185,111 @@ __global__ void __launch_bounds__(kValidateThreads) k_validate(DevParams P0, Eve
   if (key >= 0) s_pos[s_bin[key] + rank] = tid;
   __syncthreads();
   if (first + tid < E.n) validate_event(P0, E, R.event(first + s_pos[tid]));
+}
+
+// Validation by a group of L lanes per event, for batches that leave SMs idle
+// with one thread per event: a thread walks its event's partons and colour
+// links one memory latency after another (22 us for 100 events); here the
+// lanes load them side by side and the links are followed in shared memory.
+// The same tests, and the momentum sums in the serial order (a component per
+// lane), so the bits are validate_event's.  Events of more than kLaneMax
+// partons take it as it is.
+constexpr int kLaneMax = 32;
+struct LaneEvent {
+  double j[4][kLaneMax];
+  uint8_t link0[kLaneMax];
+  int8_t flav[kLaneMax];
+};
+template <int L>
+__global__ void __launch_bounds__(kValidateThreads) k_validate_lanes(DevParams P0, Events E, Ranges R) {
+  follow_launch();
+  __shared__ LaneEvent s_ev[kValidateThreads / L];
+  const int sub = static_cast<int>(threadIdx.x) % L, first = (static_cast<int>(threadIdx.x) & 31) - sub;
+  const unsigned gm = (L == 32 ? 0xffffffffu : (1u << L) - 1u) << first;
+  LaneEvent& w = s_ev[threadIdx.x / L];
+  const int64_t t = static_cast<int64_t>(blockIdx.x) * (kValidateThreads / L) + threadIdx.x / L;
+  if (t >= E.n) return;  // (whole groups)
+  const int64_t ev = R.event(t);
+  const DevParams& P = params_of_event(P0, E, ev);
+  const int n = min(max(E.n_partons[ev], 0), E.cap);
+  if (n > kLaneMax) {
+    if (sub == 0) validate_event(P0, E, ev);
+    return;
+  }
+  int bits = 0;
+  long long fsum = 0;
+  bool colour_ok = true;
+  const int u_s = normal_exponent(P.sqrt_s);
+  for (int i = sub; i < n; i += L) {
+    const size_t a = E.at(i, ev);
+    const double e = E.e[a], x = E.px[a], y = E.py[a], z = E.pz[a];
+    const int fl = E.flav[a], c = E.col[a], ac = E.acol[a];
+    const int l0 = E.link[E.link_at(0, i, ev)], l1 = E.link[E.link_at(1, i, ev)];
+    if (!(finite_bits(e) && finite_bits(x) && finite_bits(y) && finite_bits(z))) bits |= 32;
+    if (!(finite_bits(e) ? positive_finite_bits(e) : e > 0.0)) bits |= 4;
+    if (off_shell(fma(-z, z, fma(-y, y, fma(-x, x, e * e))), e, P.sqrt_s, u_s)) bits |= 2;
+    if (fl == kGluon) {
+      colour_ok &= c > 0 && ac > 0;
+    } else if (fl >= 1 && fl <= 5) {
+      colour_ok &= c > 0 && ac == 0;
+      fsum += 1ll << (8 * fl);
+    } else if (fl <= -1 && fl >= -5) {
+      colour_ok &= c == 0 && ac > 0;
+      fsum -= 1ll << (-8 * fl);
+    } else {
+      colour_ok = false;
+    }
+    const bool in0 = l0 != kNoLink && l0 < n, in1 = l1 != kNoLink && l1 < n;
+    if (c > 0) {
+      colour_ok &= in0 && E.acol[E.at(in0 ? l0 : 0, ev)] == c && E.link[E.link_at(1, in0 ? l0 : 0, ev)] == i;
+    } else {
+      colour_ok &= l0 == kNoLink;
+    }
+    if (ac > 0) {
+      colour_ok &= in1 && E.col[E.at(in1 ? l1 : 0, ev)] == ac && E.link[E.link_at(0, in1 ? l1 : 0, ev)] == i;
+    } else {
+      colour_ok &= l1 == kNoLink;
+    }
+    w.j[0][i] = e;
+    w.j[1][i] = x;
+    w.j[2][i] = y;
+    w.j[3][i] = z;
+    w.link0[i] = static_cast<uint8_t>(l0);
+    w.flav[i] = static_cast<int8_t>(fl);
+  }
+  __syncwarp(gm);
+  for (int c = sub; c < 4; c += L) {
+    double sum = 0.0;
+    for (int i = 0; i < n; ++i) sum += w.j[c][i];
+    if (fabs(c == 0 ? sum - P.sqrt_s : sum) > 1e-10) bits |= 1;
+  }
+  colour_ok = __all_sync(gm, colour_ok);
+  if (colour_ok) {  // consistent links: every chain from a quark ends
+    int visited = 0;
+    for (int i = sub; i < n; i += L) {
+      const int fl = w.flav[i];
+      if (!(fl >= 1 && fl <= 5)) continue;
+      int cur = i;
+      for (int guard = 0; guard <= n; ++guard) {
+        ++visited;
+        const int nxt = w.link0[cur];
+        if (nxt == kNoLink) break;
+        cur = nxt;
+      }
+      colour_ok &= w.flav[cur] <= -1 && w.flav[cur] >= -5;
+    }
+#pragma unroll
+    for (int o = 1; o < L; o <<= 1) visited += __shfl_xor_sync(gm, visited, o);
+    colour_ok &= visited == n;
+  }
+  if (!colour_ok) bits |= 8;
+#pragma unroll
+  for (int o = 1; o < L; o <<= 1) {
+    bits |= __shfl_xor_sync(gm, bits, o);
+    fsum += __shfl_xor_sync(gm, fsum, o);
+  }
+  if (fsum != 0) bits |= 16;
+  if (sub == 0) E.valid[ev] = bits;
 }
 
 // ---------------------------------------------------------- histograms
@@ -286,9 +392,10 @@ __device__ __forceinline__ void split_sum_to128(unsigned long long lo_sum, long 
 // it is given.  Multi-job batch: a job's events lie together, so nearly
 // every fill is the home job's; the others go to acc directly as 128-bit
 // adds; every event at its own job's scales.
-template <bool kJobs>
+template <bool kJobs, bool kSplit>
 __global__ void __launch_bounds__(256) k_hist_fixed(DevParams P, const DevParams* scale_src, Events E,
                                                     unsigned long long* acc, Ranges R) {
+  follow_launch();
   // per cell: sum lo(w), sum hi(w), sum lo(w^2), sum hi(w^2), entries
   __shared__ unsigned long long sh[GAPS_HIST_FIXED_WORDS];
   __shared__ long long s_w[256], s_w2[256];
@@ -305,8 +412,10 @@ __global__ void __launch_bounds__(256) k_hist_fixed(DevParams P, const DevParams
     sc_w = scale_src->hist_sw;
     sc_w2 = scale_src->hist_sw2;
   }
+  // kSplit: the eight warps take an observable each of the same 32 events
   // every lane of a warp runs the same iterations (the match needs them all)
-  for (int64_t base = b0 + warp0; base < b1; base += blockDim.x) {
+  const int h0 = kSplit ? warp0 / 32 : 0, h1 = kSplit ? h0 + 1 : GAPS_N_OBS;
+  for (int64_t base = b0 + (kSplit ? 0 : warp0); base < b1; base += kSplit ? 32 : 256) {
     const int64_t t = base + lane;
     const int64_t ev = t < b1 ? R.event(t) : 0;
     const bool fill = t < b1 && E.status[ev] == GAPS_DONE && E.valid[ev] == 0;
@@ -318,14 +427,14 @@ __global__ void __launch_bounds__(256) k_hist_fixed(DevParams P, const DevParams
     // the event's observables, all loads in flight at once
     double o[GAPS_N_OBS];
 #pragma unroll
-    for (int h = 0; h < GAPS_N_OBS; ++h) o[h] = fill ? E.obs[h * E.stride + ev] : -1.0;
+    for (int h = 0; h < GAPS_N_OBS; ++h) o[h] = fill && h >= h0 && h < h1 ? E.obs[h * E.stride + ev] : -1.0;
     const double w = fill ? E.weight[ev] : 0.0;
     // exact scalings by powers of two, then one rounding to an integer
     s_w[tid] = __double2ll_rn(w * sc_w);
     s_w2[tid] = __double2ll_rn((w * w) * sc_w2);
     __syncwarp();
 #pragma unroll 1
-    for (int h = 0; h < GAPS_N_OBS; ++h) {
+    for (int h = h0; h < h1; ++h) {
       const int bin = fill ? hist_bin(h, o[h]) : -1;
       const int cell = bin < 0 ? -1 : job * kCells + h * GAPS_HIST_ROW + bin;
       const unsigned peers = __match_any_sync(0xffffffffu, cell);
@@ -383,6 +492,7 @@ __global__ void __launch_bounds__(256) k_hist_fixed(DevParams P, const DevParams
 __global__ void __launch_bounds__(256) k_hist_finalize(DevParams P, const DevParams* scale_src, const DevParams* jobs,
                                                        int n_sets, const unsigned long long* n_sets_dev,
                                                        unsigned long long* acc, double* hist) {
+  follow_launch();
   const int sets = n_sets_dev ? static_cast<int>(*n_sets_dev) : n_sets;
   for (int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; k < static_cast<int64_t>(sets) * kCells;
        k += static_cast<int64_t>(gridDim.x) * blockDim.x) {
@@ -414,6 +524,7 @@ __global__ void __launch_bounds__(256) k_fill_job_of(uint16_t* job_of, const int
 
 // -------------------------------------------------------------- stats
 __global__ void __launch_bounds__(256) k_stats(Events E, gaps_stats* st) {
+  follow_launch();
   long long done = 0, over = 0, lim = 0, inval = 0, steps = 0, mx = 0, trials = 0, wins = 0, ems = 0,
             parts = 0, dips = 0;
   double sw = 0.0, sw2 = 0.0;
@@ -477,8 +588,19 @@ __global__ void __launch_bounds__(256) k_stats(Events E, gaps_stats* st) {
 
 }  // namespace
 
+// Eight lanes per event in batches under 60 000 events: 10^3 events 31 -> 16
+// us, 2x10^4 33 -> 23, 4.9x10^4 34 -> 33, but 10^5 42 -> 50 (4 and 16 lanes: 19
+// and 15, 22 and 27, 31 and 42, 47 and 70).
+constexpr int kValidateLanes = 8;
+constexpr int64_t kValidateLanesBelow = 60000;
+
 cudaError_t launch_validate(const DevParams& P, const Events& E, cudaStream_t s, const Ranges& R) {
   if (E.n == 0) return cudaSuccess;
+  if (E.n < kValidateLanesBelow) {
+    constexpr int L = kValidateLanes, kEvents = kValidateThreads / L;
+    return launch_chained(E.n < kChainBelow, k_validate_lanes<L>, (E.n + kEvents - 1) / kEvents, kValidateThreads, 0, s, P,
+                          E, R);
+  }
   const unsigned blocks = static_cast<unsigned>((E.n + kValidateThreads - 1) / kValidateThreads);
   k_validate<<<blocks, kValidateThreads, 0, s>>>(P, E, R);
   return cudaGetLastError();
@@ -489,6 +611,10 @@ cudaError_t launch_validate(const DevParams& P, const Events& E, cudaStream_t s,
 #ifndef GAPS_HIST_BLOCKS_PER_SM
 #define GAPS_HIST_BLOCKS_PER_SM 4
 #endif
+// Batches whose warps take an observable each instead of 32 events: the eight
+// fills of an event then run side by side (10^3 events 35 -> 26 us for the
+// stage, 2x10^4 38 -> 33; 4.9x10^4 41 -> 42, 10^6 165 -> 229).
+constexpr int64_t kHistSplitBelow = 30000;
 
 cudaError_t launch_hist_fixed(const DevParams& P, const DevParams* scale_src, const Events& E, unsigned long long* acc,
                               cudaStream_t s, const Ranges& R) {
@@ -496,14 +622,13 @@ cudaError_t launch_hist_fixed(const DevParams& P, const DevParams* scale_src, co
   int sms = 152;
   int dev = 0;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t want = (E.n + 255) / 256;
   const int64_t most = static_cast<int64_t>(GAPS_HIST_BLOCKS_PER_SM) * sms;
-  if (E.jobs && E.job_of) {
-    k_hist_fixed<true><<<static_cast<unsigned>(want < most ? want : most), 256, 0, s>>>(P, nullptr, E, acc, R);
-  } else {
-    k_hist_fixed<false><<<static_cast<unsigned>(want < most ? want : most), 256, 0, s>>>(P, scale_src, E, acc, R);
-  }
-  return cudaGetLastError();
+  const bool multi = E.jobs && E.job_of, split = E.n < kHistSplitBelow;
+  const int per_block = split ? 32 : 256;
+  const unsigned blocks = static_cast<unsigned>(std::min((E.n + per_block - 1) / per_block, most));
+  auto* kernel = multi ? (split ? k_hist_fixed<true, true> : k_hist_fixed<true, false>)
+                       : (split ? k_hist_fixed<false, true> : k_hist_fixed<false, false>);
+  return launch_chained(E.n < kChainBelow, kernel, blocks, 256, 0, s, P, multi ? nullptr : scale_src, E, acc, R);
 }
 
 cudaError_t launch_hist_finalize(const DevParams& P, const DevParams* scale_src, const DevParams* jobs, int n_sets,
@@ -511,8 +636,7 @@ cudaError_t launch_hist_finalize(const DevParams& P, const DevParams* scale_src,
                                  cudaStream_t s) {
   const int64_t cells = static_cast<int64_t>(n_sets) * kCells;
   const unsigned blocks = static_cast<unsigned>(std::min<int64_t>((cells + 255) / 256, 1024));
-  k_hist_finalize<<<blocks, 256, 0, s>>>(P, scale_src, jobs, n_sets, n_sets_dev, acc, hist);
-  return cudaGetLastError();
+  return launch_chained(true, k_hist_finalize, blocks, 256, 0, s, P, scale_src, jobs, n_sets, n_sets_dev, acc, hist);
 }
 
 cudaError_t launch_histograms(const DevParams& P, const DevParams* scale_src, const Events& E, double* hist,
@@ -542,8 +666,7 @@ cudaError_t launch_stats(const Events& E, gaps_stats* stats, cudaStream_t s) {
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t want = (E.n + 255) / 256;
   const unsigned blocks = static_cast<unsigned>(want < 4 * sms ? want : 4 * sms);
-  k_stats<<<blocks, 256, 0, s>>>(E, stats);
-  return cudaGetLastError();
+  return launch_chained(E.n < kChainBelow, k_stats, blocks, 256, 0, s, E, stats);
 }
 
 }  // namespace gaps
