@@ -269,7 +269,7 @@ __device__ void event_shapes(const DevParams& P0, const Events& E, int64_t ev, i
     const double cosij = dot3(jx[i], jy[i], jz[i], jx[j], jy[j], jz[j]) / (ja[i] * ja[j]);
     return 2.0 * fmin(je[i] * je[i], je[j] * je[j]) * (1.0 - cosij) * P.inv_s;
   };
-  for (int m = n; m > 1; --m) {
+  for (int m = n; m > 2; --m) {  // y of the last two jets is not recorded
     // pass 1: the smallest upper bound of the FP32 distances, and its pair
     float ubest = INFINITY;
     int ui = 0, uj = 1;
@@ -325,8 +325,8 @@ __device__ void event_shapes(const DevParams& P0, const Events& E, int64_t ev, i
         }
       }
     }
-    const int idx = m - 3;
-    if (idx >= 0 && idx < 4) yres[idx] = ymin;
+    if (m <= 6) yres[m - 3] = ymin;
+    if (m == 3) break;
     je[bi] += je[bj];
     jx[bi] += jx[bj];
     jy[bi] += jy[bj];
@@ -631,7 +631,7 @@ __device__ void event_shapes_group(const DevParams& P0, const Events& E, int64_t
     y = fminf(a.fe2[i], a.fe2[j]) * d;
     rel = 4.0e-6f + 1.0e-6f * rsqrtf(fmaxf(d, 1e-30f));
   };
-  for (int m = n; m > 1; --m) {
+  for (int m = n; m > 2; --m) {  // y of the last two jets is not recorded
     // pass 1: the smallest FP32 upper bound, the first pair on ties
     float ubest = INFINITY;
     int up = 0x7fffffff, ui = 0, uj = 1;
@@ -702,8 +702,8 @@ __device__ void event_shapes_group(const DevParams& P0, const Events& E, int64_t
         }
       }
     }
-    const int idx = m - 3;
-    if (idx >= 0 && idx < 4) yres[idx] = ymin;
+    if (m <= 6) yres[m - 3] = ymin;
+    if (m == 3) break;
     __syncwarp(gm);  // every lane is done reading the jets of this merge
     if (sub < 4) {  // a component per lane (L >= 4)
       a.j[sub][bi] += a.j[sub][bj];
@@ -1302,6 +1302,7 @@ __device__ void event_shapes_warp(const DevParams& P0, const Events& E, int64_t 
       bj = __shfl_sync(0xffffffffu, bj, 0);
     }
     if (m <= 6) yres[m - 3] = ymin;
+    if (m == 3) break;
     // jet bi takes the sum, the last jet moves into bj
     const int last = m - 1;
     __syncwarp();  // every lane is done reading the jets of this merge
