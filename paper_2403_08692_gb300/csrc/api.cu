@@ -143,6 +143,13 @@ DevParams make_dev_params(const gaps_params& p, int64_t id_offset) {
   d.as_mz_over_f = static_cast<float>(p.alphas_mz / d.as_over);
   d.as_b0_f = static_cast<float>(p.alphas_mz * d.b0);
   d.ln_mz2_f = static_cast<float>(std::log(kMZ * kMZ));
+  {  // t_C < s / 4: it has phase space (make_dipole's formulas)
+    const double b = std::sqrt(1.0 - 4.0 * p.t_cutoff / d.s), b1 = 1.0 + b;
+    const double ls = log_fp64((b1 * b1) * (d.s * d.inv_4tc));
+    d.start = DipoleRecord{d.s, 0.5 * b1, 1.0 / ls, ls};
+    d.start_x = 1.0f / (d.as2pi_f * static_cast<float>(ls));
+    d.start_y = 1.0f / (d.as2pi_f * 0.5f * static_cast<float>(kTR) * static_cast<float>(b));
+  }
   d.seed_lo = static_cast<uint32_t>(p.seed);
   d.seed_hi = static_cast<uint32_t>(p.seed >> 32);
   for (int r = 0; r < 10; ++r) {

@@ -32,6 +32,13 @@ enum : int { kQtoQG = 0, kGtoGG = 1, kGtoQQ = 2 };
 // A gluon dipole's per-dipole trial won; its kernel is drawn afterwards.
 constexpr int kKindUnchosen = 7;
 
+// FP64 part of a dipole's cache entry (see shower_cycle.cuh): one sector, so
+// that a winner's data comes in one access.  A dipole's record is kept at its
+// colour end (the parton whose side-0 link it is).
+struct alignas(32) DipoleRecord {
+  double q2, zp, inv_ls, ls;  // Q^2, z+, 1/ln(z+/z-), ln(z+/z-)
+};
+
 // Parameters of one launch, derived once on the host from gaps_params.
 struct DevParams {
   double sqrt_s, s, tc;
@@ -52,6 +59,9 @@ struct DevParams {
   double ln_s;                        // ln s, the starting scale of the evolution variable
   double inv_4tc;                     // 1 / (4 t_C)
   double inv_s;                       // 1 / s
+  // the dipole every event starts from (Q^2 = s) and its screen entry
+  DipoleRecord start;
+  float start_x, start_y;
   // event weight n_f 2 dsigma/dcos of flavour f: me_a[f-1] (1 + cos^2) + me_b[f-1] cos
   double me_a[5], me_b[5];
   double inv_as2pi_2cf, inv_as2pi_ca;  // 1 / (alpha_s^over/(2 pi) K) of q->qg and g->gg
@@ -122,13 +132,6 @@ __host__ __device__ inline double fixed128_to_double(unsigned long long lo, unsi
   }
   return (neg ? -mag : mag) * scale_inv;
 }
-
-// FP64 part of a dipole's cache entry (see shower_cycle.cuh): one sector, so
-// that a winner's data comes in one access.  A dipole's record is kept at its
-// colour end (the parton whose side-0 link it is).
-struct alignas(32) DipoleRecord {
-  double q2, zp, inv_ls, ls;  // Q^2, z+, 1/ln(z+/z-), ln(z+/z-)
-};
 
 // Pointers into the workspace (gaps_layout) for one batch.
 struct Events {
@@ -394,12 +397,13 @@ __device__ __forceinline__ double to_unit(uint32_t hi, uint32_t lo) {
 
 struct Uniforms {
   double a, b;
+  uint32_t a_hi;  // the high word of a's
 };
 
 __device__ __forceinline__ Uniforms draw2(const DevParams& P, uint32_t ev, uint32_t step, uint32_t slot,
                                           uint32_t purpose) {
   const U4 r = philox10(ev, step, slot, purpose, P.rk);
-  return Uniforms{to_unit(r.x, r.y), to_unit(r.z, r.w)};
+  return Uniforms{to_unit(r.x, r.y), to_unit(r.z, r.w), r.x};
 }
 
 // FNV-1a, 64 bit, over the eight little-endian bytes of a decision word:

@@ -171,8 +171,8 @@ __device__ __forceinline__ int choose_kernel(const DevParams& P, double zp, doub
   return P.nf;
 }
 
-// The full FP64 SelectWinnerEmission (every trial exact, recomputed from the
-// momenta); the fallback of the FP32 screen.  The log-space scale of trial
+// The full FP64 SelectWinnerEmission (every trial exact, from the dipole
+// records); the fallback of the FP32 screen.  The log-space scale of trial
 // j is L + ln(r_j)/c_j; the highest above ln t_C wins, the first on ties.
 // This form covers partons first, first + stride, ... and keeps, in *best,
 // *code and w, the best of those trials above the incoming *best (the first
@@ -187,12 +187,10 @@ __device__ inline bool select_winner_fp64_range(const DevParams& P, const Events
     const bool gluon = E.flav[E.at(i, ev)] == kGluon;
     const bool combined = gluon && per_dipole<kMode>(P);
     const int nk = gluon && !combined ? 1 + P.nf : 1;
-    const V4 pi = load_p(E, i, ev);
     for (int side = 0; side < 2; ++side) {
       const int k = E.link[E.link_at(side, i, ev)];
-      if (k == kNoLink) continue;
-      const DipoleEntry d = make_dipole(P, 2.0 * mdot(pi, load_p(E, k, ev)));
-      if (d.screen.x < 0.0f) continue;
+      if (k == kNoLink || E.dip[dip_at(E, side, i, ev)].x < 0.0f) continue;
+      const DipoleRecord rec = E.drec[E.at(side == 0 ? i : k, ev)];
       for (int kp = 0; kp < nk; kp += 2) {
         const U4 r = philox_draw<kMode>(P, key, static_cast<uint32_t>(step),
                                         static_cast<uint32_t>((2 * i + side) * 4 + kp / 2), kDrawTrial);
@@ -201,16 +199,16 @@ __device__ inline bool select_winner_fp64_range(const DevParams& P, const Events
           const int kind = combined ? kKindUnchosen : (gluon ? (kappa == 0 ? kGtoGG : kGtoQQ) : kQtoQG);
           const double u = h ? to_unit(r.z, r.w) : to_unit(r.x, r.y);
           const double inv_c =
-              combined ? inv_c_sum_fp64(P, d.rec.zp, d.rec.ls) : inv_c_fp64(P, kind, d.rec.zp, d.rec.inv_ls);
+              combined ? inv_c_sum_fp64(P, rec.zp, rec.ls) : inv_c_fp64(P, kind, rec.zp, rec.inv_ls);
           const double lt = fma(log_fp64(u), inv_c, lnt);
           if (lt > best) {
             best = lt;
             code = (2 * i + side) * 8 + kappa;
             found = true;
             w.lnt = lt;
-            w.q2 = d.rec.q2;
-            w.zp = d.rec.zp;
-            w.ls = d.rec.ls;
+            w.q2 = rec.q2;
+            w.zp = rec.zp;
+            w.ls = rec.ls;
             w.i = i;
             w.k = k;
             w.side = side;

@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(256) k_me(DevParams P0, Events E) {
   fl = fl > P.nf ? P.nf : fl;
   const double cth = 2.0 * r0.b - 1.0;
   double sphi, cphi;
-  sincospi(2.0 * r1.a, &sphi, &cphi);
+  circle_fp64(r1.a, r1.a_hi, &sphi, &cphi);
   const double sth = sqrt(1.0 - cth * cth);
   const double en = 0.5 * P.sqrt_s;
   const V4 q{en, en * sth * cphi, en * sth * sphi, en * cth};
@@ -48,8 +48,8 @@ __global__ void __launch_bounds__(256) k_me(DevParams P0, Events E) {
   E.link[E.link_at(1, 0, ev)] = kNoLink;
   E.link[E.link_at(0, 1, ev)] = kNoLink;
   E.link[E.link_at(1, 1, ev)] = 0;
-  const DipoleEntry d = make_dipole(P, 2.0 * mdot(q, qbar));
-  store_dipole(E, ev, 0, 0, 1, d);
+  // every event starts from the same dipole, Q^2 = s
+  store_dipole(E, ev, 0, 0, 1, DipoleEntry{P.start, make_float2(P.start_x, P.start_y)});
   E.weight[ev] = fma(P.me_a[fl - 1], fma(cth, cth, 1.0), P.me_b[fl - 1] * cth);
   E.me_flavour[ev] = fl;
   E.t[ev] = P.s;  // starting scale t0 = s
