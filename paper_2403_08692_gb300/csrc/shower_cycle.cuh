@@ -285,13 +285,22 @@ static __device__ __noinline__ void finish_early(const Events& E, int64_t ev, in
   finish_event(E, ev, status, exp_fp64(lnt));
 }
 
+// The |key| bound of a trial, h = |key| - m >= 0 with key = log2(u)/c <= 0
+// and m its error allowance: its upper bound, negated, so
+// that positive floats order as their bits.  u >= 2^-53: no denormals.
+__device__ __forceinline__ float trial_bound(uint32_t hi, uint32_t lo, float invc) {
+  float lg;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg) : "f"(unit_float(hi, lo)));
+  return fmaxf(invc * fmaf(-lg, 1.0f - kKeyRelKey, -kKeyRelInvc), 0.0f);
+}
+
 // The FP32 screen of SelectWinnerEmission over the trials of partons
-// first, first + stride, ... of an event: the best key (ties go to the
-// smallest code, i.e. the first trial in the loop order of the exact
-// selection), its error bound, the largest upper bound of every other
-// trial, and the work counts.
+// first, first + stride, ... of an event: the smallest |key| bound (h1) with
+// its 1/c, trial and random words, the smallest bound of every other trial,
+// and the work counts.  Equal smallest bounds leave the cycle undecided, so
+// which trial is kept is immaterial.
 struct Screen {
-  float best_key, best_m, others_hi;
+  float h1, h2, invc;
   int best_code;  // (2 i + side) * 8 + kappa, -1: no trial
   uint32_t best_hi, best_lo;
   uint32_t best_aux;  // the best trial's partner slot (bits 0-7) and gluon splitter (bit 8), as screened
@@ -299,9 +308,8 @@ struct Screen {
 };
 
 __device__ __forceinline__ void screen_none(Screen& sc) {
-  sc.best_key = -INFINITY;
-  sc.best_m = 0.0f;
-  sc.others_hi = -INFINITY;
+  sc.h1 = sc.h2 = INFINITY;
+  sc.invc = 0.0f;
   sc.best_code = -1;
   sc.best_hi = sc.best_lo = 0;
   sc.best_aux = 0;
@@ -359,22 +367,18 @@ __device__ __forceinline__ void screen_partons(const DevParams& P, const Events&
           const int kappa = kp + h;
           if (kappa >= nk) break;
           const uint32_t whi = h ? r.z : r.x, wlo = h ? r.w : r.y;
-          const float lg2u = __log2f(unit_float(whi, wlo));
           const float invc = combined ? inv_sum : (!gluon ? d.x * kInvCF2 : (kappa == 0 ? d.x * kInvCA : d.y));
-          const float key = lg2u * invc;
-          const float m = fmaf(kKeyRelKey, fabsf(key), kKeyRelInvc * invc);
+          const float bound = trial_bound(whi, wlo, invc);
           ++sc.trials;
-          if (key > sc.best_key) {
-            sc.others_hi = fmaxf(sc.others_hi, sc.best_key + sc.best_m);
-            sc.best_key = key;
-            sc.best_m = m;
-            sc.best_code = (2 * i + side) * 8 + kappa;
-            sc.best_hi = whi;
-            sc.best_lo = wlo;
-            sc.best_aux = static_cast<uint32_t>(side ? cur.link1 : cur.link0) | (gluon ? 256u : 0u);
-          } else {
-            sc.others_hi = fmaxf(sc.others_hi, key + m);
-          }
+          const bool first_now = bound < sc.h1;
+          sc.h2 = fminf(sc.h2, fmaxf(sc.h1, bound));
+          sc.h1 = fminf(sc.h1, bound);
+          sc.invc = first_now ? invc : sc.invc;
+          sc.best_code = first_now ? (2 * i + side) * 8 + kappa : sc.best_code;
+          sc.best_hi = first_now ? whi : sc.best_hi;
+          sc.best_lo = first_now ? wlo : sc.best_lo;
+          sc.best_aux =
+              first_now ? static_cast<uint32_t>(side ? cur.link1 : cur.link0) | (gluon ? 256u : 0u) : sc.best_aux;
         }
       }
     }
@@ -382,18 +386,13 @@ __device__ __forceinline__ void screen_partons(const DevParams& P, const Events&
   }
 }
 
-// Merge the screen of other trials into sc: the same result as one screen
-// over both sets in loop order (commutative and associative, so a butterfly
-// over lanes gives every lane the whole event's screen).
+// Merge the screen of other trials into sc.
 __device__ __forceinline__ void screen_merge(Screen& sc, const Screen& o) {
-  const bool o_wins = o.best_code >= 0 &&
-                      (sc.best_code < 0 || o.best_key > sc.best_key ||
-                       (o.best_key == sc.best_key && o.best_code < sc.best_code));
-  const float lose = o_wins ? sc.best_key + sc.best_m : o.best_key + o.best_m;
-  sc.others_hi = fmaxf(fmaxf(sc.others_hi, o.others_hi), lose);
+  const bool o_wins = o.h1 < sc.h1;
+  sc.h2 = fminf(fminf(sc.h2, o.h2), fmaxf(sc.h1, o.h1));
   if (o_wins) {
-    sc.best_key = o.best_key;
-    sc.best_m = o.best_m;
+    sc.h1 = o.h1;
+    sc.invc = o.invc;
     sc.best_code = o.best_code;
     sc.best_hi = o.best_hi;
     sc.best_lo = o.best_lo;
@@ -410,9 +409,9 @@ __device__ __forceinline__ void screen_group_reduce(Screen& sc) {
 #pragma unroll
   for (int off = 1; off < L; off <<= 1) {
     Screen o;
-    o.best_key = __shfl_xor_sync(0xffffffffu, sc.best_key, off);
-    o.best_m = __shfl_xor_sync(0xffffffffu, sc.best_m, off);
-    o.others_hi = __shfl_xor_sync(0xffffffffu, sc.others_hi, off);
+    o.h1 = __shfl_xor_sync(0xffffffffu, sc.h1, off);
+    o.h2 = __shfl_xor_sync(0xffffffffu, sc.h2, off);
+    o.invc = __shfl_xor_sync(0xffffffffu, sc.invc, off);
     o.best_code = __shfl_xor_sync(0xffffffffu, sc.best_code, off);
     o.best_hi = __shfl_xor_sync(0xffffffffu, sc.best_hi, off);
     o.best_lo = __shfl_xor_sync(0xffffffffu, sc.best_lo, off);
@@ -430,13 +429,16 @@ enum : int { kScreenNone = 0, kScreenWinner = 1, kScreenUndecided = 2 };
 
 // The screen's verdict; for a certain winner its exact scale (from the FP64
 // cache) and the winner's data in `task`.  Writes nothing to the record.
-// best_ub, best_lb: bounds of the best trial's key; others_hi: the largest
-// upper bound of the others'; best_code < 0: no trial.
+// h1, invc: the smallest |key| bound and its trial's 1/c; h2: the smallest
+// bound of the other trials; best_code < 0: no trial.
 template <int kMode>
-__device__ __forceinline__ int screen_verdict(const DevParams& P, const Events& E, int64_t ev, double lnt, float best_ub,
-                                              float best_lb, float others_hi, int best_code, uint32_t best_aux,
-                                              uint32_t best_hi, uint32_t best_lo, EmitTask& task) {
-
+__device__ __forceinline__ int screen_verdict(const DevParams& P, const Events& E, int64_t ev, double lnt, float h1,
+                                              float h2, float invc, int best_code, uint32_t best_aux, uint32_t best_hi,
+                                              uint32_t best_lo, EmitTask& task) {
+  // the best trial's key bounds -- |key| - m = h1 and, from it, |key| + m --
+  // and the others' upper bound
+  const float best_ub = -h1, best_lb = -(fmaf(2.0f * kKeyRelInvc, invc, h1) * (1.0f + 2.1f * kKeyRelKey));
+  const float others_hi = -h2;
   // Cutoff threshold in key units: t' > t_C  <=>  key > log2(t_C / t).
   const float lt2 = f32_from_f64(lnt) * 1.44269504f;
   const float thr = P.lg2_tc_f - lt2;
@@ -481,8 +483,8 @@ __device__ inline int cycle_screen(const DevParams& P, const Events& E, int64_t 
   E.n_steps[ev] = step + 1;
   E.n_trials[ev] += sc.trials;
   E.n_dipoles[ev] += sc.dipoles;
-  return screen_verdict<kMode>(P, E, ev, lnt, sc.best_key + sc.best_m, sc.best_key - sc.best_m, sc.others_hi,
-                               sc.best_code, sc.best_aux, sc.best_hi, sc.best_lo, task);
+  return screen_verdict<kMode>(P, E, ev, lnt, sc.h1, sc.h2, sc.invc, sc.best_code, sc.best_aux, sc.best_hi, sc.best_lo,
+                               task);
 }
 
 // The exact FP64 selection for the undecided events of a warp, each computed

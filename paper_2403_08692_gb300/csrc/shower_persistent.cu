@@ -169,15 +169,6 @@ __device__ __forceinline__ SideCounts load_dipoles(const DevParams& P0, const Ev
   return mine;
 }
 
-// The |key| bound of a trial, h = |key| - m >= 0 with key = log2(u)/c <= 0
-// and m its error allowance (shower_cycle.cuh): its upper bound, negated, so
-// that positive floats order as their bits.  u >= 2^-53: no denormals.
-__device__ __forceinline__ float trial_bound(uint32_t hi, uint32_t lo, float invc) {
-  float lg;
-  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg) : "f"(unit_float(hi, lo)));
-  return fmaxf(invc * fmaf(-lg, 1.0f - kKeyRelKey, -kKeyRelInvc), 0.0f);
-}
-
 // The screens of the warp's events, slot q on each lane (q < 0: none): every
 // trial of every event, 32 splitters at a time.  The splitters of the warp's
 // events lie one after another (a scan over the lanes' counts), first the
@@ -338,20 +329,6 @@ __device__ __forceinline__ void screen_warp(const DevParams& P0, const DevParams
     }
     __syncwarp();
   }
-}
-
-// The verdict of the calling lane's screen, from screen_warp's results: its
-// best trial's bounds are |key| - m = h1 and, from it, |key| + m.
-template <int kMode>
-__device__ __forceinline__ int screen_verdict(const DevParams& P, const Events& E, int64_t ev, double lnt,
-                                              const ScreenResults& r, EmitTask& task) {
-  const int lane = static_cast<int>(threadIdx.x & 31);
-  const uint32_t best = r.best[lane], code = r.code[lane];
-  const float h1 = __uint_as_float(best), invc = r.invc[lane];
-  const float most = fmaf(2.0f * kKeyRelInvc, invc, h1) * (1.0f + 2.1f * kKeyRelKey);
-  return screen_verdict<kMode>(P, E, ev, lnt, -h1, -most, -__uint_as_float(r.second[lane]),
-                               best == 0x7f800000u ? -1 : static_cast<int>(code & 4095u), code >> 16, r.hi[lane],
-                               r.lo[lane], task);
 }
 
 // Slot states of a pool: empty, live, live with an emission waiting, live
@@ -695,7 +672,10 @@ __global__ void __launch_bounds__(kMaxThreads)
       EmitTask task;
       if (lead) {
         lnt = w.lnt[q];
-        verdict = screen_verdict<kMode>(P, E, ev, lnt, w.r, task);
+        const uint32_t best = w.r.best[lane], code = w.r.code[lane];
+        verdict = screen_verdict<kMode>(P, E, ev, lnt, __uint_as_float(best), __uint_as_float(w.r.second[lane]),
+                                        w.r.invc[lane], best == 0x7f800000u ? -1 : static_cast<int>(code & 4095u),
+                                        code >> 16, w.r.hi[lane], w.r.lo[lane], task);
         if (verdict == kScreenUndecided) atomicAdd(&E.counters[2], 1ull);  // full FP64 cycle
       }
       bool have = verdict == kScreenWinner;
