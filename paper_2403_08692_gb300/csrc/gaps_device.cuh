@@ -518,6 +518,63 @@ __device__ __forceinline__ void dipole_map(const V4& a, const V4& b, double z, d
   pb = V4{r * b.e, r * b.x, r * b.y, r * b.z};
 }
 
+// Component c of a four-vector: 0 the energy, 1 to 3 x, y and z.
+__device__ __forceinline__ double component(const V4& v, int c) {
+  return c == 0 ? v.e : (c == 1 ? v.x : (c == 2 ? v.y : v.z));
+}
+// The four-vector of the components that the aligned group of four lanes
+// holds, lane c component c.
+__device__ __forceinline__ V4 gather4(double v) {
+  return V4{__shfl_sync(0xffffffffu, v, 0, 4), __shfl_sync(0xffffffffu, v, 1, 4), __shfl_sync(0xffffffffu, v, 2, 4),
+            __shfl_sync(0xffffffffu, v, 3, 4)};
+}
+
+// The transverse vectors of dipole_map by four lanes, lane c with component c
+// of n1 and n2 (the same operations on the same operands, so the same bits),
+// and in inv 1/|n1| (lanes 0 and 1) and 1/|n2| (lanes 2 and 3).  The vector
+// expressions take a quarter of the one-lane form's instructions, the
+// invariant products the same.  Every lane of the warp must call it.
+__device__ __forceinline__ void dipole_frame4(const V4& a, const V4& b, int c, double& n1c, double& n2c, double& inv) {
+  const double ab = mdot(a, b);
+  const long long lim = __double_as_longlong(1e-4 * ab * ab);
+  const double ac = component(a, c), bc = component(b, c);
+  V4 n1{0, 0, 0, 0};
+  double n1sq = 0.0;
+  n1c = 0.0;
+  bool found = false;
+#pragma unroll 1
+  for (int r = 0; r < 3; ++r) {
+    const double cb = b.e - (r == 0 ? b.x : (r == 1 ? b.y : b.z));
+    const double ca = a.e - (r == 0 ? a.x : (r == 1 ? a.y : a.z));
+    const double vc = fma(-ca, bc, fma(-cb, ac, c == 0 || c == r + 1 ? ab : 0.0));
+    const V4 v = gather4(vc);
+    if (!found) {  // the group's first reference that serves, or the last one
+      n1c = vc;
+      n1 = v;
+      n1sq = mdot(v, v);
+      found = (__double_as_longlong(n1sq) & 0x7fffffffffffffffll) >= lim;
+    }
+    if (__all_sync(0xffffffffu, found)) break;
+  }
+  // the minors (b, n1)_uv = b_u n1_v - b_v n1_u: m0 of lanes 0 to 3 is
+  // yz, xz, xy, ez, m1 of lanes 0 and 1 is ey, ex
+  const double bu = c == 0 ? b.y : (c == 3 ? b.e : b.x), nu = c == 0 ? n1.y : (c == 3 ? n1.e : n1.x);
+  const double bv = c == 2 ? b.y : b.z, nv = c == 2 ? n1.y : n1.z;
+  const double m0 = fma(bu, nv, -(bv * nu));
+  const double bw = c == 0 ? b.y : b.x, nw = c == 0 ? n1.y : n1.x;
+  const double m1 = fma(b.e, nw, -(bw * n1.e));
+  const double x0 = __shfl_sync(0xffffffffu, m0, c == 0 ? 0 : c - 1, 4);  // yz, yz, xz, xy
+  const double y0 = __shfl_sync(0xffffffffu, m0, c == 0 ? 1 : 3, 4);      // xz, ez, ez, -
+  const double y1 = __shfl_sync(0xffffffffu, m1, 0, 4);                   // -, -, -, ey
+  const double z0 = __shfl_sync(0xffffffffu, m0, 2, 4);                   // xy, -, -, -
+  const double z1 = __shfl_sync(0xffffffffu, m1, c == 1 ? 0 : 1, 4);      // -, ey, ex, ex
+  n2c = fma(c == 3 ? a.y : a.z, c == 0 ? z0 : z1,
+            fma(-(c < 2 ? a.y : a.x), c == 3 ? y1 : y0, (c == 0 ? a.x : a.e) * x0));
+  if (c == 2) n2c = -n2c;
+  const V4 n2 = gather4(n2c);
+  inv = rsqrt_fp64(c < 2 ? -n1sq : -mdot(n2, n2));
+}
+
 // d sigma / d cos(theta) for e+e- -> q qbar (flavour f, PDG 1..5) at LO with
 // photon and Z exchange and their interference, in pb; theta is the quark's
 // angle to the electron beam.  It is a (1 + cos^2) + b cos: dsigma_parts gives

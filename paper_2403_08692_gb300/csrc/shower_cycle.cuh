@@ -681,41 +681,36 @@ __device__ inline int cycle_select_veto(const DevParams& P0, const Events& E, in
   return cycle_decide<kMode>(P, E, ev, key, step, n, lnt, sc, task);
 }
 
-// Phase 2: GenerateEmission -- azimuth, the final-final dipole map, colours
-// and the new parton in slot n.  The dipoles whose invariant mass moved are
-// put in the block's refresh list (reserve(count) gives their first place,
-// put(place, job) writes one) under task_index; the caller recomputes them
-// after a block barrier, spread over all of its threads, so that this
-// FP64-heavy step runs in full warps.
-template <int kMode, class Reserve, class Put>
-__device__ inline void cycle_emit(const DevParams& P0, const Events& E, const EmitTask& w, Reserve reserve, Put put,
-                                  int task_index) {
-  const int64_t ev = w.ev;
-  const int job = kJobKey<kMode> ? static_cast<int>(E.job_of[ev]) : 0;
-  const DevParams& P = job_params<kJobPhysics<kMode>>(P0, E, job);
-  const EventKey key = event_key<kMode>(P, E, ev, job);
+// The splitting variables of an accepted emission: z, y and the azimuth's
+// sine and cosine.
+struct Splitting {
+  double z, y, sphi, cphi;
+};
+template <int kMode>
+__device__ __forceinline__ Splitting splitting_of(const DevParams& P, const EventKey& key, const EmitTask& w) {
+  Splitting v;
   const double t = exp_fp64(w.lnt);
-  const double z = z_fp64(w.kind, w.zp, w.ls, to_unit(w.rz_hi, w.rz_lo));
-  const double y = div_fp64(t, w.q2 * z * (1.0 - z));
+  v.z = z_fp64(w.kind, w.zp, w.ls, to_unit(w.rz_hi, w.rz_lo));
+  v.y = div_fp64(t, w.q2 * v.z * (1.0 - v.z));
   const U4 rphi = philox_draw<kMode>(P, key, static_cast<uint32_t>(w.step), 1u, kDrawWinner);
-  double sphi, cphi;
-  circle_fp64(to_unit(rphi.x, rphi.y), rphi.x, &sphi, &cphi);
+  circle_fp64(to_unit(rphi.x, rphi.y), rphi.x, &v.sphi, &v.cphi);
+  return v;
+}
+
+// Colours, links and flavours of an emission, its refresh list and counts.
+// oi, ok: the partners of the splitter and of the spectator outside their
+// dipole (the colour chain is open, so i, j, k and these are distinct).
+//
+// A gluon enters the shared colour line between splitter and spectator: on
+// side `s` it takes the splitter's line and on the other a new line m, the
+// splitter takes m on side s.  g(c, a) -> q(c, 0) + qbar(0, a) is the same on
+// the anticolour side with no line m: the antiquark connects to the holder of
+// colour a, and not to the quark.
+template <class Reserve, class Put>
+__device__ __forceinline__ void emit_colours(const Events& E, const EmitTask& w, int oi, int ok, Reserve reserve,
+                                             Put put, int task_index) {
+  const int64_t ev = w.ev;
   const int i = w.i, j = w.n, k = w.k, side = w.side;
-  const V4 a = load_p(E, i, ev);
-  const V4 b = load_p(E, k, ev);
-  // the partners of the splitter and of the spectator outside their dipole
-  // (the colour chain is open, so i, j, k and these are distinct)
-  const int oi = E.link[E.link_at(1 - side, i, ev)], ok = E.link[E.link_at(side, k, ev)];
-  V4 pi, pj, pb;
-  dipole_map(a, b, z, y, cphi, sphi, pi, pj, pb);
-  store_p(E, i, ev, pi);
-  store_p(E, j, ev, pj);
-  store_p(E, k, ev, pb);
-  // Colours.  A gluon enters the shared colour line between splitter and
-  // spectator: on side `s` it takes the splitter's line and on the other a
-  // new line m, the splitter takes m on side s.  g(c, a) -> q(c, 0) +
-  // qbar(0, a) is the same on the anticolour side with no line m: the
-  // antiquark connects to the holder of colour a, and not to the quark.
   const bool split = w.kind == kGtoQQ;
   const int s = split ? 1 : side;
   const int to = split && side == 0 ? oi : k;  // j's partner on side s
@@ -747,6 +742,88 @@ __device__ inline void cycle_emit(const DevParams& P0, const Events& E, const Em
   if (ok != kNoLink) put(at++, pack_refresh(task_index, k, side, ok));
   E.n_partons[ev] = j + 1;
   E.n_emissions[ev] += 1;
+}
+
+// Phase 2: GenerateEmission -- azimuth, the final-final dipole map, colours
+// and the new parton in slot n.  The dipoles whose invariant mass moved are
+// put in the block's refresh list (reserve(count) gives their first place,
+// put(place, job) writes one) under task_index; the caller recomputes them
+// after a block barrier, spread over all of its threads, so that this
+// FP64-heavy step runs in full warps.
+template <int kMode, class Reserve, class Put>
+__device__ inline void cycle_emit(const DevParams& P0, const Events& E, const EmitTask& w, Reserve reserve, Put put,
+                                  int task_index) {
+  const int64_t ev = w.ev;
+  const int job = kJobKey<kMode> ? static_cast<int>(E.job_of[ev]) : 0;
+  const DevParams& P = job_params<kJobPhysics<kMode>>(P0, E, job);
+  const Splitting v = splitting_of<kMode>(P, event_key<kMode>(P, E, ev, job), w);
+  const int i = w.i, j = w.n, k = w.k, side = w.side;
+  const V4 a = load_p(E, i, ev);
+  const V4 b = load_p(E, k, ev);
+  const int oi = E.link[E.link_at(1 - side, i, ev)], ok = E.link[E.link_at(side, k, ev)];
+  V4 pi, pj, pb;
+  dipole_map(a, b, v.z, v.y, v.cphi, v.sphi, pi, pj, pb);
+  store_p(E, i, ev, pi);
+  store_p(E, j, ev, pj);
+  store_p(E, k, ev, pb);
+  emit_colours(E, w, oi, ok, reserve, put, task_index);
+}
+
+// What the two warps of emit_shared exchange about one task.
+struct SharedSplitting {
+  double z, y, kt, trig[2];  // trig: cosine, sine of the azimuth
+};
+
+// GenerateEmission for up to 8 tasks by two warps of a block, four lanes a
+// task (lane c of a group: momentum component c), for lists too short to fill
+// warps with a task per thread.  A warp issues an FP64 instruction every 64
+// cycles whatever its active lanes, so a short list waits for the number of
+// them on its chain: 159 for a task in one lane.  Here the first warp forms
+// the frame (dipole_frame4) while the second forms the splitting variables,
+// and the first the momenta while the second does the colours: about 60.
+// Plain shower 10^3 events 1.03 -> 0.87 ms, 1.2x10^4 (200 GeV) 3.65 -> 3.38,
+// 10^5 2.63 -> 2.47; taken for lists of up to 16 tasks a block it measured
+// the same, up to 32 it slows 10^5 events to 2.70 ms.
+// Each value comes from the operations of cycle_emit in their order, so the
+// events are the same.  tasks[0 .. count), count > 0; splits: shared memory.
+// The first 64 threads of the block call it, with a barrier of theirs alone
+// or of the block in `sync`.
+template <int kMode, class Reserve, class Put, class Sync>
+__device__ inline void emit_shared(const DevParams& P0, const Events& E, const EmitTask* tasks, int count,
+                                   SharedSplitting* splits, int tid, Reserve reserve, Put put, Sync sync) {
+  const int g = (tid & 31) >> 2, c = tid & 3, index = min(g, count - 1);
+  const bool has = g < count;
+  const EmitTask& w = tasks[index];
+  const int64_t ev = w.ev;
+  const int i = w.i, j = w.n, k = w.k, side = w.side;
+  const V4 a = load_p(E, i, ev);
+  const V4 b = load_p(E, k, ev);
+  if (tid < 32) {
+    double n1c, n2c, inv;
+    dipole_frame4(a, b, c, n1c, n2c, inv);
+    sync();
+    const SharedSplitting v = splits[index];
+    const double kk = v.kt * v.trig[c >> 1] * inv;
+    const double kc = __shfl_sync(0xffffffffu, kk, 0, 4), ks = __shfl_sync(0xffffffffu, kk, 2, 4);
+    const double q = fma(ks, n2c, kc * n1c);
+    const double ac = component(a, c), bc = component(b, c);
+    const double fa_j = 1.0 - v.z, fb_i = fa_j * v.y, fb_j = v.z * v.y;
+    double* out = c == 0 ? E.e : (c == 1 ? E.px : (c == 2 ? E.py : E.pz));
+    if (has) {
+      out[E.at(i, ev)] = fma(fb_i, bc, fma(v.z, ac, q));
+      out[E.at(j, ev)] = fma(fb_j, bc, fma(fa_j, ac, -q));
+      out[E.at(k, ev)] = (1.0 - v.y) * bc;
+    }
+  } else {
+    const int job = kJobKey<kMode> ? static_cast<int>(E.job_of[ev]) : 0;
+    const DevParams& P = job_params<kJobPhysics<kMode>>(P0, E, job);
+    const int oi = E.link[E.link_at(1 - side, i, ev)], ok = E.link[E.link_at(side, k, ev)];
+    const Splitting v = splitting_of<kMode>(P, event_key<kMode>(P, E, ev, job), w);
+    const double kt = sqrt_fp64(v.z * (1.0 - v.z) * v.y * (2.0 * mdot(a, b)));
+    if (has && c == 0) splits[g] = SharedSplitting{v.z, v.y, kt, {v.cphi, v.sphi}};
+    sync();
+    if (has && c == 0) emit_colours(E, w, oi, ok, reserve, put, g);
+  }
 }
 
 // One dipole of the refresh list.

@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(256) k_me(DevParams P0, Events E) {
 // dipoles took several rounds of one block (4 and 16 measured the same as 8).
 constexpr int kEmitChunk = 8;
 constexpr int kStepThreads = GAPS_STEP_THREADS;
-
+static_assert(kStepThreads == 64 && kEmitChunk == 8, "emit_shared: two warps, four lanes a task");
 
 // One veto cycle over the events list_in[0 .. n_in): the list holds the
 // active events only (the previous launch wrote it), so every thread of a
@@ -290,6 +290,7 @@ __global__ void __launch_bounds__(kStepThreads, GAPS_STEP_MIN_BLOCKS)
                     unsigned long long* reset_cursor, StepPublish pub) {
   __shared__ EmitTask s_task[kStepThreads];
   __shared__ uint32_t s_jobs[kMaxRefresh * kStepThreads];
+  __shared__ SharedSplitting s_split[kEmitChunk];
   __shared__ int s_njobs;
   __shared__ unsigned long long s_base;
   const int tid = threadIdx.x;
@@ -317,7 +318,8 @@ __global__ void __launch_bounds__(kStepThreads, GAPS_STEP_MIN_BLOCKS)
   }
   const int64_t len = n_tasks_dev ? min(n_tasks, static_cast<int64_t>(*n_tasks_dev)) : n_tasks;
   // Tasks a block takes at a time: an even share of a short list, so that the
-  // dipoles they moved fit one round of the block.
+  // dipoles they moved fit one round of the block; up to kEmitChunk by four
+  // lanes each (emit_shared).
   const int chunk = static_cast<int>(
       min(static_cast<int64_t>(kStepThreads), max((len + emit_blocks - 1) / emit_blocks, static_cast<int64_t>(kEmitChunk))));
   for (;;) {
@@ -333,11 +335,15 @@ __global__ void __launch_bounds__(kStepThreads, GAPS_STEP_MIN_BLOCKS)
     const bool has = tid < chunk && k < len;
     if (has) s_task[tid] = tasks_in[k];
     __syncthreads();
-    if (has)
-      cycle_emit<kMode>(P0, E, s_task[tid], [&](int count) { return atomicAdd(&s_njobs, count); },
-                        [&](int at, uint32_t job) { s_jobs[at] = job; }, tid);
+    const auto reserve = [&](int count) { return atomicAdd(&s_njobs, count); };
+    const auto put = [&](int at, uint32_t job) { s_jobs[at] = job; };
+    if (chunk == kEmitChunk)
+      emit_shared<kMode>(P0, E, s_task, static_cast<int>(min(len - base, static_cast<int64_t>(kEmitChunk))), s_split, tid,
+                         reserve, put, [] { __syncthreads(); });
+    else if (has)
+      cycle_emit<kMode>(P0, E, s_task[tid], reserve, put, tid);
     __syncthreads();
-    for (int j = tid; j < s_njobs; j += kStepThreads) 
+    for (int j = tid; j < s_njobs; j += kStepThreads)
       refresh_dipole<kJobPhysics<kMode>>(P0, E, s_task[refresh_task(s_jobs[j])].ev, s_jobs[j]);
     if (has) E.status[s_task[tid].ev] = GAPS_ACTIVE;
     const int64_t at_list = warp_append_slot(has, list_count);
