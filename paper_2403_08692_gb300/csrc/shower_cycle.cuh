@@ -475,14 +475,27 @@ __device__ __forceinline__ int screen_verdict(const DevParams& P, const Events& 
   return kScreenUndecided;
 }
 
+// What a cycle reads of an event's own state, loaded together: a load behind
+// a store to another array is not moved before it, and each would wait for
+// its own trip to L2.
+struct EventState {
+  double lnt;
+  unsigned long long hash;
+  int trials, dipoles, winners;
+};
+__device__ __forceinline__ EventState load_state(const Events& E, int64_t ev) {
+  return EventState{E.lnt[ev], E.hash[ev], E.n_trials[ev], E.n_dipoles[ev], E.n_winners[ev]};
+}
+
 // The first part of the cycle once the screen is known: the cycle and work
 // counts, and the screen's verdict.
 template <int kMode>
-__device__ inline int cycle_screen(const DevParams& P, const Events& E, int64_t ev, int step, double lnt,
+__device__ inline int cycle_screen(const DevParams& P, const Events& E, int64_t ev, int step, const EventState& st,
                                    const Screen& sc, EmitTask& task) {
   E.n_steps[ev] = step + 1;
-  E.n_trials[ev] += sc.trials;
-  E.n_dipoles[ev] += sc.dipoles;
+  E.n_trials[ev] = st.trials + sc.trials;
+  E.n_dipoles[ev] = st.dipoles + sc.dipoles;
+  const double lnt = st.lnt;
   return screen_verdict<kMode>(P, E, ev, lnt, sc.h1, sc.h2, sc.invc, sc.best_code, sc.best_aux, sc.best_hi, sc.best_lo,
                                task);
 }
@@ -627,15 +640,15 @@ __device__ __forceinline__ bool accept_or_veto(const DevParams& P, const Events&
 // generated, kCycleVetoed otherwise.
 template <int kMode>
 __device__ inline int cycle_conclude(const DevParams& P, const Events& E, int64_t ev, const EventKey& key, int step,
-                                     int n, bool have, EmitTask& task) {
+                                     int n, const EventState& st, bool have, EmitTask& task) {
   // ---- CheckCutoff.
   if (!have) {
     finish_event(E, ev, GAPS_DONE, P.tc);
     return kCycleFinished;
   }
   E.lnt[ev] = task.lnt;
-  E.n_winners[ev] += 1;
-  unsigned long long hash = E.hash[ev];
+  E.n_winners[ev] = st.winners + 1;
+  unsigned long long hash = st.hash;
   const bool accept = accept_or_veto<kMode>(P, E, key, step, task, hash);
   E.hash[ev] = hash;
   if (!accept) return kCycleVetoed;
@@ -652,14 +665,14 @@ __device__ inline int cycle_conclude(const DevParams& P, const Events& E, int64_
 // The whole decision of a cycle in one thread, the exact selection serial.
 template <int kMode>
 __device__ inline int cycle_decide(const DevParams& P, const Events& E, int64_t ev, const EventKey& key, int step,
-                                   int n, double lnt, const Screen& sc, EmitTask& task) {
-  const int s = cycle_screen<kMode>(P, E, ev, step, lnt, sc, task);
+                                   int n, const EventState& st, const Screen& sc, EmitTask& task) {
+  const int s = cycle_screen<kMode>(P, E, ev, step, st, sc, task);
   bool have = s == kScreenWinner;
   if (s == kScreenUndecided) {
     atomicAdd(&E.counters[2], 1ull);  // screen undecided: full FP64 cycle
-    have = select_winner_fp64<kMode>(P, E, ev, key, step, n, lnt, task);
+    have = select_winner_fp64<kMode>(P, E, ev, key, step, n, st.lnt, task);
   }
-  return cycle_conclude<kMode>(P, E, ev, key, step, n, have, task);
+  return cycle_conclude<kMode>(P, E, ev, key, step, n, st, have, task);
 }
 
 // Phase 1 of a cycle for active event ev, one thread: SelectWinnerEmission
@@ -671,14 +684,14 @@ __device__ inline int cycle_select_veto(const DevParams& P0, const Events& E, in
   const EventKey key = event_key<kMode>(P, E, ev, job);
   const int n = E.n_partons[ev];
   const int step = E.n_steps[ev];
-  const double lnt = E.lnt[ev];
+  const EventState st = load_state(E, ev);
   if (step >= P.max_steps) {
-    finish_early(E, ev, GAPS_STEP_LIMIT, lnt);
+    finish_early(E, ev, GAPS_STEP_LIMIT, st.lnt);
     return kCycleFinished;
   }
   Screen sc;
   screen_partons<kMode>(P, E, ev, key, step, n, 0, 1, sc);
-  return cycle_decide<kMode>(P, E, ev, key, step, n, lnt, sc, task);
+  return cycle_decide<kMode>(P, E, ev, key, step, n, st, sc, task);
 }
 
 // The splitting variables of an accepted emission: z, y and the azimuth's
@@ -697,9 +710,22 @@ __device__ __forceinline__ Splitting splitting_of(const DevParams& P, const Even
   return v;
 }
 
+// What emit_colours reads of the record: the partners of the splitter and of
+// the spectator outside their dipole (the colour chain is open, so i, j, k
+// and these are distinct), the splitter's colour line on j's side, the next
+// free line and the emissions so far.  Loaded together, ahead of the FP64
+// work, as EventState is.
+struct EmitState {
+  int oi, ok, line, colour, emissions;
+};
+__device__ __forceinline__ EmitState load_emit_state(const Events& E, const EmitTask& w) {
+  const int64_t ev = w.ev;
+  const int s = w.kind == kGtoQQ ? 1 : w.side;
+  return EmitState{E.link[E.link_at(1 - w.side, w.i, ev)], E.link[E.link_at(w.side, w.k, ev)],
+                   (s ? E.acol : E.col)[E.at(w.i, ev)], E.next_colour[ev], E.n_emissions[ev]};
+}
+
 // Colours, links and flavours of an emission, its refresh list and counts.
-// oi, ok: the partners of the splitter and of the spectator outside their
-// dipole (the colour chain is open, so i, j, k and these are distinct).
 //
 // A gluon enters the shared colour line between splitter and spectator: on
 // side `s` it takes the splitter's line and on the other a new line m, the
@@ -707,22 +733,20 @@ __device__ __forceinline__ Splitting splitting_of(const DevParams& P, const Even
 // the anticolour side with no line m: the antiquark connects to the holder of
 // colour a, and not to the quark.
 template <class Reserve, class Put>
-__device__ __forceinline__ void emit_colours(const Events& E, const EmitTask& w, int oi, int ok, Reserve reserve,
-                                             Put put, int task_index) {
+__device__ __forceinline__ void emit_colours(const Events& E, const EmitTask& w, const EmitState& st,
+                                             Reserve reserve, Put put, int task_index) {
   const int64_t ev = w.ev;
   const int i = w.i, j = w.n, k = w.k, side = w.side;
   const bool split = w.kind == kGtoQQ;
   const int s = split ? 1 : side;
+  const int oi = st.oi, ok = st.ok;
   const int to = split && side == 0 ? oi : k;  // j's partner on side s
-  int m = 0;
-  if (!split) {
-    m = E.next_colour[ev];
-    E.next_colour[ev] = m + 1;
-  }
+  const int m = split ? 0 : st.colour;
+  if (!split) E.next_colour[ev] = m + 1;
   const size_t ai = E.at(i, ev), aj = E.at(j, ev);
   int16_t* line = s ? E.acol : E.col;
   int16_t* other = s ? E.col : E.acol;
-  line[aj] = line[ai];
+  line[aj] = static_cast<int16_t>(st.line);
   other[aj] = static_cast<int16_t>(m);
   line[ai] = static_cast<int16_t>(m);
   E.link[E.link_at(s, i, ev)] = split ? kNoLink : static_cast<uint8_t>(j);
@@ -741,7 +765,7 @@ __device__ __forceinline__ void emit_colours(const Events& E, const EmitTask& w,
   if (!split && oi != kNoLink) put(at++, pack_refresh(task_index, i, 1 - side, oi));
   if (ok != kNoLink) put(at++, pack_refresh(task_index, k, side, ok));
   E.n_partons[ev] = j + 1;
-  E.n_emissions[ev] += 1;
+  E.n_emissions[ev] = st.emissions + 1;
 }
 
 // Phase 2: GenerateEmission -- azimuth, the final-final dipole map, colours
@@ -757,16 +781,16 @@ __device__ inline void cycle_emit(const DevParams& P0, const Events& E, const Em
   const int job = kJobKey<kMode> ? static_cast<int>(E.job_of[ev]) : 0;
   const DevParams& P = job_params<kJobPhysics<kMode>>(P0, E, job);
   const Splitting v = splitting_of<kMode>(P, event_key<kMode>(P, E, ev, job), w);
-  const int i = w.i, j = w.n, k = w.k, side = w.side;
+  const int i = w.i, j = w.n, k = w.k;
   const V4 a = load_p(E, i, ev);
   const V4 b = load_p(E, k, ev);
-  const int oi = E.link[E.link_at(1 - side, i, ev)], ok = E.link[E.link_at(side, k, ev)];
+  const EmitState st = load_emit_state(E, w);
   V4 pi, pj, pb;
   dipole_map(a, b, v.z, v.y, v.cphi, v.sphi, pi, pj, pb);
   store_p(E, i, ev, pi);
   store_p(E, j, ev, pj);
   store_p(E, k, ev, pb);
-  emit_colours(E, w, oi, ok, reserve, put, task_index);
+  emit_colours(E, w, st, reserve, put, task_index);
 }
 
 // What the two warps of emit_shared exchange about one task.
@@ -795,7 +819,7 @@ __device__ inline void emit_shared(const DevParams& P0, const Events& E, const E
   const bool has = g < count;
   const EmitTask& w = tasks[index];
   const int64_t ev = w.ev;
-  const int i = w.i, j = w.n, k = w.k, side = w.side;
+  const int i = w.i, j = w.n, k = w.k;
   const V4 a = load_p(E, i, ev);
   const V4 b = load_p(E, k, ev);
   if (tid < 32) {
@@ -817,12 +841,12 @@ __device__ inline void emit_shared(const DevParams& P0, const Events& E, const E
   } else {
     const int job = kJobKey<kMode> ? static_cast<int>(E.job_of[ev]) : 0;
     const DevParams& P = job_params<kJobPhysics<kMode>>(P0, E, job);
-    const int oi = E.link[E.link_at(1 - side, i, ev)], ok = E.link[E.link_at(side, k, ev)];
+    const EmitState st = load_emit_state(E, w);
     const Splitting v = splitting_of<kMode>(P, event_key<kMode>(P, E, ev, job), w);
     const double kt = sqrt_fp64(v.z * (1.0 - v.z) * v.y * (2.0 * mdot(a, b)));
     if (has && c == 0) splits[g] = SharedSplitting{v.z, v.y, kt, {v.cphi, v.sphi}};
     sync();
-    if (has && c == 0) emit_colours(E, w, oi, ok, reserve, put, g);
+    if (has && c == 0) emit_colours(E, w, st, reserve, put, g);
   }
 }
 

@@ -166,6 +166,21 @@ __device__ __forceinline__ int64_t warp_append_slot(bool flag, unsigned long lon
   return flag ? static_cast<int64_t>(base + __popc(mask & ((1u << lane) - 1u))) : -1;
 }
 
+// The same for two lists, an item in at most one: at[0] and at[1], -1 where
+// the item is not in the list.  The two atomics are in flight together.
+__device__ __forceinline__ void warp_append_slots(bool flag0, unsigned long long* count0, bool flag1,
+                                                  unsigned long long* count1, int64_t at[2]) {
+  const unsigned m0 = __ballot_sync(0xffffffffu, flag0), m1 = __ballot_sync(0xffffffffu, flag1);
+  const int lane = threadIdx.x & 31;
+  const unsigned mine = lane == 0 ? m0 : m1;
+  unsigned long long base = 0;
+  if (lane < 2 && mine != 0u) base = atomicAdd(lane == 0 ? count0 : count1, static_cast<unsigned long long>(__popc(mine)));
+  const unsigned long long b0 = __shfl_sync(0xffffffffu, base, 0), b1 = __shfl_sync(0xffffffffu, base, 1);
+  const unsigned below = (1u << lane) - 1u;
+  at[0] = flag0 ? static_cast<int64_t>(b0 + __popc(m0 & below)) : -1;
+  at[1] = flag1 ? static_cast<int64_t>(b1 + __popc(m1 & below)) : -1;
+}
+
 // One step of the plain form with the emissions deferred by one launch.
 // The last select_blocks blocks run SelectWinnerEmission, CheckCutoff and
 // AcceptOrVeto for the events list_in[0 .. n_list) (no list: events
@@ -192,7 +207,8 @@ __device__ __forceinline__ int64_t warp_append_slot(bool flag, unsigned long lon
 // next launch, and publishes its input lengths to the host (pub).
 template <int kMode, int L>
 __device__ __forceinline__ void select_role(const DevParams& P0, const Events& E, int64_t block,
-                                            const int* list_in, int64_t len, int* list_out,
+                                            const int* list_in, int64_t n_list,
+                                            const unsigned long long* n_list_dev, int* list_out,
                                             unsigned long long* list_count, EmitTask* tasks_out,
                                             unsigned long long* task_count) {
   const int tid = threadIdx.x;
@@ -201,8 +217,11 @@ __device__ __forceinline__ void select_role(const DevParams& P0, const Events& E
   // the host sizes the grid for any lanes choice: one pass
   {
     const int64_t idx = block * kGroups + tid / L;
+    // the entry and the list's length are loaded together: entries up to the
+    // bound are readable, those behind the length stale
     int64_t ev = -1;
-    if (idx < len) ev = list_in ? static_cast<int64_t>(list_in[idx]) : idx;
+    if (idx < n_list) ev = list_in ? static_cast<int64_t>(list_in[idx]) : idx;
+    if (n_list_dev && idx >= static_cast<int64_t>(*n_list_dev)) ev = -1;
     // The event's status, size, cycle and (one lane per event) first parton
     // are loaded together, not one after another: every listed event has
     // slot 0.
@@ -229,6 +248,8 @@ __device__ __forceinline__ void select_role(const DevParams& P0, const Events& E
     } else {
       n = step = 0;
     }
+    EventState st{};
+    if (active && sub == 0) st = load_state(E, ev);
     screen_group_reduce<L>(sc);  // every lane of the warp, one call site
     const bool lead = active && sub == 0;
     int r = kCycleFinished;
@@ -236,24 +257,22 @@ __device__ __forceinline__ void select_role(const DevParams& P0, const Events& E
     // The screen's verdict; a cycle it leaves undecided gets the exact FP64
     // selection from the whole warp.
     int verdict = kScreenNone;
-    double lnt = 0.0;
     EventKey key{0u, 0u, 0u};
     if (lead && !limited) {
       const DevParams& P = job_params<kMulti>(P0, E, job);
-      lnt = E.lnt[ev];
       key = event_key<kMode>(P, E, ev, job);
-      verdict = cycle_screen<kMode>(P, E, ev, step, lnt, sc, task);
+      verdict = cycle_screen<kMode>(P, E, ev, step, st, sc, task);
       if (verdict == kScreenUndecided) atomicAdd(&E.counters[2], 1ull);  // full FP64 cycle
     }
     bool have = verdict == kScreenWinner;
     if (__any_sync(0xffffffffu, verdict == kScreenUndecided))
-      fallback_warp<kMode>(P0, E, verdict == kScreenUndecided, ev, job, key, step, n, lnt, have, task);
+      fallback_warp<kMode>(P0, E, verdict == kScreenUndecided, ev, job, key, step, n, st.lnt, have, task);
     if (lead) {
       const DevParams& P = job_params<kMulti>(P0, E, job);
       if (limited) {
-        finish_early(E, ev, GAPS_STEP_LIMIT, E.lnt[ev]);
+        finish_early(E, ev, GAPS_STEP_LIMIT, st.lnt);
       } else {
-        r = cycle_conclude<kMode>(P, E, ev, key, step, n, have, task);
+        r = cycle_conclude<kMode>(P, E, ev, key, step, n, st, have, task);
       }
       if (r == kCycleFinished) {
         atomicAdd(&E.counters[0], 1ull);
@@ -261,13 +280,13 @@ __device__ __forceinline__ void select_role(const DevParams& P0, const Events& E
       }
     }
     count_job_done(E, ev, lead && r == kCycleFinished);
-    const int64_t at_task = warp_append_slot(lead && r == kCycleAccepted, task_count);
-    if (at_task >= 0) {
-      tasks_out[at_task] = task;
+    int64_t at[2];
+    warp_append_slots(lead && r == kCycleAccepted, task_count, lead && r == kCycleVetoed, list_count, at);
+    if (at[0] >= 0) {
+      tasks_out[at[0]] = task;
       E.status[ev] = GAPS_PENDING;
     }
-    const int64_t at_list = warp_append_slot(lead && r == kCycleVetoed, list_count);
-    if (at_list >= 0) list_out[at_list] = static_cast<int>(ev);
+    if (at[1] >= 0) list_out[at[1]] = static_cast<int>(ev);
   }
 }
 
@@ -311,9 +330,8 @@ __global__ void __launch_bounds__(kStepThreads, GAPS_STEP_MIN_BLOCKS)
   }
   const int64_t emit_blocks = static_cast<int64_t>(gridDim.x) - select_blocks;
   if (static_cast<int64_t>(blockIdx.x) >= emit_blocks) {
-    const int64_t len = n_list_dev ? min(n_list, static_cast<int64_t>(*n_list_dev)) : n_list;
-    select_role<kMode, L>(P0, E, static_cast<int64_t>(blockIdx.x) - emit_blocks, list_in, len, list_out, list_count,
-                          tasks_out, task_count);
+    select_role<kMode, L>(P0, E, static_cast<int64_t>(blockIdx.x) - emit_blocks, list_in, n_list, n_list_dev, list_out,
+                          list_count, tasks_out, task_count);
     return;
   }
   const int64_t len = n_tasks_dev ? min(n_tasks, static_cast<int64_t>(*n_tasks_dev)) : n_tasks;
