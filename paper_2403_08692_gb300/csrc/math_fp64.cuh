@@ -137,6 +137,12 @@ __device__ __forceinline__ double expm1_neg_fp64(double x) {
   const ExpParts o = exp_parts(x);
   return (o.t - 1.0) + fma(o.t, o.p, o.t_lo);
 }
+// Either of the two, chosen per lane, by the same instructions.
+__device__ __forceinline__ double exp_or_expm1_fp64(double x, bool minus_one) {
+  if (!exp_range(x)) return minus_one ? expm1_library(x) : exp_library(x);
+  const ExpParts o = exp_parts(x);
+  return (minus_one ? o.t - 1.0 : o.t) + fma(o.t, o.p, o.t_lo);
+}
 
 // Sine and cosine of 2 pi u for the 52-bit uniform u of (hi, lo), u itself
 // given: the nearest k/64 comes from the top bits of hi, u - k/64 is exact,

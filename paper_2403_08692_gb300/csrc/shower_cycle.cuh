@@ -793,58 +793,97 @@ __device__ inline void cycle_emit(const DevParams& P0, const Events& E, const Em
   emit_colours(E, w, st, reserve, put, task_index);
 }
 
-// What the two warps of emit_shared exchange about one task.
-struct SharedSplitting {
-  double z, y, kt, trig[2];  // trig: cosine, sine of the azimuth
+// GenerateEmission by four lanes a task, lane c of a group with momentum
+// component c, for lists too short to fill warps with a task per thread.  A
+// warp issues an FP64 instruction every 64 cycles whatever its active lanes,
+// so a short list waits for the number of them on its chain: 159 for a task
+// in one lane.  Four lanes take about 90, and about 60 where one warp forms
+// the frame and the momenta and another the splitting variables and the
+// colours.  Each value comes from the operations of cycle_emit in their
+// order, so the events are the same.  Every lane of a warp calls these, the
+// lanes of groups without a task with another's and has = false.
+//
+// The splitting variables, on every lane of the group: splitting_of with the
+// two exponentials on two lanes, and kt = sqrt(z (1 - z) y Q^2) of
+// dipole_map.  trig: cosine, sine of the azimuth.
+struct Splitting4 {
+  double z, y, kt, trig[2];
 };
+template <int kMode>
+__device__ __forceinline__ Splitting4 splitting_of4(const DevParams& P, const EventKey& key, const EmitTask& w,
+                                                    const V4& a, const V4& b, int c) {
+  Splitting4 v;
+  const double r = to_unit(w.rz_hi, w.rz_lo);
+  const double ex = exp_or_expm1_fp64(c == 0 ? w.lnt : -r * w.ls, c != 0);
+  const double t = __shfl_sync(0xffffffffu, ex, 0, 4), em = __shfl_sync(0xffffffffu, ex, 1, 4);
+  const double zm = 1.0 - w.zp;
+  const bool split = w.kind == kGtoQQ;  // as z_fp64
+  v.z = fma(split ? w.zp - zm : -w.zp, split ? r : em, zm);
+  v.y = div_fp64(t, w.q2 * v.z * (1.0 - v.z));
+  const U4 rphi = philox_draw<kMode>(P, key, static_cast<uint32_t>(w.step), 1u, kDrawWinner);
+  circle_fp64(to_unit(rphi.x, rphi.y), rphi.x, &v.trig[1], &v.trig[0]);
+  v.kt = sqrt_fp64(v.z * (1.0 - v.z) * v.y * (2.0 * mdot(a, b)));
+  return v;
+}
 
-// GenerateEmission for up to 8 tasks by two warps of a block, four lanes a
-// task (lane c of a group: momentum component c), for lists too short to fill
-// warps with a task per thread.  A warp issues an FP64 instruction every 64
-// cycles whatever its active lanes, so a short list waits for the number of
-// them on its chain: 159 for a task in one lane.  Here the first warp forms
-// the frame (dipole_frame4) while the second forms the splitting variables,
-// and the first the momenta while the second does the colours: about 60.
-// Plain shower 10^3 events 1.03 -> 0.87 ms, 1.2x10^4 (200 GeV) 3.65 -> 3.38,
-// 10^5 2.63 -> 2.47; taken for lists of up to 16 tasks a block it measured
-// the same, up to 32 it slows 10^5 events to 2.70 ms.
-// Each value comes from the operations of cycle_emit in their order, so the
-// events are the same.  tasks[0 .. count), count > 0; splits: shared memory.
-// The first 64 threads of the block call it, with a barrier of theirs alone
-// or of the block in `sync`.
+// The momenta from the frame (dipole_frame4) and the splitting variables.
+__device__ __forceinline__ void emit_momenta4(const Events& E, const EmitTask& w, const V4& a, const V4& b, int c,
+                                              double n1c, double n2c, double inv, const Splitting4& v, bool has) {
+  const double kk = v.kt * v.trig[c >> 1] * inv;
+  const double kc = __shfl_sync(0xffffffffu, kk, 0, 4), ks = __shfl_sync(0xffffffffu, kk, 2, 4);
+  const double q = fma(ks, n2c, kc * n1c);
+  const double ac = component(a, c), bc = component(b, c);
+  const double fa_j = 1.0 - v.z, fb_i = fa_j * v.y, fb_j = v.z * v.y;
+  double* out = c == 0 ? E.e : (c == 1 ? E.px : (c == 2 ? E.py : E.pz));
+  if (!has) return;
+  out[E.at(w.i, w.ev)] = fma(fb_i, bc, fma(v.z, ac, q));
+  out[E.at(w.n, w.ev)] = fma(fb_j, bc, fma(fa_j, ac, -q));
+  out[E.at(w.k, w.ev)] = (1.0 - v.y) * bc;
+}
+
+// One warp, up to 8 tasks: w is the task of the calling lane's group.
+template <int kMode, class Reserve, class Put>
+__device__ inline void emit_warp4(const DevParams& P0, const Events& E, const EmitTask& w, bool has, Reserve reserve,
+                                  Put put, int task_index) {
+  const int c = static_cast<int>(threadIdx.x & 3);
+  const int64_t ev = w.ev;
+  const int job = kJobKey<kMode> ? static_cast<int>(E.job_of[ev]) : 0;
+  const DevParams& P = job_params<kJobPhysics<kMode>>(P0, E, job);
+  const V4 a = load_p(E, w.i, ev);
+  const V4 b = load_p(E, w.k, ev);
+  const EmitState st = load_emit_state(E, w);
+  double n1c, n2c, inv;
+  dipole_frame4(a, b, c, n1c, n2c, inv);
+  const Splitting4 v = splitting_of4<kMode>(P, event_key<kMode>(P, E, ev, job), w, a, b, c);
+  emit_momenta4(E, w, a, b, c, n1c, n2c, inv, v, has);
+  if (has && c == 0) emit_colours(E, w, st, reserve, put, task_index);
+}
+
+// Two warps (the first 64 threads of a block, with `sync` a barrier), up to 8
+// tasks: tasks[0 .. count), count > 0; splits: shared memory.  Plain shower
+// 10^3 events 1.03 -> 0.87 ms against a task per lane, 1.2x10^4 (200 GeV)
+// 3.65 -> 3.38, 10^5 2.63 -> 2.47; taken for lists of up to 16 tasks a block
+// it measured the same, up to 32 it slows 10^5 events to 2.70 ms.
 template <int kMode, class Reserve, class Put, class Sync>
 __device__ inline void emit_shared(const DevParams& P0, const Events& E, const EmitTask* tasks, int count,
-                                   SharedSplitting* splits, int tid, Reserve reserve, Put put, Sync sync) {
+                                   Splitting4* splits, int tid, Reserve reserve, Put put, Sync sync) {
   const int g = (tid & 31) >> 2, c = tid & 3, index = min(g, count - 1);
   const bool has = g < count;
   const EmitTask& w = tasks[index];
   const int64_t ev = w.ev;
-  const int i = w.i, j = w.n, k = w.k;
-  const V4 a = load_p(E, i, ev);
-  const V4 b = load_p(E, k, ev);
+  const V4 a = load_p(E, w.i, ev);
+  const V4 b = load_p(E, w.k, ev);
   if (tid < 32) {
     double n1c, n2c, inv;
     dipole_frame4(a, b, c, n1c, n2c, inv);
     sync();
-    const SharedSplitting v = splits[index];
-    const double kk = v.kt * v.trig[c >> 1] * inv;
-    const double kc = __shfl_sync(0xffffffffu, kk, 0, 4), ks = __shfl_sync(0xffffffffu, kk, 2, 4);
-    const double q = fma(ks, n2c, kc * n1c);
-    const double ac = component(a, c), bc = component(b, c);
-    const double fa_j = 1.0 - v.z, fb_i = fa_j * v.y, fb_j = v.z * v.y;
-    double* out = c == 0 ? E.e : (c == 1 ? E.px : (c == 2 ? E.py : E.pz));
-    if (has) {
-      out[E.at(i, ev)] = fma(fb_i, bc, fma(v.z, ac, q));
-      out[E.at(j, ev)] = fma(fb_j, bc, fma(fa_j, ac, -q));
-      out[E.at(k, ev)] = (1.0 - v.y) * bc;
-    }
+    emit_momenta4(E, w, a, b, c, n1c, n2c, inv, splits[index], has);
   } else {
     const int job = kJobKey<kMode> ? static_cast<int>(E.job_of[ev]) : 0;
     const DevParams& P = job_params<kJobPhysics<kMode>>(P0, E, job);
     const EmitState st = load_emit_state(E, w);
-    const Splitting v = splitting_of<kMode>(P, event_key<kMode>(P, E, ev, job), w);
-    const double kt = sqrt_fp64(v.z * (1.0 - v.z) * v.y * (2.0 * mdot(a, b)));
-    if (has && c == 0) splits[g] = SharedSplitting{v.z, v.y, kt, {v.cphi, v.sphi}};
+    const Splitting4 v = splitting_of4<kMode>(P, event_key<kMode>(P, E, ev, job), w, a, b, c);
+    if (has && c == 0) splits[g] = v;
     sync();
     if (has && c == 0) emit_colours(E, w, st, reserve, put, g);
   }

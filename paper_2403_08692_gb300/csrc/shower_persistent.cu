@@ -550,8 +550,16 @@ __global__ void __launch_bounds__(kMaxThreads)
       if (s1 == kSlotPending && r1 < tasks)
         pools[r1 >> 5].m.tasks[r1 & 31] = static_cast<uint16_t>(warp * kSlots + lane + 32);
       __syncthreads();
-      if (tid < tasks) {
-        const int task = w.m.tasks[lane], q = task & (kSlots - 1);
+#ifndef G_QUADS
+#define G_QUADS 4
+#endif
+      const bool quads = tasks <= 8 * min(n_warps, G_QUADS);
+      // the task of this lane, or the last one on the lanes left over
+      const int at_task = quads ? tid >> 2 : tid;
+      const bool has = at_task < tasks;
+      if (quads ? warp * 8 < tasks : has) {
+        const int r = min(at_task, tasks - 1);
+        const int task = pools[r >> 5].m.tasks[r & 31], q = task & (kSlots - 1);
         WarpPool& o = pools[task >> 6];
         const uint32_t won = o.won[q];
         const int64_t ev = o.sc.ev[q];
@@ -571,13 +579,19 @@ __global__ void __launch_bounds__(kMaxThreads)
         t.q2 = rec.q2;
         t.zp = rec.zp;
         t.ls = rec.ls;
-        settle_counts(E, o, q);
-        cycle_emit<kMode>(P0, E, t, [&](int count) { return atomicAdd(&blk.n_jobs, count); },
-                          [&](int at, uint32_t job) { pools[at >> 7].m.jobs[at & 127] = job; }, tid);
-        o.sc.n[q] = static_cast<uint8_t>(t.n + 1);
-        bool over = false;
-        if constexpr (kSlice) over = o.cyc[q] >= sl.cycles;
-        o.state[q] = over ? kSlotSliced : kSlotLoad;
+        const auto reserve = [&](int count) { return atomicAdd(&blk.n_jobs, count); };
+        const auto put = [&](int at, uint32_t job) { pools[at >> 7].m.jobs[at & 127] = job; };
+        if (quads)
+          emit_warp4<kMode>(P0, E, t, has, reserve, put, r);
+        else
+          cycle_emit<kMode>(P0, E, t, reserve, put, r);
+        if (has && (!quads || (tid & 3) == 0)) {
+          settle_counts(E, o, q);
+          o.sc.n[q] = static_cast<uint8_t>(t.n + 1);
+          bool over = false;
+          if constexpr (kSlice) over = o.cyc[q] >= sl.cycles;
+          o.state[q] = over ? kSlotSliced : kSlotLoad;
+        }
       }
       __syncthreads();
       const int jobs = blk.n_jobs;

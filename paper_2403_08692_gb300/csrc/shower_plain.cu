@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(kStepThreads, GAPS_STEP_MIN_BLOCKS)
                     unsigned long long* reset_cursor, StepPublish pub) {
   __shared__ EmitTask s_task[kStepThreads];
   __shared__ uint32_t s_jobs[kMaxRefresh * kStepThreads];
-  __shared__ SharedSplitting s_split[kEmitChunk];
+  __shared__ Splitting4 s_split[kEmitChunk];
   __shared__ int s_njobs;
   __shared__ unsigned long long s_base;
   const int tid = threadIdx.x;
