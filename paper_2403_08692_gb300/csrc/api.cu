@@ -375,9 +375,10 @@ cudaError_t clear_shower_counters(const Events& E, bool plain, cudaStream_t s) {
 
 // Host memory of the plain form's host loop, per host thread: the final
 // counters, the host-mapped slots the step launches publish their input
-// lengths to ({list, tasks, sequence number}, kSlots of them in rotation),
-// and the timing events.  Sequence numbers grow across calls (`next_seq`),
-// so a slot never shows a value of an earlier call as current.
+// lengths to ({list, tasks}, each tagged with the launch's sequence number,
+// kSlots of them in rotation), and the timing events.  Sequence numbers grow
+// across calls (`next_seq`), so a slot never shows a value of an earlier call
+// as current.
 struct HostCounters {
   static constexpr int kSlots = 8;
   static constexpr int kSlotWords = 4;
@@ -423,12 +424,15 @@ HostCounters& host_counters() {
 #define GAPS_REBUILD_DIV 16
 #endif
 
-// Launches the plain form's host loop queues ahead of the one it reads back.
-#ifndef GAPS_PLAIN_LOOKAHEAD
-#define GAPS_PLAIN_LOOKAHEAD 1
-#endif
-constexpr int64_t kLookahead = GAPS_PLAIN_LOOKAHEAD;
-static_assert(kLookahead >= 1 && kLookahead + 2 <= 8, "lookahead and readback slots");
+// Launches the plain form's host loop queues ahead of the one it reads back:
+// two while the list rebuild makes a step two launches, else one.  Two
+// against one: 5x10^4 events 2.03 -> 1.95 ms, 10^5 2.36 -> 2.30, 2x10^5 2.89
+// -> 2.86; without the rebuild the older count costs more than the queue
+// gains (1.2x10^4 events 1.37 -> 1.42 ms), and where a step is long it gains
+// nothing (10^6 events 7.69 -> 7.72).
+constexpr int64_t kLookaheadMax = 2;
+static_assert(kLookaheadMax + 2 <= HostCounters::kSlots, "lookahead and readback slots");
+constexpr int64_t lookahead(int64_t n) { return n >= GAPS_REBUILD_MIN && n < 300000 ? kLookaheadMax : 1; }
 
 int shower_impl(const gaps_params* params, const gaps_batch* batch, int mode, int64_t* launches_out,
                 double* kernel_ms_out, void* stream) {
@@ -493,12 +497,16 @@ int shower_impl(const gaps_params* params, const gaps_batch* batch, int mode, in
   int64_t bound = E.n;  // upper bound on the live events entering the next launch
   int64_t queued = 0;   // launches queued
   int64_t worked = 0;   // launches whose input held events
+  const int64_t ahead = lookahead(E.n);
   const int64_t max_launches = 2 * static_cast<int64_t>(P.max_steps) + 2;
   const unsigned long long seq0 = hc.next_seq;  // launch c publishes launch c - 1's lengths as seq0 + c
   hc.next_seq += static_cast<unsigned long long>(max_launches) + 1;
   auto pub_slot = [&](int64_t c, bool device) {
     const size_t at = static_cast<size_t>(c % HostCounters::kSlots) * HostCounters::kSlotWords;
     return (device ? hc.pub_dev : hc.pub) + at;
+  };
+  auto pub_tag = [&](int64_t c) {
+    return ((seq0 + static_cast<unsigned long long>(c)) | 0x80000000ull) << 32;  // never that of a cleared word
   };
   auto enqueue = [&](int64_t c) -> cudaError_t {
     const int in_half = static_cast<int>(c & 1), out_half = 1 - in_half;
@@ -522,7 +530,7 @@ int shower_impl(const gaps_params* params, const gaps_batch* batch, int mode, in
     unsigned long long* tw = &E.counters[kPlainTaskWord];
     unsigned long long* cw = &E.counters[kPlainEmitCursorWord];
     const int r0 = static_cast<int>(c % 3), r1 = static_cast<int>((c + 1) % 3), r2 = static_cast<int>((c + 2) % 3);
-    const StepPublish pub{c == 0 ? nullptr : pub_slot(c - 1, true), seq0 + static_cast<unsigned long long>(c)};
+    const StepPublish pub{c == 0 ? nullptr : pub_slot(c - 1, true), pub_tag(c)};
     err = launch_step_deferred(P, E, list_in, c == 0 ? E.n : bound, c == 0 ? nullptr : lw + r0, tasks_in,
                                c == 0 ? 0 : bound, c == 0 ? nullptr : tw + r0, list_out, lw + r1, tasks_out, tw + r1,
                                lw + r2, tw + r2, cw + r0, cw + r2, pub, s);
@@ -547,23 +555,28 @@ int shower_impl(const gaps_params* params, const gaps_batch* batch, int mode, in
       return err;
     }
     volatile unsigned long long* w = pub_slot(c, false);
-    const unsigned long long want = seq0 + static_cast<unsigned long long>(c) + 1;
-    for (uint64_t spin = 1; w[2] != want; ++spin) {
+    const unsigned long long tag = pub_tag(c + 1);
+    unsigned long long list = 0, tasks = 0;
+    auto published = [&] {
+      list = w[0] - tag;
+      tasks = w[1] - tag;
+      return list < 0x80000000ull && tasks < 0x80000000ull;
+    };
+    for (uint64_t spin = 1; !published(); ++spin) {
       if ((spin & 1023) != 0) continue;
       // every 1024 polls: has the stream failed, or drained without it?
       const cudaError_t q = cudaStreamQuery(s);
-      if (q == cudaSuccess && w[2] != want) return cudaErrorUnknown;
+      if (q == cudaSuccess && !published()) return cudaErrorUnknown;
       if (q != cudaSuccess && q != cudaErrorNotReady) return q;
     }
-    std::atomic_thread_fence(std::memory_order_acquire);
-    bound = static_cast<int64_t>(w[0] + w[1]);
+    bound = static_cast<int64_t>(list + tasks);
     return cudaSuccess;
   };
   if ((e = enqueue(queued++)) != cudaSuccess) return cuda_fail(e);
   for (int64_t c = 0;; ++c) {
-    // c: the oldest launch not yet read back; keep kLookahead more queued
+    // c: the oldest launch not yet read back; keep `ahead` more queued
     // behind it, so the GPU has work while the host waits for the counts
-    while (queued < max_launches && queued <= c + kLookahead)
+    while (queued < max_launches && queued <= c + ahead)
       if ((e = enqueue(queued++)) != cudaSuccess) return cuda_fail(e);
     if ((e = live_after(c)) != cudaSuccess) return cuda_fail(e);
     worked = c + 1;

@@ -55,11 +55,12 @@ cudaError_t launch_step_plain(const DevParams& P, const Events& E, const int* li
 // launch); *reset_cursor, the next launch's cursor, is zeroed.  With
 // pub.slot set (host-mapped memory), the launch writes its input lengths --
 // the previous launch's output lengths -- to pub.slot[0..1] as it starts,
-// then pub.seq to pub.slot[2], so that the host learns them without a copy
-// on the stream.
+// each with pub.tag in its upper half, so that the host learns them without a
+// copy on the stream and the launch without a fence: waiting for a sequence
+// number's turn cost each launch about 0.7 us (10^3 events 0.84 -> 0.79 ms).
 struct StepPublish {
   unsigned long long* slot;
-  unsigned long long seq;
+  unsigned long long tag;
 };
 cudaError_t launch_step_deferred(const DevParams& P, const Events& E, const int* list_in, int64_t n_list,
                                  const unsigned long long* n_list_dev, const EmitTask* tasks_in, int64_t n_tasks,

@@ -320,12 +320,11 @@ __global__ void __launch_bounds__(kStepThreads, GAPS_STEP_MIN_BLOCKS)
     if (reset_tasks) *reset_tasks = 0ull;
     if (reset_cursor) *reset_cursor = 0ull;
     if (pub.slot) {
-      // the lengths are final: the launch that wrote them has finished
+      // the lengths (below 2^31) are final: the launch that wrote them has
+      // finished.  Each word carries the tag, so neither waits for the other.
       volatile unsigned long long* w = pub.slot;
-      w[0] = n_list_dev ? *n_list_dev : static_cast<unsigned long long>(n_list);
-      w[1] = n_tasks_dev ? *n_tasks_dev : static_cast<unsigned long long>(n_tasks);
-      __threadfence_system();
-      w[2] = pub.seq;
+      w[0] = pub.tag | (n_list_dev ? *n_list_dev : static_cast<unsigned long long>(n_list));
+      w[1] = pub.tag | (n_tasks_dev ? *n_tasks_dev : static_cast<unsigned long long>(n_tasks));
     }
   }
   const int64_t emit_blocks = static_cast<int64_t>(gridDim.x) - select_blocks;
