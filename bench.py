@@ -32,14 +32,16 @@ UNIT = "events/s"
 # Trial ranking and veto decisions give the same outcome in FP32 and are not
 # counted.  "simple" = +, -, x or a fused a*b+c; the other operations are
 # converted to DFMA-equivalents with their throughput measured on the device
-# in the same run (gaps_probe_fp64_rates; a log at the rate of the faster of
-# the library's and the shower's own table-driven log).
+# in the same run (gaps_probe_fp64_rates), or by the FP64 instructions of the
+# shower's own functions where those are fewer (csrc/math_fp64.cuh; a log at
+# the measured rate of the faster of the library's and the shower's own).
 #   per winner:   ln r and the scaled update of ln t
 #   per emission: t = exp(ln t), z (expm1), y, the azimuth (sincospi), the
 #                 dipole map (transverse frame, k_perp, three momenta) and
 #                 four dipole-cache refreshes (Q^2, z+, ln(z+/z-), 1/ln)
 WORK_PER_WINNER = {"simple": 5, "log": 1}
 WORK_PER_EMISSION = {"simple": 164, "div": 18, "sqrt": 7, "log": 4, "exp": 2, "sincospi": 1}
+OWN_FP64_INSTRUCTIONS = {"exp": 13, "sincospi": 18, "div": 6, "sqrt": 6}
 # FP64 units: two DFMA per SM per clock (the sm__sass_thread_inst_executed_op_dfma
 # peak ncu reports for this GB300), two flops per DFMA.
 DFMA_PER_SM_PER_CLOCK = 2
@@ -112,24 +114,27 @@ def pipe_fractions():
             "source": "profiles/k_step_deferred_1e5.md (ncu --set full, launches 21-22 of a 10^5-event pass)"}
 
 
-def dfma_equivalents(counts, rates, library_log=False):
-    """DFMA-equivalents of an operation count; a logarithm costs what the
-    faster of the library's log and the shower's table-driven one costs (the
-    library's alone with library_log)."""
-    def rate(op):
-        if op == "log" and not library_log:
-            return max(rates["log"], rates.get("log_fp64", 0.0))
-        return rates[op]
-    return sum(n * (1.0 if op == "simple" else rates["dfma"] / rate(op)) for op, n in counts.items())
+def dfma_equivalents(counts, rates, library=False):
+    """DFMA-equivalents of an operation count; a function costs what the
+    cheaper of the library's and the shower's own costs (the library's with
+    `library`)."""
+    def cost(op):
+        if op == "simple":
+            return 1.0
+        c = rates["dfma"] / rates[op]
+        if not library:
+            c = min(c, rates["dfma"] / rates.get("log_fp64", rates["log"]) if op == "log" else OWN_FP64_INSTRUCTIONS[op])
+        return c
+    return sum(n * cost(op) for op, n in counts.items())
 
 
-def kernels_outside_shower(capacity):
+def kernels_outside_shower(capacity, events):
     """Library kernels per pass besides the shower cycles: matrix element,
-    validation, the three bucketing kernels and one event-shape kernel per
-    multiplicity class (16, 32, 64, 128, 256 slots), the fixed-point
-    histogram fill and its conversion."""
-    classes = sum(1 for lo in (0, 16, 32, 64, 128) if capacity > lo)
-    return 1 + 1 + 3 + classes + 2
+    validation, bucketing (one kernel up to 4096 events, else three), one
+    event-shape kernel per multiplicity class (up to 16, 128 and 255 partons),
+    the fixed-point histogram fill and its conversion."""
+    classes = sum(1 for lo in (0, 16, 128) if capacity > lo)
+    return 1 + 1 + (1 if events <= 4096 else 3) + classes + 2
 
 
 def parse():
@@ -583,7 +588,7 @@ def main():
             times.append(e0.elapsed_time(e1))
         variants["persistent"] = {"value": n * args.steps / (sum(times) / 1e3), "unit": UNIT,
                                   "ms_per_step": sum(times) / args.steps, "config": cfg.as_dict(),
-                                  "launches_per_pass": kernels_outside_shower(args.capacity) + 1}
+                                  "launches_per_pass": kernels_outside_shower(args.capacity, n) + 1}
         # CUDA graph of the whole pass
         side = torch.cuda.Stream()
         side.wait_stream(stream)
@@ -854,7 +859,7 @@ def main():
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": 48,
                 "d2h_bytes_per_step": 8 * g.HIST_DOUBLES + len(bytes(g.Stats())),
                 "api": "gaps_run (parameters from host, histograms and statistics back to host)"},
-        "gpu_launches": int(args.steps * (kernels_outside_shower(args.capacity) + int(counters[27]))
+        "gpu_launches": int(args.steps * (kernels_outside_shower(args.capacity, n) + int(counters[27]))
                             + launches_total),
         "roofline": {"bound": "alu", "kernel": "k_step_deferred (plain-form step: select/veto + deferred emissions)",
                      "achieved": achieved_tflops, "peak": peak_tflops, "unit": "TFLOP/s",
@@ -886,8 +891,8 @@ def main():
                                     f"MEASURED_PEAKS.json has no FP64 entry",
                      "work_model": f"required FP64 work: {dfma_per_winner:.1f} DFMA-equivalents per winner, "
                                    f"{dfma_per_emission:.1f} per accepted emission (oracle formulas; "
-                                   f"transcendentals at their measured cost, a log at the faster of "
-                                   f"the library's and the table-driven one), x2 flops",
+                                   f"functions at the cheaper of the library's measured cost and the "
+                                   f"shower's own), x2 flops",
                      "launches_per_pass": launches_per_pass,
                      "avg_launch_ms": kernel_s_per_launch * 1e3,
                      "fp64_probe_per_s": {k: float(f"{v:.4g}") for k, v in rates.items()},

@@ -10,8 +10,9 @@
 //  2. Decide.  Each lane settles its event's winner (FP64 scale), cutoff and
 //     veto.  An event with an accepted emission waits; a finished one leaves.
 // Once enough emissions wait, the block's warps generate them together,
-// packed into as few warps as hold them, and refresh the dipoles they moved
-// with all threads.  Slots of events that left are written back and refilled
+// packed into as few warps as hold them (four lanes each where that is
+// fewer than a warp a scheduler), and refresh the dipoles they moved with all
+// threads.  Slots of events that left are written back and refilled
 // from a global event cursor.  Events therefore leave as soon as they finish
 // -- the paper's cutoff inefficiency (Sec. 2, Fig. 3: finished events wait
 // for the last one) disappears.
@@ -28,9 +29,9 @@
 // 11).  Keeping the state in shared memory leaves one 32-byte record per
 // cycle and event to global memory.  Measured (GB300, shower kernel alone;
 // before: block pools of one or two events per thread, each event's trials
-// in one thread, state in global memory): 10^6 LEP events 7.39 -> 5.59 ms,
-// 10^5 1.31 -> 0.94 ms, 10^5 at 200 GeV and t_C = 0.5 3.30 -> 2.5 ms, 100
-// events 0.54 -> 0.20 ms.  At 10^6 events the FP64 pipe is busy 45 % of the
+// in one thread, state in global memory): 10^6 LEP events 7.39 -> 5.57 ms,
+// 10^5 1.31 -> 0.90 ms, 10^5 at 200 GeV and t_C = 0.5 3.30 -> 2.4 ms, 100
+// events 0.54 -> 0.19 ms.  At 10^6 events the FP64 pipe is busy 45 % of the
 // time and 36 % of the issue slots are used; 20 or 24 resident warps (fewer
 // registers) and pools of 40 to 56 events were no faster.
 //
@@ -53,6 +54,8 @@ namespace {
 constexpr int kSlots = 64;
 // The register budget is set for 16 warps per SM.
 constexpr int kMaxThreads = 512;
+// Warp schedulers of an SM.
+constexpr int kSchedulers = 4;
 // Veto cycles a warp runs between two votes of its block (1 to 8 were alike).
 constexpr int kTurns = 3;
 
@@ -550,10 +553,12 @@ __global__ void __launch_bounds__(kMaxThreads)
       if (s1 == kSlotPending && r1 < tasks)
         pools[r1 >> 5].m.tasks[r1 & 31] = static_cast<uint16_t>(warp * kSlots + lane + 32);
       __syncthreads();
-#ifndef G_QUADS
-#define G_QUADS 4
-#endif
-      const bool quads = tasks <= 8 * min(n_warps, G_QUADS);
+      // Four lanes a task while the tasks then take at most a warp on each of
+      // the SM's schedulers, whose FP64 issue one warp fills: a chain of 90
+      // FP64 instructions instead of 159.  Beyond, a thread a task takes half
+      // the instructions.  100 events 0.197 -> 0.190 ms, 2x10^4 0.253 ->
+      // 0.244 (up to 1, 2, 4 or 8 such warps alike), 10^6 unchanged.
+      const bool quads = tasks <= 8 * min(n_warps, kSchedulers);
       // the task of this lane, or the last one on the lanes left over
       const int at_task = quads ? tid >> 2 : tid;
       const bool has = at_task < tasks;
@@ -749,8 +754,8 @@ cudaError_t launch_m(const DevParams& P, const Events& E, const gaps_persistent_
   if (fit < 1) return cudaErrorInvalidConfiguration;
   const int per_sm = cfg.blocks_per_sm > 0 && cfg.blocks_per_sm < fit ? cfg.blocks_per_sm : fit;
   // At least a dozen events per warp while there are fewer than fill the
-  // device: the emissions then fill their warps better (5x10^3 events 0.517 ->
-  // 0.500 ms, 2x10^4 0.621 -> 0.603 ms).
+  // device: the emissions then fill their warps better (six, eight or sixteen
+  // a warp measure within 3 % from 3x10^3 to 5x10^4 events).
   const int64_t warps = threads == 32 ? n : (n + 11) / 12;
   const int64_t blocks = std::min(static_cast<int64_t>(sms) * per_sm,
                                   std::max<int64_t>((warps + threads / 32 - 1) / (threads / 32), std::min<int64_t>(sms, n)));
