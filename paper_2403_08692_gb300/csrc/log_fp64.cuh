@@ -31,6 +31,13 @@
 
 namespace gaps {
 
+// Out of line: inlined, the conversion is predicated instead of branched
+// around, and an FP64-pipe instruction takes its 16 cycles with no lane
+// active, one in ten of the shower's and the event shapes' FP64 cycles.
+#ifdef __CUDACC__
+static __device__ __noinline__ float f32_hardware(double x) { return __double2float_rn(x); }
+#endif
+
 // double -> float, round to nearest even, with integer instructions for
 // every result in the normal float range (the FP64 pipe's conversion costs
 // as much as an FMA on this part; the ALU's instructions a small fraction of
@@ -47,7 +54,7 @@ __host__ __device__ __forceinline__ float f32_from_f64(double x) {
   // exponent field 897 .. 1150: normal floats, before rounding
   if (mag - 0x3810000000000000ull >= 0x0fe0000000000000ull) {
 #ifdef __CUDA_ARCH__
-    return __double2float_rn(x);
+    return f32_hardware(x);
 #else
     return static_cast<float>(x);
 #endif
