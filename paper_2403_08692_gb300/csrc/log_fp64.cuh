@@ -94,7 +94,7 @@ __host__ __device__ __forceinline__ double log_fp64(double x) {
 #endif
   // positive normal x (tested on the bits: the FP64 pipe's compares cost as
   // much as its FMAs on this part)
-  if (bits - 0x0010000000000000ull >= 0x7fe0000000000000ull) return log_library(x);
+  if (static_cast<uint32_t>(bits >> 32) - 0x00100000u >= 0x7fe00000u) return log_library(x);
   constexpr uint64_t kFrac = (uint64_t{1} << 52) - 1;
   constexpr uint64_t kSqrt2Frac = 0x6a09e667f3bcdull;  // fraction bits of sqrt(2)
   const uint64_t frac = bits & kFrac;

@@ -425,6 +425,13 @@ __device__ __forceinline__ void screen_group_reduce(Screen& sc) {
 // What the FP32 screen settles about a cycle: no trial above the cutoff, a
 // certain winner (its exact scale computed), or neither -- then the exact
 // FP64 selection decides (select_winner_fp64 / fallback_warp).
+// a > b for numbers (b not -0), from their bits put in order: the FP64 pipe's
+// compares cost as much as its FMAs.
+__device__ __forceinline__ bool above(double a, double b) {
+  const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+  return (x ^ ((x >> 63) & 0x7fffffffffffffffll)) > (y ^ ((y >> 63) & 0x7fffffffffffffffll));
+}
+
 enum : int { kScreenNone = 0, kScreenWinner = 1, kScreenUndecided = 2 };
 
 // The screen's verdict; for a certain winner its exact scale (from the FP64
@@ -459,7 +466,7 @@ __device__ __forceinline__ int screen_verdict(const DevParams& P, const Events& 
     const double inv_c =
         combined ? inv_c_sum_fp64(P, rec.zp, rec.ls) : inv_c_fp64(P, kind, rec.zp, rec.inv_ls);
     const double lt = fma(log_fp64(to_unit(best_hi, best_lo)), inv_c, lnt);
-    if (lt > P.ln_tc) {
+    if (above(lt, P.ln_tc)) {
       task.lnt = lt;
       task.q2 = rec.q2;
       task.zp = rec.zp;
