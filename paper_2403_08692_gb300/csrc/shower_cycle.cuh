@@ -517,8 +517,7 @@ __device__ inline int cycle_screen(const DevParams& P, const Events& E, int64_t 
 // needing lanes.  Every lane of the warp must call it.
 template <int kMode>
 __device__ __noinline__ void fallback_warp(const DevParams& P0, const Events& E, bool need, int64_t ev, int job,
-                                           const EventKey& key, int step, int n, double lnt, bool& have,
-                                           EmitTask& task) {
+                                           EventKey key, int step, int n, double lnt, bool& have, EmitTask& task) {
   const int lane = static_cast<int>(threadIdx.x & 31);
   unsigned pending = __ballot_sync(0xffffffffu, need);
   while (pending) {

@@ -698,9 +698,20 @@ __global__ void __launch_bounds__(kMaxThreads)
         if (verdict == kScreenUndecided) atomicAdd(&E.counters[2], 1ull);  // full FP64 cycle
       }
       bool have = verdict == kScreenWinner;
-      if (__any_sync(0xffffffffu, verdict == kScreenUndecided))
-        fallback_warp<kMode>(P0, E, verdict == kScreenUndecided, ev, job, key, step, q >= 0 ? w.sc.n[q] : 0, lnt, have,
-                             task);
+      // The exact selection's results in their own variables: the call, out of
+      // line, takes them by address, and `task` itself would live in local
+      // memory for every cycle (10^6 events 5.55 -> 5.33 ms; the plain step,
+      // at half the registers, is 2 % faster with it there).
+      if (__any_sync(0xffffffffu, verdict == kScreenUndecided)) {
+        EmitTask exact;
+        bool found = false;
+        fallback_warp<kMode>(P0, E, verdict == kScreenUndecided, ev, job, key, step, q >= 0 ? w.sc.n[q] : 0, lnt, found,
+                             exact);
+        if (verdict == kScreenUndecided) {
+          have = found;
+          task = exact;
+        }
+      }
       if (limited) w.state[q] = kSlotLimit;
       if (lead) {
         w.step[q] = step + 1;
