@@ -1,8 +1,8 @@
 """The finalisation kernels' forms for small batches give what the forms for
 large ones give, bit for bit: event shapes by 16, 8 or 4 lanes per event and
 by one thread, validation by lanes and by threads (on broken records too),
-histograms with an observable per warp, the buckets of one block; and a small
-pass captured in a CUDA graph, where its launches are chained.  Requires a
+histograms with an observable per warp, the buckets of one block; and a pass
+captured in a CUDA graph, where its launches are chained.  Requires a
 GB300."""
 import numpy as np
 import pytest
@@ -96,12 +96,13 @@ def test_histograms(g, large):
     assert torch.equal(whole, parts)
 
 
-def test_small_pass_in_a_graph(g):
-    p = g.make_params(seed=43)
-    n = 3000
+@pytest.mark.parametrize("n,cap", [(3000, CAP), (3000, 160), (70_000, 160)])
+def test_pass_in_a_graph(g, n, cap):
+    """Chained launches, and event-shape classes beside one another."""
+    p = g.make_params(seed=43, sqrt_s=200.0, t_cutoff=0.5)
     want = torch.zeros(g.HIST_DOUBLES, dtype=torch.float64).pin_memory()
-    assert g.run(p, g.Workspace(n, CAP), want, g.SHOWER_PERSISTENT)[0] == 0
-    ws, hist = g.Workspace(n, CAP), torch.zeros(g.HIST_DOUBLES, dtype=torch.float64, device="cuda")
+    assert g.run(p, g.Workspace(n, cap), want, g.SHOWER_PERSISTENT)[0] == 0
+    ws, hist = g.Workspace(n, cap), torch.zeros(g.HIST_DOUBLES, dtype=torch.float64, device="cuda")
     stats = torch.zeros(64, dtype=torch.int64, device="cuda")
     side = torch.cuda.Stream()
     side.wait_stream(torch.cuda.current_stream())
