@@ -549,40 +549,45 @@ __global__ void __launch_bounds__(256) k_stats(Events E, gaps_stats* st) {
     sw += w;
     sw2 += w * w;
   }
-  // warp reduction, then one atomic per warp
+  // warp reductions, the block's in shared memory, then one atomic per block
+  // (per warp, the adds to the same few words took most of the kernel)
+  __shared__ long long s_sum[10][8], s_max[8];
+  __shared__ double s_w[2][8];
+  const int lane = static_cast<int>(threadIdx.x & 31), warp = static_cast<int>(threadIdx.x >> 5);
+  long long sums[10] = {done, over, lim, inval, steps, trials, wins, ems, parts, dips};
   for (int o = 16; o > 0; o >>= 1) {
-    done += __shfl_down_sync(0xffffffffu, done, o);
-    over += __shfl_down_sync(0xffffffffu, over, o);
-    lim += __shfl_down_sync(0xffffffffu, lim, o);
-    inval += __shfl_down_sync(0xffffffffu, inval, o);
-    steps += __shfl_down_sync(0xffffffffu, steps, o);
+#pragma unroll
+    for (int k = 0; k < 10; ++k) sums[k] += __shfl_down_sync(0xffffffffu, sums[k], o);
     const long long om = __shfl_down_sync(0xffffffffu, mx, o);
     mx = om > mx ? om : mx;
-    trials += __shfl_down_sync(0xffffffffu, trials, o);
-    wins += __shfl_down_sync(0xffffffffu, wins, o);
-    ems += __shfl_down_sync(0xffffffffu, ems, o);
-    parts += __shfl_down_sync(0xffffffffu, parts, o);
-    dips += __shfl_down_sync(0xffffffffu, dips, o);
     sw += __shfl_down_sync(0xffffffffu, sw, o);
     sw2 += __shfl_down_sync(0xffffffffu, sw2, o);
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0)
-    atomicAdd(reinterpret_cast<unsigned long long*>(&st->n_events), static_cast<unsigned long long>(E.n));
-  if ((threadIdx.x & 31) == 0) {
-    auto add = [](int64_t* p, long long v) {
-      if (v) atomicAdd(reinterpret_cast<unsigned long long*>(p), static_cast<unsigned long long>(v));
-    };
-    add(&st->n_done, done);
-    add(&st->n_overflow, over);
-    add(&st->n_step_limit, lim);
-    add(&st->n_invalid, inval);
-    add(&st->sum_steps, steps);
+  if (lane == 0) {
+#pragma unroll
+    for (int k = 0; k < 10; ++k) s_sum[k][warp] = sums[k];
+    s_max[warp] = mx;
+    s_w[0][warp] = sw;
+    s_w[1][warp] = sw2;
+  }
+  __syncthreads();
+  int64_t* const words[10] = {&st->n_done,     &st->n_overflow,  &st->n_step_limit,  &st->n_invalid,   &st->sum_steps,
+                              &st->sum_trials, &st->sum_winners, &st->sum_emissions, &st->sum_partons, &st->sum_dipoles};
+  if (threadIdx.x == 0) {
+    if (blockIdx.x == 0)
+      atomicAdd(reinterpret_cast<unsigned long long*>(&st->n_events), static_cast<unsigned long long>(E.n));
+#pragma unroll
+    for (int k = 0; k < 10; ++k) {
+      long long v = 0;
+      for (int w = 0; w < 8; ++w) v += s_sum[k][w];
+      if (v) atomicAdd(reinterpret_cast<unsigned long long*>(words[k]), static_cast<unsigned long long>(v));
+    }
+    for (int w = 1; w < 8; ++w) {
+      mx = s_max[w] > mx ? s_max[w] : mx;
+      sw += s_w[0][w];
+      sw2 += s_w[1][w];
+    }
     atomicMax(reinterpret_cast<unsigned long long*>(&st->max_steps), static_cast<unsigned long long>(mx));
-    add(&st->sum_trials, trials);
-    add(&st->sum_winners, wins);
-    add(&st->sum_emissions, ems);
-    add(&st->sum_partons, parts);
-    add(&st->sum_dipoles, dips);
     atomicAdd(&st->sum_weight, sw);
     atomicAdd(&st->sum_weight2, sw2);
   }
