@@ -29,10 +29,10 @@
 // 11).  Keeping the state in shared memory leaves one 32-byte record per
 // cycle and event to global memory.  Measured (GB300, shower kernel alone;
 // before: block pools of one or two events per thread, each event's trials
-// in one thread, state in global memory): 10^6 LEP events 7.39 -> 5.57 ms,
-// 10^5 1.31 -> 0.90 ms, 10^5 at 200 GeV and t_C = 0.5 3.30 -> 2.4 ms, 100
-// events 0.54 -> 0.19 ms.  At 10^6 events the FP64 pipe is busy 45 % of the
-// time and 36 % of the issue slots are used; 20 or 24 resident warps (fewer
+// in one thread, state in global memory): 10^6 LEP events 7.39 -> 5.33 ms,
+// 10^5 1.31 -> 0.88 ms, 10^5 at 200 GeV and t_C = 0.5 3.30 -> 2.3 ms, 100
+// events 0.54 -> 0.19 ms.  At 3x10^5 events the FP64 pipe is busy 43 % of the
+// time and 37 % of the issue slots are used; 20 or 24 resident warps (fewer
 // registers) and pools of 40 to 56 events were no faster.
 //
 // Nothing waits on another block: a block ends when its pools are empty and
