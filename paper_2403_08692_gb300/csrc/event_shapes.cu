@@ -39,20 +39,6 @@ namespace gaps {
 
 namespace {
 
-// follow_launch of a kernel whose next launch may run beside it: the next one
-// is let go after this one's wait, so what came before is complete for both.
-__device__ __forceinline__ void follow_launch_first() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-// A kernel that runs beside the launch before it (which called
-// follow_launch_first or these two): it starts at once, and its last block
-// ends after that launch has, so that it completes last for what comes next.
-__device__ __forceinline__ void beside_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void end_beside_launch() {
-  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-
 constexpr int kShapeThreads = 128;
 constexpr int kMaskMax = 64;
 
@@ -1504,28 +1490,21 @@ __global__ void __launch_bounds__(1024) k_buckets_small(Events E, int* offsets, 
 // blocks of its largest events, dealt out last).
 template <int MAXJ>
 __global__ void __launch_bounds__(kShapeThreads) k_event_shapes(DevParams P, Events E, const int* order,
-                                                                const int* offsets, int n_lo, int n_hi, bool beside) {
-  if (beside)
-    beside_launch();
-  else
-    follow_launch();
+                                                                const int* offsets, int n_lo, int n_hi) {
+  follow_launch();
   const int begin = offsets[n_lo], end = offsets[n_hi + 1 > 256 ? 256 : n_hi + 1];
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < end - begin; j += gridDim.x * blockDim.x) {
     const int64_t ev = order[end - 1 - j];
     event_shapes<MAXJ>(P, E, ev, E.n_partons[ev]);
   }
-  if (beside) end_beside_launch();
 }
 
 // Events of buckets n_lo..n_hi (all with n <= MAXJ), L lanes per event, T
 // threads per block.
 template <int MAXJ, int L, int T>
 __global__ void __launch_bounds__(T) k_event_shapes_group(DevParams P, Events E, const int* order,
-                                                          const int* offsets, int n_lo, int n_hi, bool beside) {
-  if (beside)
-    beside_launch();
-  else
-    follow_launch();
+                                                          const int* offsets, int n_lo, int n_hi) {
+  follow_launch();
   constexpr int G = T / L;
   __shared__ GroupArrays<MAXJ> s_ev[G];
   const int g = threadIdx.x / L, sub = threadIdx.x % L;
@@ -1536,7 +1515,6 @@ __global__ void __launch_bounds__(T) k_event_shapes_group(DevParams P, Events E,
     event_shapes_group<MAXJ, L>(P, E, ev, E.n_partons[ev], s_ev[g], sub, gm);
     __syncwarp(gm);  // the group's arrays are free for its next event
   }
-  if (beside) end_beside_launch();
 }
 
 // Events of buckets n_lo..n_hi (all with n <= MAXJ), a warp each, T threads
@@ -1544,25 +1522,22 @@ __global__ void __launch_bounds__(T) k_event_shapes_group(DevParams P, Events E,
 // one by one from *cursor (zero before the launch).
 template <int MAXJ, int T>
 __global__ void __launch_bounds__(T) k_event_shapes_warp(DevParams P, Events E, const int* order, const int* offsets,
-                                                         int n_lo, int n_hi, int* cursor, bool beside) {
-  if (beside)
-    beside_launch();
-  else
-    follow_launch_first();
+                                                         int n_lo, int n_hi, int* cursor) {
+  follow_launch();
   extern __shared__ __align__(16) unsigned char s_shapes[];
   WarpEvent<MAXJ>& a = reinterpret_cast<WarpEvent<MAXJ>*>(s_shapes)[threadIdx.x >> 5];
   const int lane = static_cast<int>(threadIdx.x & 31);
   const int begin = offsets[n_lo], end = offsets[n_hi + 1 > 256 ? 256 : n_hi + 1];
-  while (begin < end) {
+  if (begin == end) return;
+  for (;;) {
     int k = 0;
     if (lane == 0) k = atomicAdd(cursor, 1);
     k = __shfl_sync(0xffffffffu, k, 0);
-    if (k >= end - begin) break;
+    if (k >= end - begin) return;
     const int64_t ev = order[end - 1 - k];
     event_shapes_warp<MAXJ>(P, E, ev, E.n_partons[ev], a, lane);
     __syncwarp();  // the arrays are free for the next event
   }
-  if (beside) end_beside_launch();
 }
 
 // Events of up to 16 partons take one thread each in batches of at least
@@ -1623,26 +1598,9 @@ cudaError_t launch_observables(const DevParams& P, const Events& E, int* buckets
     const int64_t want = (E.n + per_block - 1) / per_block;
     return static_cast<unsigned>(want < static_cast<int64_t>(per_sm) * sms ? want : static_cast<int64_t>(per_sm) * sms);
   };
-  // One class up to 128 partons (96 registers leave five blocks per SM), one
-  // beyond, then the small events beside them: a lone large event takes about
-  // as long alone (stage at 10^6 events 0.82 -> 0.78 ms).  The large classes'
-  // cursors are the bucket cursors of 0 and 1 partons, which no event has: zero.
-  bool beside = false;
-  if (E.cap > 128) {
-    e = launch_chained(chain, k_event_shapes_warp<256, 64>, grid(2, 6), 64, 2 * sizeof(WarpEvent<256>), s, P, E, order,
-                       offsets, 129, 255, cursor + 1, beside);
-    beside = true;
-  }
-  if (e == cudaSuccess && E.cap > 16) {
-    e = launch_chained(chain || beside, k_event_shapes_warp<128, 128>, grid(4, 5), 128, 4 * sizeof(WarpEvent<128>), s, P,
-                       E, order, offsets, 17, 128, cursor, beside);
-    beside = true;
-  }
-  if (e != cudaSuccess) return e;
   const auto groups = [&](auto lanes) {
     constexpr int L = decltype(lanes)::value;
-    return launch_chained(chain || beside, k_event_shapes_group<16, L, 128>, grid(128 / L, 8), 128, 0, s, P, E, order,
-                          offsets, 0, 16, beside);
+    return launch_chained(chain, k_event_shapes_group<16, L, 128>, grid(128 / L, 8), 128, 0, s, P, E, order, offsets, 0, 16);
   };
   if (E.n < 10000) {
     e = groups(std::integral_constant<int, 16>{});
@@ -1651,9 +1609,18 @@ cudaError_t launch_observables(const DevParams& P, const Events& E, int* buckets
   } else if (E.n < kThreadsFrom) {
     e = groups(std::integral_constant<int, 4>{});
   } else {
-    e = launch_chained(chain || beside, k_event_shapes<16>, grid(kShapeThreads, kShapeBlocksPerSm), kShapeThreads, 0, s, P,
-                       E, order, offsets, 0, 16, beside);
+    e = launch_chained(chain, k_event_shapes<16>, grid(kShapeThreads, kShapeBlocksPerSm), kShapeThreads, 0, s, P, E, order,
+                       offsets, 0, 16);
   }
+  // One class up to 128 partons (96 registers leave five blocks per SM), one
+  // beyond.  Their cursors are the bucket cursors of 0 and 1 partons, which no
+  // event has: zero.
+  if (e == cudaSuccess && E.cap > 16)
+    e = launch_chained(chain, k_event_shapes_warp<128, 128>, grid(4, 5), 128, 4 * sizeof(WarpEvent<128>), s, P, E, order,
+                       offsets, 17, 128, cursor);
+  if (e == cudaSuccess && E.cap > 128)
+    e = launch_chained(chain, k_event_shapes_warp<256, 64>, grid(2, 6), 64, 2 * sizeof(WarpEvent<256>), s, P, E, order,
+                       offsets, 129, 255, cursor + 1);
   return e;
 }
 

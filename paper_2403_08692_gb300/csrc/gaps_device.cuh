@@ -211,8 +211,10 @@ inline void set_layout(Events& E, int layout, int64_t n_events, int capacity) {
 // At the top of a kernel that may be launched as a programmatic dependent
 // (launch_chained): let the stream's next launch be set up beside this one,
 // and wait for the one before to be complete.  Every thread of every block
-// passes it, so the launches stay ordered.  Without that attribute it does
-// nothing.
+// passes it before its first read, so the launches stay ordered: PTX promises
+// the sight of earlier launches' writes only after the reader's own wait,
+// also where the launch in between has waited.  Without that attribute it
+// does nothing.
 __device__ __forceinline__ void follow_launch() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");

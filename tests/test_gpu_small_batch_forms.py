@@ -98,7 +98,7 @@ def test_histograms(g, large):
 
 @pytest.mark.parametrize("n,cap", [(3000, CAP), (3000, 160), (70_000, 160)])
 def test_pass_in_a_graph(g, n, cap):
-    """Chained launches, and event-shape classes beside one another."""
+    """Chained launches, and every event-shape class."""
     p = g.make_params(seed=43, sqrt_s=200.0, t_cutoff=0.5)
     want = torch.zeros(g.HIST_DOUBLES, dtype=torch.float64).pin_memory()
     assert g.run(p, g.Workspace(n, cap), want, g.SHOWER_PERSISTENT)[0] == 0
