@@ -879,19 +879,25 @@ __device__ inline void emit_shared(const DevParams& P0, const Events& E, const E
   const int64_t ev = w.ev;
   const V4 a = load_p(E, w.i, ev);
   const V4 b = load_p(E, w.k, ev);
-  if (tid < 32) {
-    double n1c, n2c, inv;
+  // the frame's warp and the splitting variables' meet at one barrier that
+  // the whole block passes, not at one in each branch
+  const bool frame = tid < 32;
+  double n1c = 0.0, n2c = 0.0, inv = 0.0;
+  EmitState st{};
+  if (frame) {
     dipole_frame4(a, b, c, n1c, n2c, inv);
-    sync();
-    emit_momenta4(E, w, a, b, c, n1c, n2c, inv, splits[index], has);
   } else {
     const int job = kJobKey<kMode> ? static_cast<int>(E.job_of[ev]) : 0;
     const DevParams& P = job_params<kJobPhysics<kMode>>(P0, E, job);
-    const EmitState st = load_emit_state(E, w);
+    st = load_emit_state(E, w);
     const Splitting4 v = splitting_of4<kMode>(P, event_key<kMode>(P, E, ev, job), w, a, b, c);
     if (has && c == 0) splits[g] = v;
-    sync();
-    if (has && c == 0) emit_colours(E, w, st, reserve, put, g);
+  }
+  sync();
+  if (frame) {
+    emit_momenta4(E, w, a, b, c, n1c, n2c, inv, splits[index], has);
+  } else if (has && c == 0) {
+    emit_colours(E, w, st, reserve, put, g);
   }
 }
 

@@ -1,5 +1,6 @@
 """Rules that the CUDA sources keep and no run can show: a kernel that may be
-placed while the launch before it runs reads nothing before its own wait."""
+placed while the launch before it runs reads nothing before its own wait, and
+a barrier handed to a function is passed by the whole block at once."""
 import os
 import re
 
@@ -60,3 +61,13 @@ def test_chained_kernels_wait_before_they_read():
         assert at >= 0 and _depth(body, at) == 0, name
         before = body[:at]
         assert not re.search(r"\b(if|for|while|return)\b|E\.|->", before), (name, before)
+
+
+def test_shared_emission_meets_at_one_barrier():
+    """emit_shared's two warps take different branches; the barrier between
+    them stands outside both, once."""
+    text = _sources()["shower_cycle.cuh"]
+    body = _body(text, text.index("emit_shared("))
+    calls = [m.start() for m in re.finditer(r"\bsync\(\);", body)]
+    assert len(calls) == 1 and _depth(body, calls[0]) == 0
+    assert "__syncthreads" not in body
