@@ -377,8 +377,11 @@ cudaError_t clear_shower_counters(const Events& E, bool plain, cudaStream_t s) {
 // counters, the host-mapped slots the step launches publish their input
 // lengths to ({list, tasks}, each tagged with the launch's sequence number,
 // kSlots of them in rotation), and the timing events.  Sequence numbers grow
-// across calls (`next_seq`), so a slot never shows a value of an earlier call
-// as current.
+// across calls by the launches queued (`next_seq`), and a call starts with
+// cleared slots (the one before has drained its launches, or failed), so a
+// slot never shows a value of an earlier call as current, though a tag holds
+// 31 bits of its number: by the launches a call may queue, 2^32 + 2 without a
+// cycle limit, every eighth call's tags would meet an earlier one's.
 struct HostCounters {
   static constexpr int kSlots = 8;
   static constexpr int kSlotWords = 4;
@@ -500,7 +503,7 @@ int shower_impl(const gaps_params* params, const gaps_batch* batch, int mode, in
   const int64_t ahead = lookahead(E.n);
   const int64_t max_launches = 2 * static_cast<int64_t>(P.max_steps) + 2;
   const unsigned long long seq0 = hc.next_seq;  // launch c publishes launch c - 1's lengths as seq0 + c
-  hc.next_seq += static_cast<unsigned long long>(max_launches) + 1;
+  std::memset(hc.pub, 0, HostCounters::kSlots * HostCounters::kSlotWords * sizeof(unsigned long long));
   auto pub_slot = [&](int64_t c, bool device) {
     const size_t at = static_cast<size_t>(c % HostCounters::kSlots) * HostCounters::kSlotWords;
     return (device ? hc.pub_dev : hc.pub) + at;
@@ -509,6 +512,7 @@ int shower_impl(const gaps_params* params, const gaps_batch* batch, int mode, in
     return ((seq0 + static_cast<unsigned long long>(c)) | 0x80000000ull) << 32;  // never that of a cleared word
   };
   auto enqueue = [&](int64_t c) -> cudaError_t {
+    hc.next_seq = seq0 + static_cast<unsigned long long>(c) + 1;  // whatever comes of the launch
     const int in_half = static_cast<int>(c & 1), out_half = 1 - in_half;
     const int* list_in = c == 0 ? nullptr : E.active + static_cast<size_t>(in_half) * E.n;
     int* list_out = E.active + static_cast<size_t>(out_half) * E.n;
