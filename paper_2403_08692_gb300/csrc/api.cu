@@ -361,15 +361,15 @@ bool config_ok(const gaps_persistent_config& c) {
          c.blocks_per_sm <= 32 && layout_ok(c.layout);
 }
 
-// Clear the shower's counters (finished, step-limited, FP64 fallbacks, the
-// persistent form's event cursor).
-cudaError_t clear_shower_counters(const Events& E, bool plain, cudaStream_t s) {
-  // words 0..8 (word 9 keeps the job count) and the plain form's list and
-  // task counts and emission cursors
-  cudaError_t e = cudaMemsetAsync(E.counters, 0, 9 * sizeof(unsigned long long), s);
-  if (!plain) return e;
-  if (e == cudaSuccess) e = cudaMemsetAsync(E.counters + kPlainListWord, 0, 7 * sizeof(unsigned long long), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(E.counters + kPlainEmitCursorWord, 0, 3 * sizeof(unsigned long long), s);
+// Clear the shower's counters: words 0..8 (finished, step-limited, FP64
+// fallbacks, the persistent form's event cursor; word 9 keeps the job count)
+// and those from the plain form's list lengths on (its task counts, rebuilds
+// and emission cursors; among them the pool slices' cursor, which every slice
+// clears for itself), so that they are the last call's in both forms.
+cudaError_t clear_shower_counters(const Events& E, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(E.counters, 0, kJobCountWord * sizeof(unsigned long long), s);
+  if (e == cudaSuccess)
+    e = cudaMemsetAsync(E.counters + kPlainListWord, 0, (kCounterWords - kPlainListWord) * sizeof(unsigned long long), s);
   return e;
 }
 
@@ -461,7 +461,7 @@ int shower_impl(const gaps_params* params, const gaps_batch* batch, int mode, in
       if (b) cudaEventDestroy(b);
     }
   } guard{ev0, ev1};
-  e = clear_shower_counters(E, mode == GAPS_SHOWER_PLAIN, s);
+  e = clear_shower_counters(E, s);
   if (e != cudaSuccess) return cuda_fail(e);
   unsigned long long cnt[2] = {0, 0};  // finished events, events stopped at max_steps
   if (mode == GAPS_SHOWER_PERSISTENT) {
@@ -627,7 +627,7 @@ int gaps_shower_persistent(const gaps_params* params, const gaps_batch* batch,
   if (!config_ok(c)) return GAPS_ERR_INVALID;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (E.n == 0) return GAPS_OK;
-  cudaError_t e = clear_shower_counters(E, false, s);
+  cudaError_t e = clear_shower_counters(E, s);
   if (e == cudaSuccess) e = launch_shower_persistent(P, E, c, s);
   return e == cudaSuccess ? GAPS_OK : cuda_fail(e);
 }
@@ -663,7 +663,7 @@ int gaps_autotune_persistent(const gaps_params* params, const gaps_batch* batch,
         float shape_ms = -1.0f;  // the better of two timings of the shape
         for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
           e = launch_me(P, E, s);
-          if (e == cudaSuccess) e = clear_shower_counters(E, false, s);
+          if (e == cudaSuccess) e = clear_shower_counters(E, s);
           if (e == cudaSuccess) e = cudaEventRecord(a, s);
           if (e == cudaSuccess) e = launch_shower_persistent(P, E, c, s);
           if (e == cudaSuccess) e = cudaEventRecord(b, s);
