@@ -11,7 +11,7 @@
 //   rcp_fp64          3                   0.51 ulp
 //   div_fp64          6                   0.51 ulp
 //   rsqrt_fp64        5                   0.51 ulp
-//   sqrt_fp64         6                   1.1 ulp
+//   sqrt_fp64         8                   0.51 ulp
 //   exp_fp64          12                  0.55 ulp
 //   expm1_neg_fp64    13                  1.6 ulp (near 2^(-1/64), where t - 1 and t p cancel in part)
 //   circle_fp64       18                  1.2 ulp (sine and cosine; near the axes, from theta's own rounding)
@@ -91,8 +91,9 @@ __device__ __forceinline__ double sqrt_fp64(double x) {
   if (!seed_range(x)) return sqrt_library(x);
   const double y0 = from_seed(rsqrtf(seed_of(x)));
   const double e = fma(-x, y0 * y0, 1.0);
-  const double h = x * y0;
-  return fma(e * h, fma(e, 0.375, 0.5), h);
+  // x y0 in two parts: its own rounding would cost another half ulp
+  const double h = x * y0, l = fma(x, y0, -h);
+  return h + fma(e * h, fma(e, 0.375, 0.5), l);
 }
 
 // e^x = 2^m 2^(k/64) e^r with 64 m + k the integer nearest to 64 x / ln 2 and

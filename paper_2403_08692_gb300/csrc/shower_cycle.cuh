@@ -802,7 +802,7 @@ __device__ inline void cycle_emit(const DevParams& P0, const Events& E, const Em
 // GenerateEmission by four lanes a task, lane c of a group with momentum
 // component c, for lists too short to fill warps with a task per thread.  A
 // warp issues an FP64 instruction every 64 cycles whatever its active lanes,
-// so a short list waits for the number of them on its chain: 159 for a task
+// so a short list waits for the number of them on its chain: 161 for a task
 // in one lane.  Four lanes take about 90, and about 60 where one warp forms
 // the frame and the momenta and another the splitting variables and the
 // colours.  Each value comes from the operations of cycle_emit in their

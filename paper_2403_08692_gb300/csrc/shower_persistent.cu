@@ -555,7 +555,7 @@ __global__ void __launch_bounds__(kMaxThreads)
       __syncthreads();
       // Four lanes a task while the tasks then take at most a warp on each of
       // the SM's schedulers, whose FP64 issue one warp fills: a chain of 90
-      // FP64 instructions instead of 159.  Beyond, a thread a task takes half
+      // FP64 instructions instead of 161.  Beyond, a thread a task takes half
       // the instructions.  100 events 0.197 -> 0.190 ms, 2x10^4 0.253 ->
       // 0.244 (up to 1, 2, 4 or 8 such warps alike), 10^6 unchanged.
       const bool quads = tasks <= 8 * min(n_warps, kSchedulers);

@@ -8,8 +8,6 @@ import pytest
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-L = np.longdouble  # at least FP64; errors are taken on its differences
-
 
 @pytest.fixture(scope="module")
 def g():
@@ -61,6 +59,18 @@ def test_square_roots(g, name, lo, hi):
     p, e = _two_product(y, y)  # y - x^-1/2 = (x y^2 - 1) y / 2
     q, f = _two_product(p, x)
     assert _ulps(y, (((q - 1.0) + f) + e * x) * y / 2.0).max() <= 0.52
+
+
+@pytest.mark.parametrize("name,lo,hi", POSITIVE)
+def test_square_root_is_as_close_as_the_division(g, name, lo, hi):
+    """Half an ulp of the last rounding, and the dropped terms: the low part of
+    x y0 is below 2^-53 of the root and its own rounding, with that of the
+    correction (2^-21 of the root), below 2^-73."""
+    rng = np.random.default_rng(6)
+    x = 10.0 ** rng.uniform(lo, hi, 400_000)
+    y = _on_device(g, "sqrt", x)
+    p, e = _two_product(y, y)
+    assert _ulps(y, ((p - x) + e) / (2.0 * y)).max() <= 0.52
 
 
 def _decimal_check(fn, xs, ys):
