@@ -219,9 +219,9 @@ enum {
  * threads per block (64 events per warp; batches with fewer events than the
  * device has resident warps run one warp per block); compact_period (>= 1):
  * a block generates its waiting emissions at the latest once 4
- * compact_period per warp wait (at most 32); blocks_per_sm: resident blocks
- * per SM (0 = as many as fit); layout: the record layout the autotuner found fastest
- * with this shape (gaps_autotune_persistent's output, to be used as the
+ * compact_period per warp wait, at most 32 (values above 8 change nothing);
+ * blocks_per_sm: resident blocks per SM (0 = as many as fit); layout: the
+ * record layout the autotuner found fastest with this shape (gaps_autotune_persistent's output, to be used as the
  * batch's layout; launches take the layout from the batch and ignore this
  * field, which must be a valid layout). */
 typedef struct gaps_persistent_config {
@@ -430,7 +430,7 @@ int gaps_shower_persistent(const gaps_params* params, const gaps_batch* batch,
 
 /* Autotuner of the persistent form (batching): times every record layout
  * (structure of arrays, tiles of 8 and of 32 events), block size {128, 256,
- * 512} and compaction period {2, 4, 8, 16} on this batch's workspace, the
+ * 512} and compaction period {2, 4, 8} on this batch's workspace, the
  * better of two timings each (matrix element + shower each time, CUDA events
  * on `stream`), and returns the fastest in *best (layout included; its time
  * in *best_ms, may be NULL).  Overwrites the batch's events: regenerate them

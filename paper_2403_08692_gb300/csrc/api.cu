@@ -632,6 +632,20 @@ int gaps_shower_persistent(const gaps_params* params, const gaps_batch* batch,
   return e == cudaSuccess ? GAPS_OK : cuda_fail(e);
 }
 
+namespace {
+
+// The periods the autotuner times, every one another launch.
+constexpr int kTunedPeriods[] = {2, 4, 8};
+constexpr bool each_its_own_launch() {
+  for (const int a : kTunedPeriods)
+    for (const int b : kTunedPeriods)
+      if (a != b && emissions_awaited(a) == emissions_awaited(b)) return false;
+  return true;
+}
+static_assert(each_its_own_launch(), "a shape timed twice");
+
+}  // namespace
+
 int gaps_autotune_persistent(const gaps_params* params, const gaps_batch* batch, gaps_persistent_config* best,
                              double* best_ms, void* stream) {
   DevParams P;
@@ -648,7 +662,6 @@ int gaps_autotune_persistent(const gaps_params* params, const gaps_batch* batch,
   double best_time = -1.0;
   const int layouts[3] = {GAPS_LAYOUT_SOA, GAPS_LAYOUT_TILE8, GAPS_LAYOUT_TILE32};
   const int threads[3] = {128, 256, 512};
-  const int periods[4] = {2, 4, 8, 16};
   for (int li = 0; li < 3 && e == cudaSuccess; ++li) {
     // the same workspace read in another record layout (sized for all)
     gaps_batch bl = *batch;
@@ -658,8 +671,9 @@ int gaps_autotune_persistent(const gaps_params* params, const gaps_batch* batch,
       break;
     }
     for (int ti = 0; ti < 3 && e == cudaSuccess; ++ti) {
-      for (int pi = 0; pi < 4 && e == cudaSuccess; ++pi) {
-        const gaps_persistent_config c = {threads[ti], periods[pi], 0, layouts[li]};
+      for (const int period : kTunedPeriods) {
+        if (e != cudaSuccess) break;
+        const gaps_persistent_config c = {threads[ti], period, 0, layouts[li]};
         float shape_ms = -1.0f;  // the better of two timings of the shape
         for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
           e = launch_me(P, E, s);

@@ -36,6 +36,11 @@ cudaError_t launch_chained(bool chain, void (*kernel)(Params...), int64_t blocks
 // Batches whose finalisation launches are chained.
 constexpr int64_t kChainBelow = 50000;
 
+// Waiting emissions per warp that make a block of the persistent form generate
+// them at the latest: half of a warp's 64 events, so that periods above 8 are
+// the launch of 8 (any period is taken; 4 times the largest would overflow).
+constexpr int emissions_awaited(int compact_period) { return 4 * (compact_period < 8 ? compact_period : 8); }
+
 cudaError_t launch_me(const DevParams& P, const Events& E, cudaStream_t s);
 // One plain-form cycle over list_in[0 .. n_in) (list_in = NULL: events
 // 0 .. n_in); survivors are appended to list_out (may be NULL) through

@@ -771,7 +771,7 @@ cudaError_t launch_m(const DevParams& P, const Events& E, const gaps_persistent_
   const int64_t blocks = std::min(static_cast<int64_t>(sms) * per_sm,
                                   std::max<int64_t>((warps + threads / 32 - 1) / (threads / 32), std::min<int64_t>(sms, n)));
   if (blocks == 0) return cudaSuccess;
-  kernel<<<static_cast<unsigned>(blocks), threads, smem, s>>>(P, E, std::min(32, 4 * cfg.compact_period), sl);
+  kernel<<<static_cast<unsigned>(blocks), threads, smem, s>>>(P, E, emissions_awaited(cfg.compact_period), sl);
   return cudaGetLastError();
 }
 
