@@ -80,7 +80,7 @@ enum { GAPS_TRIALS_PER_KERNEL = 0, GAPS_TRIALS_PER_DIPOLE = 1 };
  * arrays): [ceil(n_events / T)][capacity][T], element (i, e) at
  * (e / T) * capacity * T + i * T + e % T, so all slots of an event lie within
  * capacity * T elements while a warp of consecutive events still reads
- * contiguous segments.  The [2][capacity] arrays (link, dip, dq2, dzp, dinv)
+ * contiguous segments.  The [2][capacity] arrays (link, dip)
  * are [2][capacity][n_events] and [ceil(n_events / T)][2][capacity][T]. */
 enum { GAPS_LAYOUT_SOA = 0, GAPS_LAYOUT_TILE8 = 1, GAPS_LAYOUT_TILE32 = 2 };
 
@@ -112,8 +112,9 @@ typedef struct gaps_layout {
                              (colour line) and side 1 (anticolour line), 255 = none */
   int64_t dip;            /* float2 [2][capacity][n_events]: per-dipole cache of the trial
                              densities (library-internal contents) */
-  int64_t dq2, dzp, dinv; /* double [2][capacity][n_events]: room for the FP64 part of the dipole
-                             cache (library-internal contents) */
+  int64_t dq2, dzp, dinv; /* 32-byte records [capacity][n_events] from dq2 to the end of dinv: FP64
+                             part of the dipole cache, a dipole's at its colour end
+                             (library-internal contents; dzp and dinv lie inside) */
   int64_t t;              /* double [n_events]: evolution scale t (GeV^2) at which the event
                              finished: t_C at the cutoff, the last winner's scale otherwise */
   int64_t lnt;            /* double [n_events]: ln t while the event is showering */
@@ -221,8 +222,8 @@ enum {
  * a block generates its waiting emissions at the latest once 4
  * compact_period per warp wait, at most 32 (values above 8 change nothing);
  * blocks_per_sm: resident blocks per SM (0 = as many as fit); layout: the
- * record layout the autotuner found fastest with this shape (gaps_autotune_persistent's output, to be used as the
- * batch's layout; launches take the layout from the batch and ignore this
+ * record layout the autotuner found fastest with this shape
+ * (gaps_autotune_persistent's output, to be used as the batch's layout; launches take the layout from the batch and ignore this
  * field, which must be a valid layout). */
 typedef struct gaps_persistent_config {
   int32_t block_threads;

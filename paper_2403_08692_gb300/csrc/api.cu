@@ -46,9 +46,12 @@ void compute_layout(int64_t n, int32_t cap, gaps_layout* L) {
   L->acol = take(2 * pc);
   L->link = take(2 * pc);
   L->dip = take(16 * pc);
+  // the dipole records, 32 pc bytes in one piece: pc is a multiple of 32, so
+  // each part is one of the alignment and no gap lies between them
+  static_assert(sizeof(DipoleRecord) == 32 && (8 * 32) % kAlign == 0, "the records' parts lie back to back");
   L->dq2 = take(16 * pc);
-  L->dzp = take(16 * pc);
-  L->dinv = take(16 * pc);
+  L->dzp = take(8 * pc);
+  L->dinv = take(8 * pc);
   L->t = take(8 * n);
   L->lnt = take(8 * n);
   L->weight = take(8 * n);
@@ -179,8 +182,6 @@ Events make_events(const gaps_batch& b) {
   E.acol = reinterpret_cast<int16_t*>(base + L.acol);
   E.link = reinterpret_cast<uint8_t*>(base + L.link);
   E.dip = reinterpret_cast<float2*>(base + L.dip);
-  // 32 bytes a dipole: the bytes of dq2 and dzp, which lie side by side (each
-  // is a multiple of the alignment)
   E.drec = reinterpret_cast<DipoleRecord*>(base + L.dq2);
   E.lnt = reinterpret_cast<double*>(base + L.lnt);
   E.t = reinterpret_cast<double*>(base + L.t);

@@ -140,7 +140,7 @@ struct Events {
   int16_t *col, *acol;
   uint8_t* link;  // [2][cap][n]
   float2* dip;    // [2][cap][n] dipole cache (see shower_cycle.cuh)
-  DipoleRecord* drec;  // [cap][n] FP64 part of the dipole cache (in the bytes of the layout's dq2 and dzp)
+  DipoleRecord* drec;  // [cap][n] FP64 part of the dipole cache (the layout's dq2, dzp and dinv)
   double* lnt;               // [n] ln t of the active events
   double *t, *weight;
   unsigned long long* hash;

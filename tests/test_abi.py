@@ -77,6 +77,15 @@ def test_workspace_layout(g):
         g.layout(10, 300)
 
 
+def test_dipole_records_take_their_own_bytes(g):
+    """32 bytes a slot from dq2 on, with no gap inside and none left over."""
+    for n, cap in ((1, 4), (33, 5), (10000, 128), (12345, 50), (1000000, 255)):
+        L = g.layout(n, cap)
+        slots = cap * ((n + 31) // 32 * 32)
+        assert L.t - L.dq2 == 32 * slots
+        assert L.dq2 < L.dzp < L.dinv < L.t
+
+
 def test_param_checks(g):
     assert g.check_params(g.make_params()) == 0
     assert g.check_params(g.make_params(t_cutoff=0.0)) == -1
