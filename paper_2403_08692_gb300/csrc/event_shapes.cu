@@ -8,10 +8,10 @@
 // to 16 partons take one thread each, with per-thread arrays (in batches of
 // fewer than 180 000 events, groups of 4 to 16 lanes: the event's momenta sit in
 // shared memory, the lanes split the pairs of each search and reduce their
-// partial results in the serial loop's order, and the O(n) FP64 steps run on
-// every lane alike, so the results are the one-thread results).  Larger
-// events take a warp each (event_shapes_warp), with the O(n) steps spread
-// over the lanes and a nearest-neighbour table in the clustering.
+// partial results in the serial loop's order, and the O(n) FP64 sums run one
+// component per lane in that order, so the results are the one-thread
+// results).  Larger events take a warp each (event_shapes_warp), with the O(n)
+// steps spread over the lanes and a nearest-neighbour table in the clustering.
 //
 // Precision.  As in the shower, the searches run in FP32 and the answers in
 // FP64:
@@ -40,7 +40,6 @@ namespace gaps {
 namespace {
 
 constexpr int kShapeThreads = 128;
-constexpr int kMaskMax = 64;
 
 // The products and sums of this file in fused form (the library is built
 // without automatic contraction): both the per-thread and the lane-group
@@ -160,9 +159,10 @@ __device__ void event_shapes(const DevParams& P0, const Events& E, int64_t ev, i
     ay = jy[0] * inv_l;
     az = jz[0] * inv_l;
     decided = true;
-  } else if (n <= kMaskMax) {
+  } else {
+    static_assert(MAXJ < 64, "a partition is a word");
     Top2 top;
-    const unsigned long long full = n == 64 ? ~0ull : ((1ull << n) - 1ull);
+    const unsigned long long full = (1ull << n) - 1ull;
     for (int j = 0; j < n; ++j) {
       for (int k = j + 1; k < n; ++k) {
         const float nx = crossf(fy[j], fz[k], fz[j], fy[k]);
@@ -355,14 +355,10 @@ __device__ void event_shapes(const DevParams& P0, const Events& E, int64_t ev, i
 }
 
 // ------------------------------------------------------- lane groups
-// Lanes of this thread's aligned group of L (L a power of two, <= 32).
+// Lanes of this thread's aligned group of L (L a power of two, < 32).
 template <int L>
 __device__ __forceinline__ unsigned group_lanes() {
-  if constexpr (L == 32) {
-    return 0xffffffffu;
-  } else {
-    return ((1u << L) - 1u) << ((threadIdx.x & 31u) & ~static_cast<unsigned>(L - 1));
-  }
+  return ((1u << L) - 1u) << ((threadIdx.x & 31u) & ~static_cast<unsigned>(L - 1));
 }
 
 // The pairs (j, k), j < k < n, of one lane: positions sub, sub + L, ... of
@@ -507,9 +503,10 @@ __device__ void event_shapes_group(const DevParams& P0, const Events& E, int64_t
     ay = a.j[2][0] * inv_l;
     az = a.j[3][0] * inv_l;
     decided = true;
-  } else if (n <= kMaskMax) {
+  } else {
+    static_assert(MAXJ < 64, "a partition is a word");
     Top2 top;
-    const unsigned long long full = n == 64 ? ~0ull : ((1ull << n) - 1ull);
+    const unsigned long long full = (1ull << n) - 1ull;
     PairWalk w;
     for (w.start(n, sub); w.valid(n); w.next<L>(n)) {
       const int j = w.j, k = w.k();

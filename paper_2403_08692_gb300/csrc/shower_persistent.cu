@@ -66,17 +66,16 @@ constexpr int kTurns = 3;
 constexpr int kDips = 6;
 constexpr uint8_t kInRecord = 255;
 
-// What the screens of a warp read of its events, S slots.
-template <int S>
+// What the screens of a warp read of its events.
 struct ScreenPool {
-  float dip_x[kDips][S], dip_y[kDips][S];  // the dipoles' screen entries
-  uint32_t dip_m[kDips][S];                // slot on side 0 | slot on side 1 << 8 | gluons << 16, 17
-  int32_t ev[S];
+  float dip_x[kDips][kSlots], dip_y[kDips][kSlots];  // the dipoles' screen entries
+  uint32_t dip_m[kDips][kSlots];                     // slot on side 0 | slot on side 1 << 8 | gluons << 16, 17
+  int32_t ev[kSlots];
   // the event's splitters, dipole * 2 + side: those with a gluon's kernels
   // from the front, those with one trial from the back; how many of either
   // kind (n_all = kInRecord: in the record)
-  uint8_t split[2 * kDips][S];
-  uint8_t n_all[S], n_one[S], n[S];
+  uint8_t split[2 * kDips][kSlots];
+  uint8_t n_all[kSlots], n_one[kSlots], n[kSlots];
   uint8_t owner[64];
 };
 // The screens' results, per lane.
@@ -101,8 +100,8 @@ struct SideCounts {
 // partons' data are loaded side by side over the lanes, so a few events take
 // one or two memory latencies whatever their size.  Every lane of the warp
 // must call it.
-template <int kMode, int S>
-__device__ __forceinline__ SideCounts load_dipoles(const DevParams& P0, const Events& E, ScreenPool<S>& w, int q, int job,
+template <int kMode>
+__device__ __forceinline__ SideCounts load_dipoles(const DevParams& P0, const Events& E, ScreenPool& w, int q, int job,
                                                    int L) {
   const int lane = static_cast<int>(threadIdx.x & 31);
   const int el = lane / L, sub = lane - el * L;
@@ -182,9 +181,9 @@ __device__ __forceinline__ SideCounts load_dipoles(const DevParams& P0, const Ev
 // is not the smallest is displaced or loses exactly once, whatever the order.
 // Equal bounds leave the cycle undecided, so which of them is kept is
 // immaterial.
-template <int kMode, int S>
-__device__ __forceinline__ void screen_warp(const DevParams& P0, const DevParams& P, const Events& E, ScreenPool<S>& w, ScreenResults& r, int q,
-                                            const EventKey& key, int step) {
+template <int kMode>
+__device__ __forceinline__ void screen_warp(const DevParams& P0, const DevParams& P, const Events& E, ScreenPool& w,
+                                            ScreenResults& r, int q, const EventKey& key, int step) {
   constexpr float kInvCF2 = static_cast<float>(1.0 / (2.0 * kCF));
   constexpr float kInvCA = static_cast<float>(1.0 / kCA);
   constexpr uint32_t kInf = 0x7f800000u;
@@ -352,7 +351,7 @@ enum : uint8_t {
 struct WarpPool {
   double lnt[kSlots];
   unsigned long long hash[kSlots];
-  ScreenPool<kSlots> sc;
+  ScreenPool sc;
   uint32_t rz_hi[kSlots], rz_lo[kSlots], won[kSlots];  // the waiting emission
   int32_t step[kSlots];
   int32_t first_step[kSlots];    // cycle the event came in at
