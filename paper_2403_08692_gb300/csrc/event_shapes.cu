@@ -22,6 +22,12 @@
 //    the FP32 error bound (or, in large events, is the longest of those within
 //    it), its |P| and axis are recomputed in FP64; otherwise the whole search
 //    runs in FP64.
+//    A momentum within FP32 rounding of a pair's plane may get the wrong side,
+//    which that bound does not cover: above 16 partons the sides in doubt are
+//    decided in FP64, pair by pair (sides_fp32, sides_fp64), so that the search
+//    sees the exact algorithm's partitions; the winner must also be the
+//    partition that its own axis defines.  Up to 16 partons every partition
+//    has to be missed by all its pairs to go unseen: sides are as FP32 has them.
 //  * Durham.  Pair distances min(E_i^2, E_j^2) |u_i - u_j|^2 (u = unit
 //    momentum, free of the 1 - cos cancellation) are compared in FP32 with a
 //    per-pair error bound; every pair that could be the minimum is evaluated
@@ -730,8 +736,8 @@ __device__ void event_shapes_group(const DevParams& P0, const Events& E, int64_t
 }
 
 // ------------------------------------------------- a warp per large event
-// The event of a warp in shared memory.  f: FP32 momenta in the thrust
-// search, then unit directions with E^2.  Durham's nearest neighbours: jet
+// The event of a warp in shared memory.  f: FP32 unit directions, with |p| in
+// the thrust search and E^2 in the clustering.  Durham's nearest neighbours: jet
 // r's smallest upper bound ub of the distance to another jet (near, with
 // lower bound lb) and a lower bound lb2 of all others: the smallest of theirs
 // (near2's), or no more than that once near2 is gone (near2 = kGone).
@@ -741,6 +747,7 @@ struct WarpEvent {
   float4 f[MAXJ];
   float ub[MAXJ], lb[MAXJ], lb2[MAXJ];
   uint8_t near[MAXJ], near2[MAXJ];
+  uint32_t full[MAXJ / 32], lengthy[MAXJ / 32];  // partitions' bits in use, and those of partons of some length
 };
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -749,8 +756,8 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// A partition of up to 32 W partons as sign bits (set: the minus side), the
-// first of each 32 highest.  Top two distinct ones by score, as Top2.
+// A partition of up to 32 W partons as sign bits (set: the minus side), 32 a
+// word (side_bit).
 template <int W>
 struct Partition {
   uint32_t w[W];
@@ -797,6 +804,117 @@ struct TopPartitions {
     }
   }
 };
+
+// Bit of parton i in word c of a partition of n partons.  The pairs' loop
+// collects two bits a parton, the last one's lowest, the first 16 of a word
+// apart from its second 16: the first have the odd bits, the second the even.
+__device__ __forceinline__ uint32_t side_bit(int n, int i, int c) {
+  const int first = i & ~15, last = min(n, first + 16) - 1;
+  return i >> 5 == c ? 1u << (2 * (last - i) + ((i & 16) == 0 ? 1 : 0)) : 0u;
+}
+
+// The sides of a pair's plane: the other partons' partition and their signed
+// sum (the pair's own two in neither).
+template <int W>
+struct Sides {
+  Partition<W> m;
+  float x, y, z;
+};
+
+// FP32 sides.  A product of the unit direction u_i with the normal u_j x u_k
+// is off by up to 6.6e-7: the directions' components by 2^-23 each (three
+// vectors, 3.6e-7), the normal's by 2^-23 (1.2e-7), the product's rounding by
+// 3 x 2^-24 (1.8e-7).  Normals are scaled by 2^21, so that a product within
+// 2^-20 of zero, whose sign is in doubt, is one below 2: the top bit of its
+// exponent is clear.  The two top bits of every product are collected, the
+// sign and whether it is certain, by one shift as the sign alone would be.
+// Returns whether every parton's of some length is certain, the pair's own two
+// excepted.
+constexpr float kNormalScale = 2097152.0f;  // 2^21
+template <int MAXJ>
+__device__ __forceinline__ bool sides_fp32(const WarpEvent<MAXJ>& a, int n, int j, int k, Sides<MAXJ / 32>& o) {
+  const float4 uj = a.f[j], uk = a.f[k];
+  const float nx = kNormalScale * crossf(uj.y, uk.z, uj.z, uk.y);
+  const float ny = kNormalScale * crossf(uj.z, uk.x, uj.x, uk.z);
+  const float nz = kNormalScale * crossf(uj.x, uk.y, uj.y, uk.x);
+  const uint32_t jbit = side_bit(n, j, j >> 5), kbit = side_bit(n, k, k >> 5);
+  o.x = o.y = o.z = 0.0f;
+  uint32_t own_j = 0u, own_k = 0u, doubt = 0u;
+#pragma unroll
+  for (int c = 0; c < MAXJ / 32; ++c) {
+    o.m.w[c] = 0u;
+    if (32 * c >= n) continue;
+    uint32_t odd = 0u, even = 0u;
+    const auto take = [&](int i, uint32_t& bits) {
+      const float4 u = a.f[i];
+      const uint32_t s = __float_as_uint(dot3f(u.x, u.y, u.z, nx, ny, nz));
+      const float w = __uint_as_float((s & 0x80000000u) | __float_as_uint(u.w));
+      o.x = fmaf(w, u.x, o.x);
+      o.y = fmaf(w, u.y, o.y);
+      o.z = fmaf(w, u.z, o.z);
+      bits = __funnelshift_l(s, bits, 2);
+    };
+    const int n_odd = min(n - 32 * c, 16), n_even = min(max(n - 32 * c - 16, 0), 16);
+    int t = 0;
+#pragma unroll 1
+    for (; t < n_even; ++t) {
+      take(32 * c + t, odd);
+      take(32 * c + 16 + t, even);
+    }
+#pragma unroll 1
+    for (; t < n_odd; ++t) take(32 * c + t, odd);
+    const uint32_t sign = (odd & 0xaaaaaaaau) | ((even & 0xaaaaaaaau) >> 1);
+    const uint32_t known = ((odd & 0x55555555u) << 1) | (even & 0x55555555u);
+    const uint32_t jb = j >> 5 == c ? jbit : 0u, kb = k >> 5 == c ? kbit : 0u;
+    doubt |= a.lengthy[c] & ~(known | jb | kb);
+    own_j |= sign & jb;
+    own_k |= sign & kb;
+    o.m.w[c] = sign & ~(jb | kb);
+  }
+  // without the pair itself
+  const float wj = own_j ? uj.w : -uj.w, wk = own_k ? uk.w : -uk.w;
+  o.x = fmaf(wk, uk.x, fmaf(wj, uj.x, o.x));
+  o.y = fmaf(wk, uk.y, fmaf(wj, uj.y, o.y));
+  o.z = fmaf(wk, uk.z, fmaf(wj, uj.z, o.z));
+  return doubt == 0u;
+}
+
+// FP64 sides, with the exact search's formulas, by the whole warp; false where
+// the pair spans no plane.  About one pair in 10^4 of an isotropic event comes
+// here, every pair of a planar one.
+template <int MAXJ>
+__device__ __noinline__ bool sides_fp64(const WarpEvent<MAXJ>& a, int n, int j, int k, int lane, Sides<MAXJ / 32>& o) {
+  const double nx = cross(a.j[2][j], a.j[3][k], a.j[3][j], a.j[2][k]);
+  const double ny = cross(a.j[3][j], a.j[1][k], a.j[1][j], a.j[3][k]);
+  const double nz = cross(a.j[1][j], a.j[2][k], a.j[2][j], a.j[1][k]);
+  if (nx == 0.0 && ny == 0.0 && nz == 0.0) return false;
+  float x = 0.0f, y = 0.0f, z = 0.0f;
+#pragma unroll
+  for (int c = 0; c < MAXJ / 32; ++c) {
+    const int i = 32 * c + lane;
+    uint32_t bit = 0u;
+    if (i < n && i != j && i != k) {
+      const bool plus = dot3(a.j[1][i], a.j[2][i], a.j[3][i], nx, ny, nz) >= 0.0;
+      const float4 u = a.f[i];
+      const float w = plus ? u.w : -u.w;
+      x = fmaf(w, u.x, x);
+      y = fmaf(w, u.y, y);
+      z = fmaf(w, u.z, z);
+      bit = plus ? 0u : side_bit(n, i, c);
+    }
+    o.m.w[c] = __reduce_or_sync(0xffffffffu, bit);
+  }
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    x += __shfl_xor_sync(0xffffffffu, x, off);
+    y += __shfl_xor_sync(0xffffffffu, y, off);
+    z += __shfl_xor_sync(0xffffffffu, z, off);
+  }
+  o.x = x;
+  o.y = y;
+  o.z = z;
+  return true;
+}
 
 // FP32 bounds of the distance of jets a and b (unit directions, E^2 in w):
 // per-pair relative error 4e-6 + 1e-6 / |u_a - u_b|.
@@ -928,12 +1046,14 @@ __device__ __noinline__ double thrust_fp64_warp(int n, const WarpEvent<MAXJ>& a,
 // Thrust: the lanes take the pairs; a pair's partition is built from the
 // signs of the other momenta's products with its normal without a branch (the
 // pair's own two, whose products are rounding, are taken out of the sum
-// afterwards).  With the four best distinct partitions known, those within
-// the FP32 error of the best are compared in FP64, unless the fourth is one
-// of them (with many partons the best two often are: one event in fifty of 17
-// .. 80 partons was left to the exact search, which takes half a
-// millisecond); the winner must also be the one its own axis defines, which
-// the longest one is.
+// afterwards), and again by the warp in FP64 where a sign is in doubt: of 65
+// momenta that lie 10^-8 out of a plane or of three directions, FP32 signs
+// alone gave another axis than the exact search.  With the four best distinct
+// partitions known, those within the FP32 error of the best are compared in
+// FP64, unless the fourth is one of them (with many partons the best two often
+// are: one event in fifty of 17 .. 80 partons was left to the exact search,
+// which takes half a millisecond); the winner must also be the one its own
+// axis defines, which the longest one is.
 //
 // Durham: a merge changes the distances to one jet only, so every jet keeps
 // its nearest neighbour and a lower bound of the others' (Row); a merge renews
@@ -943,12 +1063,13 @@ __device__ __noinline__ double thrust_fp64_warp(int n, const WarpEvent<MAXJ>& a,
 // FP32 bounds as before; y in FP64 is only formed for the four merges that
 // are recorded.
 //
-// Bound by FP32 issue in the thrust pairs (n^3 / 2 products; issue slots 65 %
-// busy).  20 000 RAMBO events of 17 .. 80 partons: 25.3 -> 3.2 ms against every
-// merge searching all its pairs twice, events beyond 64 partons searched in
-// FP64, and two blocks per SM with a fixed share of the events each (with
-// these in place: 7.3 ms with two partitions kept and every row that pointed
-// at a merged jet renewed, 4.8 ms with fixed shares).
+// Bound by FP32 issue in the thrust pairs (n^3 / 2 products, eight
+// instructions each).  20 000 RAMBO events of 17 .. 80 partons: 25.3 -> 3.1 ms
+// against every merge searching all its pairs twice, events beyond 64 partons
+// searched in FP64, and two blocks per SM with a fixed share of the events
+// each (with these in place: 7.3 ms with two partitions kept and every row that
+// pointed at a merged jet renewed, 4.8 ms with fixed shares); 3.2 ms with the
+// signs made certain (3.4 with the two halves of a word in loops of their own).
 template <int MAXJ>
 __device__ void event_shapes_warp(const DevParams& P0, const Events& E, int64_t ev, int n, WarpEvent<MAXJ>& a, int lane) {
   constexpr int W = MAXJ / 32;
@@ -961,8 +1082,12 @@ __device__ void event_shapes_warp(const DevParams& P0, const Events& E, int64_t 
     a.j[1][i] = x;
     a.j[2][i] = y;
     a.j[3][i] = z;
-    a.f[i] = make_float4(f32_from_f64(x), f32_from_f64(y), f32_from_f64(z), 0.0f);
-    sum_abs += sqrt_obs(dot3(x, y, z, x, y, z));
+    const double length = sqrt_obs(dot3(x, y, z, x, y, z));
+    sum_abs += length;
+    const float fx = f32_from_f64(x), fy = f32_from_f64(y), fz = f32_from_f64(z);
+    const float l2 = dot3f(fx, fy, fz, fx, fy, fz), r = rsqrtf(l2);
+    // (of no length in single precision: on either side, and no part of a sum)
+    a.f[i] = l2 == 0.0f ? make_float4(0.0f, 0.0f, 0.0f, 0.0f) : make_float4(fx * r, fy * r, fz * r, f32_from_f64(length));
   }
   sum_abs = warp_sum(sum_abs);
   const float sum_absf = f32_from_f64(sum_abs);
@@ -971,72 +1096,65 @@ __device__ void event_shapes_warp(const DevParams& P0, const Events& E, int64_t 
   // ---- thrust
   TopPartitions<W> top;
   top.clear();
-  uint32_t full[W];  // the bits in use
 #pragma unroll
   for (int c = 0; c < W; ++c) {
-    const int r = n - 32 * c;
-    full[c] = r >= 32 ? 0xffffffffu : (r > 0 ? (1u << r) - 1u : 0u);
+    const int i = 32 * c + lane;
+    const uint32_t bit = i < n ? side_bit(n, i, c) : 0u;
+    const uint32_t all = __reduce_or_sync(0xffffffffu, bit);
+    const uint32_t some = __reduce_or_sync(0xffffffffu, i < n && a.f[i].w != 0.0f ? bit : 0u);
+    if (lane == 0) {
+      a.full[c] = all;
+      a.lengthy[c] = some;
+    }
   }
-  // bit of parton i: the last of its word is lowest
-  const auto bit_of = [&](int i, int c) { return i >> 5 == c ? 1u << (min(n - 32 * c, 32) - 1 - (i & 31)) : 0u; };
+  __syncwarp();
   PairWalk pw;
+  pw.start(n, lane);
 #pragma unroll 1
-  for (pw.start(n, lane); pw.valid(n); pw.next<32>(n)) {
-    const int j = pw.j, k = pw.k();
-    const float4 pj = a.f[j], pk = a.f[k];
-    const float nx = crossf(pj.y, pk.z, pj.z, pk.y);
-    const float ny = crossf(pj.z, pk.x, pj.x, pk.z);
-    const float nz = crossf(pj.x, pk.y, pj.y, pk.x);
-    if (nx == 0.0f && ny == 0.0f && nz == 0.0f) continue;
-    float px = 0.0f, py = 0.0f, pz = 0.0f;
-    Partition<W> m;
-#pragma unroll
-    for (int c = 0; c < W; ++c) {
-      uint32_t bits = 0u;
-      const int end = min(n, 32 * c + 32);
-#pragma unroll 4
-      for (int i = 32 * c; i < end; ++i) {
-        const float4 q = a.f[i];
-        const uint32_t s = __float_as_uint(dot3f(q.x, q.y, q.z, nx, ny, nz));
-        const float sg = __uint_as_float((s & 0x80000000u) | 0x3f800000u);
-        px = fmaf(sg, q.x, px);
-        py = fmaf(sg, q.y, py);
-        pz = fmaf(sg, q.z, pz);
-        bits = __funnelshift_l(s, bits, 1);
-      }
-      m.w[c] = bits;
-    }
-    // without the pair itself
-    uint32_t bj = 0u, bk = 0u;
-#pragma unroll
-    for (int c = 0; c < W; ++c) {
-      const uint32_t jb = bit_of(j, c), kb = bit_of(k, c);
-      bj |= m.w[c] & jb;
-      bk |= m.w[c] & kb;
-      m.w[c] &= ~(jb | kb);
-    }
-    const float sj = bj ? 1.0f : -1.0f, sk = bk ? 1.0f : -1.0f;
-    px = fmaf(sk, pk.x, fmaf(sj, pj.x, px));
-    py = fmaf(sk, pk.y, fmaf(sj, pj.y, py));
-    pz = fmaf(sk, pk.z, fmaf(sj, pj.z, pz));
+  for (;;) {
+    bool has = pw.valid(n);
+    if (!__any_sync(0xffffffffu, has)) break;
+    const int j = has ? pw.j : 0, k = has ? pw.k() : 1;
+    Sides<W> sides;
+    const bool certain = sides_fp32<MAXJ>(a, n, j, k, sides);
+    unsigned doubt = __ballot_sync(0xffffffffu, has && !certain);
 #pragma unroll 1
-    for (int c4 = 0; c4 < 4; ++c4) {
-      const float fj = (c4 & 2) ? -1.0f : 1.0f, fk = (c4 & 1) ? -1.0f : 1.0f;
-      const float cx = fmaf(fk, pk.x, fmaf(fj, pj.x, px));
-      const float cy = fmaf(fk, pk.y, fmaf(fj, pj.y, py));
-      const float cz = fmaf(fk, pk.z, fmaf(fj, pj.z, pz));
-      const float score = dot3f(cx, cy, cz, cx, cy, cz);
-      if (score <= top.least) continue;
-      Partition<W> t;
-#pragma unroll
-      for (int c = 0; c < W; ++c)
-        t.w[c] = m.w[c] | ((c4 & 2) ? bit_of(j, c) : 0u) | ((c4 & 1) ? bit_of(k, c) : 0u);
-      if (t.w[0] & bit_of(0, 0)) {  // a partition and its complement are one candidate
-#pragma unroll
-        for (int c = 0; c < W; ++c) t.w[c] = ~t.w[c] & full[c];
+    while (doubt != 0u) {
+      const int src = __ffs(doubt) - 1;
+      doubt &= doubt - 1u;
+      Sides<W> exact;
+      const bool plane = sides_fp64<MAXJ>(a, n, __shfl_sync(0xffffffffu, j, src), __shfl_sync(0xffffffffu, k, src), lane, exact);
+      if (lane == src) {
+        has = plane;
+        sides.x = exact.x;
+        sides.y = exact.y;
+        sides.z = exact.z;
+        sides.m = exact.m;
       }
-      top.add(score, t);
     }
+    if (has) {
+      const float4 uj = a.f[j], uk = a.f[k];
+      const uint32_t jbit = side_bit(n, j, j >> 5), kbit = side_bit(n, k, k >> 5), bit0 = side_bit(n, 0, 0);
+#pragma unroll 1
+      for (int c4 = 0; c4 < 4; ++c4) {
+        const float wj = (c4 & 2) ? -uj.w : uj.w, wk = (c4 & 1) ? -uk.w : uk.w;
+        const float cx = fmaf(wk, uk.x, fmaf(wj, uj.x, sides.x));
+        const float cy = fmaf(wk, uk.y, fmaf(wj, uj.y, sides.y));
+        const float cz = fmaf(wk, uk.z, fmaf(wj, uj.z, sides.z));
+        const float score = dot3f(cx, cy, cz, cx, cy, cz);
+        if (score <= top.least) continue;
+        Partition<W> t;
+#pragma unroll
+        for (int c = 0; c < W; ++c)
+          t.w[c] = sides.m.w[c] | ((c4 & 2) && j >> 5 == c ? jbit : 0u) | ((c4 & 1) && k >> 5 == c ? kbit : 0u);
+        if (t.w[0] & bit0) {  // a partition and its complement are one candidate
+#pragma unroll
+          for (int c = 0; c < W; ++c) t.w[c] = ~t.w[c] & a.full[c];
+        }
+        top.add(score, t);
+      }
+    }
+    pw.next<32>(n);
   }
 #pragma unroll 1
   for (int off = 1; off < 32; off <<= 1) {
@@ -1083,7 +1201,7 @@ __device__ void event_shapes_warp(const DevParams& P0, const Events& E, int64_t 
       for (int i = lane; i < n; i += 32) {
         uint32_t minus = 0u;
 #pragma unroll
-        for (int c = 0; c < W; ++c) minus |= m.w[c] & bit_of(i, c);
+        for (int c = 0; c < W; ++c) minus |= m.w[c] & side_bit(n, i, c);
         const double sg = minus ? -1.0 : 1.0;
         px = fma(sg, a.j[1][i], px);
         py = fma(sg, a.j[2][i], py);
@@ -1114,7 +1232,7 @@ __device__ void event_shapes_warp(const DevParams& P0, const Events& E, int64_t 
     for (int i = lane; i < n; i += 32) {
       uint32_t minus = 0u;
 #pragma unroll
-      for (int c = 0; c < W; ++c) minus |= won.w[c] & bit_of(i, c);
+      for (int c = 0; c < W; ++c) minus |= won.w[c] & side_bit(n, i, c);
       const double d = dot3(a.j[1][i], a.j[2][i], a.j[3][i], ax, ay, az);
       decided = decided && (minus ? d <= 0.0 : d >= 0.0);
     }
@@ -1517,8 +1635,8 @@ __global__ void __launch_bounds__(T) k_event_shapes_group(DevParams P, Events E,
 // Events of buckets n_lo..n_hi (all with n <= MAXJ), a warp each, T threads
 // per block, the largest first; the warps of the resident blocks take them
 // one by one from *cursor (zero before the launch).
-template <int MAXJ, int T>
-__global__ void __launch_bounds__(T) k_event_shapes_warp(DevParams P, Events E, const int* order, const int* offsets,
+template <int MAXJ, int T, int kBlocks>
+__global__ void __launch_bounds__(T, kBlocks) k_event_shapes_warp(DevParams P, Events E, const int* order, const int* offsets,
                                                          int n_lo, int n_hi, int* cursor) {
   follow_launch();
   extern __shared__ __align__(16) unsigned char s_shapes[];
@@ -1546,7 +1664,8 @@ __global__ void __launch_bounds__(T) k_event_shapes_warp(DevParams P, Events E, 
 // The per-thread grid holds one thread per event up to kShapeBlocksPerSm
 // blocks per SM (largest events first, above): 0.86 ms at 10^6 events then; a
 // second launch of lane groups for 7, 9, 11 or 13 .. 16 partons there took the
-// stage to 1.10, 1.00, 0.99 and 0.93.
+// stage to 1.10, 1.00, 0.99 and 0.93.  All of LEP events (4.9 partons on
+// average); the lines take no account of the multiplicities.
 constexpr int kShapeBlocksPerSm = 64;
 constexpr int64_t kThreadsFrom = 180000;
 
@@ -1562,8 +1681,8 @@ cudaError_t preload_observables() {
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_group<16, 4, 128>);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_group<16, 8, 128>);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_group<16, 16, 128>);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_warp<128, 128>);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_warp<256, 64>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_warp<128, 128, 5>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_event_shapes_warp<256, 64, 6>);
   return e;
 }
 
@@ -1613,10 +1732,10 @@ cudaError_t launch_observables(const DevParams& P, const Events& E, int* buckets
   // beyond.  Their cursors are the bucket cursors of 0 and 1 partons, which no
   // event has: zero.
   if (e == cudaSuccess && E.cap > 16)
-    e = launch_chained(chain, k_event_shapes_warp<128, 128>, grid(4, 5), 128, 4 * sizeof(WarpEvent<128>), s, P, E, order,
+    e = launch_chained(chain, k_event_shapes_warp<128, 128, 5>, grid(4, 5), 128, 4 * sizeof(WarpEvent<128>), s, P, E, order,
                        offsets, 17, 128, cursor);
   if (e == cudaSuccess && E.cap > 128)
-    e = launch_chained(chain, k_event_shapes_warp<256, 64>, grid(2, 6), 64, 2 * sizeof(WarpEvent<256>), s, P, E, order,
+    e = launch_chained(chain, k_event_shapes_warp<256, 64, 6>, grid(2, 6), 64, 2 * sizeof(WarpEvent<256>), s, P, E, order,
                        offsets, 129, 255, cursor + 1);
   return e;
 }

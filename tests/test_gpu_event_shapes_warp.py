@@ -67,3 +67,24 @@ def test_degenerate_events_among_others(g, oracle_mod):
         want = oracle_mod.event_shapes(p, SQRT_S ** 2)
         assert np.all(np.abs(o - want) <= H.OBS_REL * np.abs(want) + H.OBS_ABS)
     assert got[3][4] == pytest.approx(0.0, abs=1e-12)  # all along one direction: T = 1
+
+
+@pytest.mark.parametrize("spread", [1e-4, 1e-6, 1e-7, 1e-8])
+def test_thrust_of_nearly_planar_and_narrow_events(g, oracle_mod, spread):
+    """Third momenta within the FP32 rounding of many pairs' planes: the thrust
+    axis found must still be the longest one."""
+    rng = np.random.default_rng(11)
+    events = []
+    for n in (17, 65, 128, 255):
+        for _ in range(3):
+            phi = rng.uniform(0.0, 2.0 * np.pi, n)
+            flat = np.stack([np.cos(phi), np.sin(phi), spread * rng.normal(size=n)], axis=1)
+            narrow = np.array([[0.0, 0.0, 1.0], [0.8, 0.0, -0.6], [-0.8, 0.0, -0.6]])[rng.integers(0, 3, n)]
+            for u in (flat, narrow + spread * rng.normal(size=(n, 3))):
+                u /= np.linalg.norm(u, axis=1)[:, None]
+                e = rng.exponential(size=n) + 0.01
+                p = np.concatenate([e[:, None], (e[:, None] * u) @ S.random_rotation(rng).T], axis=1)
+                events.append(p * (SQRT_S / e.sum()))
+    for p, o in zip(events, _observables(g, events, 255)):
+        want = oracle_mod.event_shapes(p, SQRT_S ** 2)[4]
+        assert abs(o[4] - want) <= H.OBS_REL * abs(want) + H.OBS_ABS, (len(p), o[4], want)
