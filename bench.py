@@ -68,8 +68,8 @@ RECORD_BYTES_PER_PARTON = 44
 
 def step_kernel_profile():
     """Figures of the committed ncu captures of the plain-form step kernel
-    (profiles/k_step_deferred_1e5.md): DRAM bytes per event-cycle of a whole
-    pass and the FP64-pipe, issue-slot and SM-active fractions of mid-shower
+    (profiles/k_step_deferred_1e5.md): DRAM bytes per event-cycle and the
+    FP64-pipe, issue-slot and SM-active fractions of mid-shower
     launches; None once the kernel sources differ from the captured ones."""
     import hashlib
     import re
@@ -92,8 +92,8 @@ def step_kernel_profile():
 
 def step_kernel_traffic(event_cycles_per_launch, warm=False):
     """DRAM bytes per launch of the plain-form step kernel: the per-event-cycle
-    traffic of the committed ncu capture (all step launches of one pass at
-    10^5 events, the deferred emissions included; cold caches as ncu runs by
+    traffic of the committed ncu capture (three mid-shower launches at 10^5
+    events, the deferred emissions included; cold caches as ncu runs by
     default, or warm: caches as the pass leaves them) times this run's
     event-cycles per launch; None once the kernel sources differ from the
     captured ones."""
@@ -881,8 +881,8 @@ def main():
                                                step_kernel_traffic(float(st.sum_steps)) / record_bytes),
                      "traffic": step_kernel_traffic(st.sum_steps / max(1.0, launches_per_pass)),
                      "traffic_warm": step_kernel_traffic(st.sum_steps / max(1.0, launches_per_pass), warm=True),
-                     "traffic_source": "profiles/k_step_deferred_1e5.md: DRAM bytes per event-cycle from one ncu "
-                                       "capture x this run's event-cycles per launch (traffic: caches flushed "
+                     "traffic_source": "profiles/k_step_deferred_1e5.md: DRAM bytes per event-cycle of three "
+                                       "mid-shower launches x this run's event-cycles per launch (traffic: caches flushed "
                                        "before each launch, ncu's default; traffic_warm: caches as the pass "
                                        "leaves them, which at 10^5 events hold most of the record)",
                      "pipes": pipe_fractions(),

@@ -417,10 +417,10 @@ HostCounters& host_counters() {
 
 // The plain form rebuilds its active list in event order after a launch
 // while the list holds at least 1/GAPS_REBUILD_DIV of the batch, in batches of
-// GAPS_REBUILD_MIN events or more: below, the second-level cache serves the
-// scattered loads and the rebuild only costs its launch (10^3 events 1.53 ->
-// 1.20 ms and 1.2x10^4 4.60 -> 4.11 ms without it
-// above; 10^5 events 2.89 with it, 2.99 ms without).
+// GAPS_REBUILD_MIN events or more: in smaller ones the second-level cache
+// serves the scattered loads and the rebuild only costs its launch.  With and
+// without it, in one revision of the step: 10^3 events 1.53 and 1.20 ms,
+// 1.2x10^4 4.60 and 4.11, 10^5 2.89 and 2.99.
 #ifndef GAPS_REBUILD_MIN
 #define GAPS_REBUILD_MIN 50000
 #endif
@@ -429,14 +429,16 @@ HostCounters& host_counters() {
 #endif
 
 // Launches the plain form's host loop queues ahead of the one it reads back:
-// two while the list rebuild makes a step two launches, else one.  Two
-// against one: 5x10^4 events 2.03 -> 1.95 ms, 10^5 2.36 -> 2.30, 2x10^5 2.89
-// -> 2.86; without the rebuild the older count costs more than the queue
-// gains (1.2x10^4 events 1.37 -> 1.42 ms), and where a step is long it gains
-// nothing (10^6 events 7.69 -> 7.72).
+// two while the list rebuild makes a step two launches and a step is short,
+// below kLookaheadBelow events, else one.  One and two (LEP events): 5x10^4
+// events 2.03 and 1.95 ms, 10^5 2.36 and 2.30, 2x10^5 2.89 and 2.86; without
+// the rebuild the older count costs more than the queue gains (1.2x10^4 events
+// 1.37 and 1.42 ms), and where a step is long it gains nothing (10^6 events
+// 7.69 and 7.72).
 constexpr int64_t kLookaheadMax = 2;
+constexpr int64_t kLookaheadBelow = 300000;
 static_assert(kLookaheadMax + 2 <= HostCounters::kSlots, "lookahead and readback slots");
-constexpr int64_t lookahead(int64_t n) { return n >= GAPS_REBUILD_MIN && n < 300000 ? kLookaheadMax : 1; }
+constexpr int64_t lookahead(int64_t n) { return n >= GAPS_REBUILD_MIN && n < kLookaheadBelow ? kLookaheadMax : 1; }
 
 int shower_impl(const gaps_params* params, const gaps_batch* batch, int mode, int64_t* launches_out,
                 double* kernel_ms_out, void* stream) {

@@ -597,7 +597,7 @@ __global__ void __launch_bounds__(256) k_stats(Events E, gaps_stats* st) {
 
 // Eight lanes per event in batches under 60 000 events: 10^3 events 31 -> 16
 // us, 2x10^4 33 -> 23, 4.9x10^4 34 -> 33, but 10^5 42 -> 50 (4 and 16 lanes: 19
-// and 15, 22 and 27, 31 and 42, 47 and 70).
+// and 15, 22 and 27, 31 and 42, 47 and 70).  LEP events.
 constexpr int kValidateLanes = 8;
 constexpr int64_t kValidateLanesBelow = 60000;
 
@@ -620,7 +620,7 @@ cudaError_t launch_validate(const DevParams& P, const Events& E, cudaStream_t s,
 #endif
 // Batches whose warps take an observable each instead of 32 events: the eight
 // fills of an event then run side by side (10^3 events 35 -> 26 us for the
-// stage, 2x10^4 38 -> 33; 4.9x10^4 41 -> 42, 10^6 165 -> 229).
+// stage, 2x10^4 38 -> 33; 4.9x10^4 41 -> 42, 10^6 165 -> 229).  LEP events.
 constexpr int64_t kHistSplitBelow = 30000;
 
 cudaError_t launch_hist_fixed(const DevParams& P, const DevParams* scale_src, const Events& E, unsigned long long* acc,

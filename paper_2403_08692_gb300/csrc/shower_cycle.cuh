@@ -422,9 +422,6 @@ __device__ __forceinline__ void screen_group_reduce(Screen& sc) {
   }
 }
 
-// What the FP32 screen settles about a cycle: no trial above the cutoff, a
-// certain winner (its exact scale computed), or neither -- then the exact
-// FP64 selection decides (select_winner_fp64 / fallback_warp).
 // a > b for numbers (b not -0), from their bits put in order: the FP64 pipe's
 // compares cost as much as its FMAs.
 __device__ __forceinline__ bool above(double a, double b) {
@@ -432,6 +429,9 @@ __device__ __forceinline__ bool above(double a, double b) {
   return (x ^ ((x >> 63) & 0x7fffffffffffffffll)) > (y ^ ((y >> 63) & 0x7fffffffffffffffll));
 }
 
+// What the FP32 screen settles about a cycle: no trial above the cutoff, a
+// certain winner (its exact scale computed), or neither -- then the exact
+// FP64 selection decides (select_winner_fp64 / fallback_warp).
 enum : int { kScreenNone = 0, kScreenWinner = 1, kScreenUndecided = 2 };
 
 // The screen's verdict; for a certain winner its exact scale (from the FP64

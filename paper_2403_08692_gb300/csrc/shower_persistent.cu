@@ -61,8 +61,10 @@ constexpr int kTurns = 3;
 
 // Dipoles with phase space kept per event in shared memory; an event with
 // more takes its screen's inputs from the record.  Six hold nearly every LEP
-// event; 8 or 4 were 5 and 14 % slower for the persistent form at 10^6 events
-// (less first-level cache, more events in the record).
+// event; 8 or 4 were 5 and 14 % slower for the persistent form at 10^6 LEP
+// events (less first-level cache, more events in the record).  Event-cycles in
+// the record: LEP 0.8 %, 200 GeV 1.8 % at t_C = 2 GeV^2 and 8.5 % at 0.5, 500
+// GeV 12 % at 1 and 19 % at 0.5; other counts were not timed there.
 constexpr int kDips = 6;
 constexpr uint8_t kInRecord = 255;
 
